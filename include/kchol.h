@@ -107,22 +107,25 @@ typedef struct {
 /* Options of the persistent kernels (zero-initialise for defaults). */
 typedef struct {
     int64_t spin_limit_cycles;     /* bound of every device wait; 0 -> ~4e9 cycles */
-    int32_t rows_per_task;         /* rows of a column per task; 0 -> factor: about (nnz - N) / (depth x
-                                      resident warps), a power of two in 16..128; factor by column groups:
-                                      see kc_factor_blocked; backward solve: 128 */
+    int32_t rows_per_task;         /* rows of a column per task; 0 -> factor: from the rows per level and the
+                                      row length, a power of two in 4..128 (FP64: 8..128) per warp that works
+                                      on the task; factor by column groups: see kc_factor_blocked; backward
+                                      solve: 128 */
     int32_t ctas_per_sm;           /* persistent grid = SMs x this; 0 -> occupancy; < 0 (factor) ->
                                       occupancy + this (at least 1): leaves that many CTA slots per
                                       SM to kernels on other streams (latency of concurrent solves) */
-    int32_t warps_per_cta;         /* 0 -> the CTA size (8, 4, 2 or 1 warps) with the most resident warps */
+    int32_t warps_per_cta;         /* 0 -> the CTA size (8, 4, 2 or 1 warps) with the most resident warps, and
+                                      no more CTAs than the dependency levels are wide */
     int32_t test_hold_column;      /* test hook: 0 = off; c+1 makes column c never signal
                                       ready, so a wait on it runs out (KC_ETIMEOUT) */
     int32_t lanes_per_row;         /* factor: lanes merging one row (1,2,4,..,32); 0 -> 8 (FP32 form) or
                                       4 (FP64): one 32-byte sector of values per group load */
-    int32_t unroll;                /* factor: (col, val) loads staged ahead per lane, 4, 8 or 16 (16: FP32
-                                      form only; FP64 takes 8); 0 -> FP32 form: 16 when the mean row
-                                      holds >= 400 entries, else 8; FP64: 4 */
+    int32_t unroll;                /* factor with other lanes_per_row than the default: (col, val) loads staged
+                                      ahead per lane, 4, 8 or 16 (16: FP32 form only; FP64 takes 8); 0 ->
+                                      FP32 form: 16 when the mean row holds >= 400 entries, else 8; FP64: 4.
+                                      The default number of lanes streams the rows through shared memory */
     int32_t adaptive_chunks;       /* factor: nonzero -> a task takes at least |R_i|/4 rows */
-    int32_t stage_bytes;           /* factor: <= 0 -> row prefixes loaded into registers (the default);
+    int32_t stage_bytes;           /* factor: <= 0 -> row prefixes streamed through shared memory (the default);
                                       > 0 -> bulk form: each warp fills two shared-memory stage buffers of
                                       this many bytes (<= 65536) with bulk (TMA) copies of row prefixes */
 } kc_opts;

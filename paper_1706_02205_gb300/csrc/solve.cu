@@ -613,7 +613,7 @@ kc_status solver_init(Solver& S, const kc_pattern* P, int nrhs_cap, const kc_opt
     S.P = P;
     S.rpt = (o && o->rows_per_task > 0) ? o->rows_per_task : KC_SOLVE_ROWS;
     if (o && o->spin_limit_cycles > 0) S.spin = o->spin_limit_cycles;
-    KC_TRY(build_tasks(P, S.rpt, A, s, &S.tasks, &S.ntasks, &S.maxr));
+    KC_TRY(build_tasks(P, S.rpt, A, s, &S.tasks, nullptr, &S.ntasks));
     S.nrhs_cap = nrhs_cap;
     KC_TRY(A.get(&S.ready, P->N));
     KC_TRY(A.get(&S.cnt, P->N));

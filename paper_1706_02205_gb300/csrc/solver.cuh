@@ -9,7 +9,6 @@ struct Solver {
     int2* tasks = nullptr;
     int64_t ntasks = 0;
     int rpt = 64;
-    int maxr = 0;
     int* ready = nullptr;
     unsigned* cnt = nullptr;
     unsigned* gcnt = nullptr;
@@ -22,8 +21,8 @@ struct Solver {
     long long spin = 4000000000LL;
 };
 
-kc_status build_tasks(const kc_pattern* P, int rpt, Arena& A, cudaStream_t s, int2** tasks_out, int64_t* ntasks_out,
-                      int* max_row_out, bool adaptive = false);
+kc_status build_tasks(const kc_pattern* P, int rpt, Arena& A, cudaStream_t s, int2** tasks_out,
+                      const int64_t** count_out, int64_t* ntasks_out, bool adaptive = false);
 kc_status solver_init(Solver& S, const kc_pattern* P, int nrhs_cap, const kc_opts* o, Arena& A, cudaStream_t s);
 template <typename T>
 kc_status solver_apply(Solver& S, const T* val, const double* diag, double diag_fallback, const double* rhs,
