@@ -389,7 +389,7 @@ def supernodal_leg(args, l, xo, pat0, kern):
 TRAFFIC_CAPTURE = {"sources": ("paper_1706_02205_gb300/csrc/factor.cu", "paper_1706_02205_gb300/csrc/common.cuh",
                                "paper_1706_02205_gb300/csrc/grid.cuh", "paper_1706_02205_gb300/csrc/covariance.cuh",
                                "paper_1706_02205_gb300/csrc/ichol.cuh"),
-                   "sha256": "c451b48af040465db22b9ae542e07ca7ca5e83489e6c40929c7eb84dd5b9fd1d",
+                   "sha256": "715564d71b1c18fd9b4b06937a5f53888dd9f969bf0372631509373322b352d8",
                    "dram_per_algorithmic_byte": (26.960658 + 0.946831) / 26.387813}
 
 

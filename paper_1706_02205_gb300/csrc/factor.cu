@@ -1017,7 +1017,7 @@ static kc_status max_row(const kc_pattern* P, Arena& A, cudaStream_t s, int* out
 }
 
 // Tasks a pattern has at most: one per column and one more per rpt rows below the diagonal.
-static int64_t tasks_bound(const kc_pattern* P, int rpt) { return P->N + (P->nnz - P->N) / rpt; }
+int64_t tasks_bound(const kc_pattern* P, int rpt) { return P->N + (P->nnz - P->N) / rpt; }
 
 // Build the task list of a pattern (its columns in the schedule's order:
 // by level, within a level in space-filling-curve order when the schedule was

@@ -3,7 +3,7 @@
 //
 // Forward  L y = b:   y_j = (b_j - sum_{k in R_j} L_jk y_k) / L_jj, one warp per
 //                     row, rows in (level, index) order; row j waits for the
-//                     ready flags of its R_j.
+//                     values of its R_j.
 // Backward L^T x = y: x_i = (y_i - sum_{j in C_i} L_ji x_j) / L_ii, over the
 //                     CSC columns in reverse level order; wide columns are cut
 //                     into chunks of rows, each chunk stores its partial sums
@@ -16,11 +16,19 @@
 // Vectors are point-major inside with a power-of-two stride NR >= nrhs
 // (v[k * NR + r]), so one point's right-hand sides are one aligned run that a
 // lane gathers with 16-byte loads.  A lane owns entries of the row (or rows of
-// the column): the readiness checks go out as relaxed loads all at once (a
-// bounded spin only on points not yet solved, then one acquire fence), the
-// values and the gathers follow in a few rounds, and the warp reduces its NR
+// the column): their columns and values are loaded first, then their points'
+// values in a few rounds; a value not yet set is polled (await_words), which
+// for the early, coarse points of a row never happens, so their products are
+// done while the last ones are still on their way.  The warp reduces its NR
 // partial sums with a reduce-scatter.  A dropped pivot (L_ii = 0) uses
 // sqrt(Theta_ii).
+//
+// Bound by the chain of dependency levels (each a store, a poll, the warp's
+// reduction and a division) and, at 16 right-hand sides, by the gathers (128
+// bytes an entry from L1 and L2).  Values that carry their own readiness,
+// against ready flags with fences on both sides: 2000 points, one right-hand
+// side 1.0 -> 0.5 ms; 100,003 points 3.9 -> 1.4; 2^20 points, rho = 3, 11.0 ->
+// 6.8 (one) and 14.3 -> 12.0 (16, FP32 form), 22.6 -> 18.4 (16, FP64).
 //
 // Arithmetic.  FP64 form: vectors, products and sums in FP64.  FP32 form (L in
 // FP32): the GB300's FP64 pipe is a small fraction of its FP32 rate, so the
@@ -47,10 +55,20 @@ namespace kc {
 #define KC_SOLVE_MINB 3
 #endif
 
-// Longest back-off (ns) between two polls of a readiness flag.
-#ifndef KC_SOLVE_BACKOFF_MAX
-#define KC_SOLVE_BACKOFF_MAX 512
+// Right-hand sides up to which a row's b, y and pivot are fetched before its
+// waits (beyond, the registers they hold cost more).
+#ifndef KC_SOLVE_EARLY
+#define KC_SOLVE_EARLY 4
 #endif
+
+// Warps per row of a dependency level that a solve launches at most.
+#ifndef KC_SOLVE_WAVES
+#define KC_SOLVE_WAVES 8.0
+#endif
+
+// Longest back-off (ns) between two polls of a value.
+template <int NR>
+constexpr int BACKOFF_MAX = NR > 4 ? 128 : 64;
 
 template <typename T>
 struct SolveArgs {
@@ -62,7 +80,7 @@ struct SolveArgs {
     const int64_t* __restrict__ slot;
     const int32_t* __restrict__ order;
     const int2* __restrict__ tasks;
-    int64_t ntasks;
+    const int64_t* __restrict__ ntasks;  // device
     int rpt;
     const T* __restrict__ val;
     const double* __restrict__ diag;
@@ -75,59 +93,97 @@ struct SolveArgs {
     double* acc;      // partial sums of the chunks of wide columns: NR per task, at the task's index
     unsigned* cnt;    // finished chunk groups per column (backward)
     unsigned* gcnt;   // finished chunks per group of 32, at the group's first task
-    int* ready;       // per point flag
     unsigned long long* ticket;
     int* status;
     long long spin_limit;
 };
 
-__device__ __forceinline__ int ld_relaxed_s32(const int* p) {
-    int v;
-    asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+// A point's vector values carry their own readiness: the buffers start as all
+// ones (a NaN no value takes, see word_of), every value is stored once as one
+// 8-byte word, and whoever needs it loads it until it is set.  A row's result
+// then reaches the rows that wait for it in one store and one load; with ready
+// flags it took a fence before the flag, the poll, another fence and only then
+// the gathers (2^20 points, rho = 3, one right-hand side, FP32 form: 10.6 ms).
+
+
+// 16 (8) bytes of vector values through L1: coarse points are gathered by nearly
+// every row.  A line cached before its values were set only sends the reader to
+// the polling loads below, which go to L2.
+__device__ __forceinline__ ulonglong2 ld_first(const ulonglong2* p) {
+    ulonglong2 v;
+    asm volatile("ld.global.ca.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p) : "memory");
     return v;
 }
-// bounded wait (backoff) on a point not yet solved; false when the budget ran
-// out or the kernel is stopping
-__device__ __forceinline__ bool spin_flag(const int* f, const int* status, long long limit) {
+__device__ __forceinline__ unsigned long long ld_first(const unsigned long long* p) {
+    unsigned long long v;
+    asm volatile("ld.global.ca.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ unsigned long long ld_again(const unsigned long long* p) {
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_value(unsigned long long* p, unsigned long long v) {
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+// The word of a value; a NaN that happens to be all ones in its first half
+// becomes the usual one, so that no value looks unset.
+__device__ __forceinline__ unsigned long long word_of(double v) {
+    const unsigned long long w = (unsigned long long)__double_as_longlong(v);
+    return (unsigned)(w >> 32) == 0xffffffffu ? 0x7fffffffffffffffull : w;
+}
+__device__ __forceinline__ unsigned long long word_of(float2 v) {
+    const unsigned hi = __float_as_uint(v.x);
+    return ((unsigned long long)__float_as_uint(v.y) << 32) | (hi == 0xffffffffu ? 0x7fffffffu : hi);
+}
+// FP64: the high half tells; pairs: hi, in the low half
+template <typename V>
+__device__ __forceinline__ bool is_unset(unsigned long long w);
+template <>
+__device__ __forceinline__ bool is_unset<double>(unsigned long long w) { return (unsigned)(w >> 32) == 0xffffffffu; }
+template <>
+__device__ __forceinline__ bool is_unset<float2>(unsigned long long w) { return (unsigned)w == 0xffffffffu; }
+
+// N words of a point's values, loaded once (no wait)
+template <int N>
+__device__ __forceinline__ void ld_words(const unsigned long long* p, unsigned long long (&w)[N]) {
+    if constexpr (N == 1) {
+        w[0] = ld_first(p);
+    } else {
+#pragma unroll
+        for (int q = 0; q < N / 2; ++q) {
+            const ulonglong2 x = ld_first((const ulonglong2*)p + q);
+            w[2 * q] = x.x;
+            w[2 * q + 1] = x.y;
+        }
+    }
+}
+// Bounded wait (backoff) until all of them are set; false when the budget ran
+// out or the kernel is stopping.
+template <typename V, int NR, int N>
+__device__ __forceinline__ bool await_words(const unsigned long long* p, unsigned long long (&w)[N], const int* status,
+                                            long long limit) {
+    bool open = false;
+#pragma unroll
+    for (int q = 0; q < N; ++q) open |= is_unset<V>(w[q]);
+    if (!open) return true;
     const long long t0 = clock64();
     unsigned ns = 32;
-    while (ld_relaxed_s32(f) == 0) {
-        if (clock64() - t0 > limit || ld_volatile_s32(status) != 0) return false;
-        __nanosleep(ns);  // back off so waiting warps do not flood L2 with polls
-        if (ns < KC_SOLVE_BACKOFF_MAX) ns <<= 1;
-    }
-    return true;
-}
-
-// Loads of a point's vector values, which other SMs write during the launch.
-// When one point's values fill whole 128-byte lines by themselves (LINE =
-// bytes per point = 128, i.e. 16 right-hand sides), no SM can read a line of
-// point k before k's ready flag is set, after its values were written, so the
-// line may be cached in L1 (KC_SOLVE_GATHER_L1); coarse points are gathered by
-// nearly every row.  Otherwise lines are shared by neighbouring points and the
-// loads go to L2.
-#ifndef KC_SOLVE_GATHER_L1
-#define KC_SOLVE_GATHER_L1 1
-#endif
-template <int LINE, typename V>
-__device__ __forceinline__ V ld_vec(const V* p) {
-    if constexpr (KC_SOLVE_GATHER_L1 && LINE == 128) return __ldca(p);
-    else return __ldcg(p);
-}
-
-// The NR values of point k (16-byte loads).
-template <int NR>
-__device__ __forceinline__ void gather(const double* v, int k, double* out) {
-    if constexpr (NR == 1) {
-        out[0] = __ldcg(v + k);
-    } else {
-        const double2* p = (const double2*)(v + (int64_t)k * NR);
+    for (int poll = 1;; ++poll) {
+        w[0] = ld_again(p);  // one word stands for the point until it is set
+        if (!is_unset<V>(w[0])) {
+            open = false;
 #pragma unroll
-        for (int q = 0; q < NR / 2; ++q) {
-            const double2 w = ld_vec<NR * 8>(p + q);
-            out[2 * q] = w.x;
-            out[2 * q + 1] = w.y;
+            for (int q = 1; q < N; ++q) {
+                w[q] = ld_again(p + q);
+                open |= is_unset<V>(w[q]);
+            }
+            if (!open) return true;
         }
+        if (clock64() - t0 > limit || ((poll & 15) == 0 && ld_volatile_s32(status) != 0)) return false;
+        __nanosleep(ns);  // back off so waiting warps do not flood L2 with polls
+        if (ns < BACKOFF_MAX<NR>) ns <<= 1;
     }
 }
 
@@ -172,58 +228,31 @@ struct Depth {
     static constexpr int E = NR >= 4 ? 32 / NR : 8;
 };
 
-// Readiness of the points kk[0..D) (negative: none): relaxed loads together,
-// bounded spins on the rest, one acquire fence.  False: a wait ran out.
-template <int D>
-__device__ __forceinline__ bool points_ready(const int* ready, const int (&kk)[D], const int* status, long long lim) {
-    unsigned pend = 0;
-#pragma unroll
-    for (int u = 0; u < D; ++u)
-        if (kk[u] >= 0 && ld_relaxed_s32(&ready[kk[u]]) == 0) pend |= 1u << u;
+// acc[r] += w[u] * v[k[u] * NR + r] for the D entries in order, E gathers at a
+// time, each point waited for where it is not solved yet.  False: a wait ran out.
+template <int NR, int D>
+__device__ __forceinline__ bool gather_fma(const double* v, const int (&k)[D], const double (&w)[D], double (&acc)[NR],
+                                           const int* status, long long limit) {
+    constexpr int E = Depth<NR>::E < D ? Depth<NR>::E : D;
     bool ok = true;
 #pragma unroll
-    for (int u = 0; u < D; ++u)
-        if (ok && ((pend >> u) & 1u)) ok = spin_flag(&ready[kk[u]], status, lim);
-    ok = __all_sync(0xffffffffu, ok);
-    fence_acq_rel_gpu();  // acquire: the points' values are visible from here on
-    return ok;
-}
-
-// acc[r] += w[u] * v[k[u] * NR + r] for the D entries, E gathers at a time
-template <int NR, int D>
-__device__ __forceinline__ void gather_fma(const double* v, const int (&k)[D], const double (&w)[D],
-                                           double (&acc)[NR]) {
-    constexpr int E = Depth<NR>::E < D ? Depth<NR>::E : D;
-#pragma unroll
     for (int u0 = 0; u0 < D; u0 += E) {
-        double g[E][NR];
-#pragma unroll
-        for (int q = 0; q < E; ++q) {
-            if (k[u0 + q] >= 0) gather<NR>(v, k[u0 + q], g[q]);
-            else
-#pragma unroll
-                for (int r = 0; r < NR; ++r) g[q][r] = 0.0;
-        }
+        unsigned long long g[E][NR];
 #pragma unroll
         for (int q = 0; q < E; ++q)
-            if (k[u0 + q] >= 0)  // the FP64 pipe is scarce: no products for empty slots
+            if (k[u0 + q] >= 0) ld_words<NR>((const unsigned long long*)v + (int64_t)k[u0 + q] * NR, g[q]);
 #pragma unroll
-                for (int r = 0; r < NR; ++r) acc[r] = fma(w[u0 + q], g[q][r], acc[r]);
+        for (int q = 0; q < E; ++q)
+            if (k[u0 + q] >= 0) {  // the FP64 pipe is scarce: no products for empty slots
+                if (ok)
+                    ok = await_words<double, NR, NR>((const unsigned long long*)v + (int64_t)k[u0 + q] * NR, g[q], status,
+                                                 limit);
+#pragma unroll
+                for (int r = 0; r < NR; ++r)
+                    acc[r] = fma(w[u0 + q], __longlong_as_double((long long)g[q][r]), acc[r]);
+            }
     }
-}
-
-// Publish a solved point: the warp's writes of its values, then its ready
-// flag with release semantics (KC_SOLVE_PUB_FENCE: with a fence of every lane
-// before the warp barrier as well).
-#ifndef KC_SOLVE_PUB_FENCE
-#define KC_SOLVE_PUB_FENCE 1
-#endif
-__device__ __forceinline__ void publish_ready(int* f, int lane) {
-#if KC_SOLVE_PUB_FENCE
-    fence_acq_rel_gpu();
-#endif
-    __syncwarp();
-    if (lane == 0) st_release_s32(f, 1);
+    return ok;
 }
 
 // Sum over cnt slots of NR doubles (slot p0, p0 + stride, ...) in a fixed
@@ -277,7 +306,7 @@ __device__ __forceinline__ bool combine_chunks(double* part, unsigned* gcnt, uns
 }
 
 template <typename T, int NR>
-__global__ void __launch_bounds__(256) fwd_solve_k(SolveArgs<T> A) {
+__global__ void __launch_bounds__(256, 2) fwd_solve_k(SolveArgs<T> A) {
     constexpr int D = 8;  // entries of R_j per lane per round
     const int lane = lane_id();
     const unsigned FULL = 0xffffffffu;
@@ -290,6 +319,14 @@ __global__ void __launch_bounds__(256) fwd_solve_k(SolveArgs<T> A) {
         const int j = A.order[t];
         const int64_t a = A.rowptr[j];
         const int n = (int)(A.rowptr[j + 1] - 1 - a);
+        // what finishes the row, fetched before the waits
+        const int r = rhs_of_lane<NR>(lane);
+        const bool wr = rhs_writer<NR>(lane);
+        double bj = 0.0, dj = 0.0;
+        if constexpr (NR <= KC_SOLVE_EARLY) {
+            if (wr) bj = A.b[(int64_t)j * NR + r];
+            dj = A.diag[j];
+        }
         double acc[NR];
 #pragma unroll
         for (int r = 0; r < NR; ++r) acc[r] = 0.0;
@@ -303,25 +340,25 @@ __global__ void __launch_bounds__(256) fwd_solve_k(SolveArgs<T> A) {
             double w[D];  // static data: loaded before the wait
 #pragma unroll
             for (int u = 0; u < D; ++u) w[u] = kk[u] >= 0 ? (double)__ldg(&A.val[a + e0 + lane + 32 * u]) : 0.0;
-            if (!points_ready<D>(A.ready, kk, A.status, A.spin_limit)) {
+            if (!__all_sync(FULL, gather_fma<NR, D>(A.y, kk, w, acc, A.status, A.spin_limit))) {
                 if (lane == 0) atomicCAS(A.status, 0, DEV_TIMEOUT);
                 return;
             }
-            gather_fma<NR, D>(A.y, kk, w, acc);
         }
         const double s = reduce_scatter<NR>(acc, lane);
-        if (rhs_writer<NR>(lane)) {
-            const int r = rhs_of_lane<NR>(lane);
-            double dj = A.diag[j];
+        if (wr) {
+            if constexpr (NR > KC_SOLVE_EARLY) {
+                bj = A.b[(int64_t)j * NR + r];
+                dj = A.diag[j];
+            }
             if (!(dj > 0.0)) dj = A.diag_fallback;
-            A.y[(int64_t)j * NR + r] = (A.b[(int64_t)j * NR + r] - s) / dj;
+            st_value((unsigned long long*)A.y + (int64_t)j * NR + r, word_of((bj - s) / dj));
         }
-        publish_ready(&A.ready[j], lane);
     }
 }
 
 template <typename T, int NR>
-__global__ void __launch_bounds__(256) bwd_solve_k(SolveArgs<T> A) {
+__global__ void __launch_bounds__(256, 2) bwd_solve_k(SolveArgs<T> A) {
     constexpr int D = 4;  // rows of the chunk per lane per round
     const int lane = lane_id();
     const unsigned FULL = 0xffffffffu;
@@ -329,9 +366,10 @@ __global__ void __launch_bounds__(256) bwd_solve_k(SolveArgs<T> A) {
         unsigned long long t = 0;
         if (lane == 0) t = atomicAdd(A.ticket, 1ULL);
         t = __shfl_sync(FULL, t, 0);
-        if ((int64_t)t >= A.ntasks) return;
+        const int64_t nt = __ldg(A.ntasks);
+        if ((int64_t)t >= nt) return;
         if (ld_volatile_s32(A.status) != 0) return;
-        const int64_t ti = A.ntasks - 1 - (int64_t)t;
+        const int64_t ti = nt - 1 - (int64_t)t;
         const int2 tk = A.tasks[ti];
         const int i = tk.x, c = tk.y;
         const int64_t c0 = A.colptr[i], c1 = A.colptr[i + 1];
@@ -339,6 +377,14 @@ __global__ void __launch_bounds__(256) bwd_solve_k(SolveArgs<T> A) {
         const unsigned nch = m <= 0 ? 1u : (unsigned)((m + A.rpt - 1) / A.rpt);
         const int64_t qs = c0 + 1 + (int64_t)c * A.rpt;
         const int nq = (int)(min(c1, qs + A.rpt) - qs);
+        // what finishes a column of one chunk, fetched before the waits
+        int r = rhs_of_lane<NR>(lane);
+        bool wr = rhs_writer<NR>(lane);
+        double yi = 0.0, di = 0.0;
+        if constexpr (NR <= KC_SOLVE_EARLY) {
+            if (wr) yi = A.y[(int64_t)i * NR + r];
+            di = A.diag[i];
+        }
         double acc[NR];
 #pragma unroll
         for (int r = 0; r < NR; ++r) acc[r] = 0.0;
@@ -354,29 +400,27 @@ __global__ void __launch_bounds__(256) bwd_solve_k(SolveArgs<T> A) {
             double w[D];  // static data: loaded before the wait
 #pragma unroll
             for (int u = 0; u < D; ++u) w[u] = jj[u] >= 0 ? (double)__ldg(&A.val[pp[u]]) : 0.0;
-            if (!points_ready<D>(A.ready, jj, A.status, A.spin_limit)) {
+            if (!__all_sync(FULL, gather_fma<NR, D>(A.x, jj, w, acc, A.status, A.spin_limit))) {
                 if (lane == 0) atomicCAS(A.status, 0, DEV_TIMEOUT);
                 return;
             }
-            gather_fma<NR, D>(A.x, jj, w, acc);
         }
         double s = reduce_scatter<NR>(acc, lane);
-        bool wr = rhs_writer<NR>(lane);
-        int r = rhs_of_lane<NR>(lane);
         bool finish = true;
         if (nch > 1) {
             if (wr) A.acc[ti * NR + r] = s;
             finish = combine_chunks<NR>(A.acc, A.gcnt, A.cnt, i, ti, c, nch, lane, s);
             wr = lane < NR;  // the combined sums: right-hand side lane % NR
             r = lane % NR;
+            if constexpr (NR <= KC_SOLVE_EARLY) yi = A.y[(int64_t)i * NR + r];
         }
-        if (finish) {
-            if (wr) {
-                double di = A.diag[i];
-                if (!(di > 0.0)) di = A.diag_fallback;
-                A.x[(int64_t)i * NR + r] = (A.y[(int64_t)i * NR + r] - s) / di;
+        if (finish && wr) {
+            if constexpr (NR > KC_SOLVE_EARLY) {
+                yi = A.y[(int64_t)i * NR + r];
+                di = A.diag[i];
             }
-            publish_ready(&A.ready[i], lane);
+            if (!(di > 0.0)) di = A.diag_fallback;
+            st_value((unsigned long long*)A.x + (int64_t)i * NR + r, word_of((yi - s) / di));
         }
     }
 }
@@ -439,41 +483,37 @@ __device__ __forceinline__ bool pair_writer(int lane) {
     return (lane & ((32 >> PL::L) - 1) & ~(PL::P - 1)) == 0;
 }
 
-// (s, c)[r] += w[u] * v[k[u]][block + r], E gathers at a time, nothing for empty slots
+// (s, c)[r] += w[u] * v[k[u]][block + r] for the D entries in order, E gathers
+// at a time, nothing for empty slots; each point waited for where it is not
+// solved yet.  False: a wait ran out.
 template <int NR, int D>
-__device__ __forceinline__ void gather_pair_add(const float2* v, const int (&k)[D], const float (&w)[D], int block,
-                                                float (&s)[PairLayout<NR>::NRL], float (&c)[PairLayout<NR>::NRL]) {
+__device__ __forceinline__ bool gather_pair_add(const float2* v, const int (&k)[D], const float (&w)[D], int block,
+                                                float (&s)[PairLayout<NR>::NRL], float (&c)[PairLayout<NR>::NRL],
+                                                const int* status, long long limit) {
     constexpr int NRL = PairLayout<NR>::NRL;
     constexpr int E0 = NRL >= 2 ? 16 / NRL : 8;  // at most 16 pairs in flight per lane
     constexpr int E = E0 < D ? E0 : D;
+    bool ok = true;
 #pragma unroll
     for (int u0 = 0; u0 < D; u0 += E) {
-        float hi[E][NRL], lo[E][NRL];
-#pragma unroll
-        for (int q = 0; q < E; ++q)
-            if (k[u0 + q] >= 0) {
-                const float2* p = v + (int64_t)k[u0 + q] * NR + block;
-                if constexpr (NRL == 1) {
-                    const float2 x = __ldcg(p);
-                    hi[q][0] = x.x;
-                    lo[q][0] = x.y;
-                } else {
-#pragma unroll
-                    for (int m = 0; m < NRL / 2; ++m) {
-                        const float4 x = ld_vec<NR * 8>((const float4*)p + m);
-                        hi[q][2 * m] = x.x;
-                        lo[q][2 * m] = x.y;
-                        hi[q][2 * m + 1] = x.z;
-                        lo[q][2 * m + 1] = x.w;
-                    }
-                }
-            }
+        unsigned long long g[E][NRL];
 #pragma unroll
         for (int q = 0; q < E; ++q)
             if (k[u0 + q] >= 0)
+                ld_words<NRL>((const unsigned long long*)v + (int64_t)k[u0 + q] * NR + block, g[q]);
 #pragma unroll
-                for (int r = 0; r < NRL; ++r) pair_add(s[r], c[r], w[u0 + q], hi[q][r], lo[q][r]);
+        for (int q = 0; q < E; ++q)
+            if (k[u0 + q] >= 0) {
+                if (ok)
+                    ok = await_words<float2, NR, NRL>((const unsigned long long*)v + (int64_t)k[u0 + q] * NR + block, g[q],
+                                                  status, limit);
+#pragma unroll
+                for (int r = 0; r < NRL; ++r)
+                    pair_add(s[r], c[r], w[u0 + q], __uint_as_float((unsigned)g[q][r]),
+                             __uint_as_float((unsigned)(g[q][r] >> 32)));
+            }
     }
+    return ok;
 }
 
 template <int NR>
@@ -492,6 +532,14 @@ __global__ void __launch_bounds__(256, KC_SOLVE_MINB) fwd_solve_pair_k(SolveArgs
         const int j = A.order[t];
         const int64_t a = A.rowptr[j];
         const int n = (int)(A.rowptr[j + 1] - 1 - a);
+        // what finishes the row, fetched before the waits
+        const int r = pair_rhs<NR>(lane);
+        const bool wr = pair_writer<NR>(lane);
+        double bj = 0.0, dj = 0.0;
+        if constexpr (NR <= KC_SOLVE_EARLY) {
+            if (wr) bj = A.b[(int64_t)j * NR + r];
+            dj = A.diag[j];
+        }
         float s[PL::NRL], c[PL::NRL];
 #pragma unroll
         for (int r = 0; r < PL::NRL; ++r) s[r] = c[r] = 0.f;
@@ -504,20 +552,20 @@ __global__ void __launch_bounds__(256, KC_SOLVE_MINB) fwd_solve_pair_k(SolveArgs
                 kk[u] = e < n ? __ldg(&A.col[a + e]) : -1;
                 w[u] = e < n ? __ldg(&A.val[a + e]) : 0.f;
             }
-            if (!points_ready<D>(A.ready, kk, A.status, A.spin_limit)) {
+            if (!__all_sync(FULL, gather_pair_add<NR, D>(A.yf, kk, w, block, s, c, A.status, A.spin_limit))) {
                 if (lane == 0) atomicCAS(A.status, 0, DEV_TIMEOUT);
                 return;
             }
-            gather_pair_add<NR, D>(A.yf, kk, w, block, s, c);
         }
         const double sum = reduce_scatter_pair<NR>(s, c, lane);
-        if (pair_writer<NR>(lane)) {
-            const int r = pair_rhs<NR>(lane);
-            double dj = A.diag[j];
+        if (wr) {
+            if constexpr (NR > KC_SOLVE_EARLY) {
+                bj = A.b[(int64_t)j * NR + r];
+                dj = A.diag[j];
+            }
             if (!(dj > 0.0)) dj = A.diag_fallback;
-            A.yf[(int64_t)j * NR + r] = pair_of((A.b[(int64_t)j * NR + r] - sum) / dj);
+            st_value((unsigned long long*)A.yf + (int64_t)j * NR + r, word_of(pair_of((bj - sum) / dj)));
         }
-        publish_ready(&A.ready[j], lane);
     }
 }
 
@@ -532,9 +580,10 @@ __global__ void __launch_bounds__(256, KC_SOLVE_MINB) bwd_solve_pair_k(SolveArgs
         unsigned long long t = 0;
         if (lane == 0) t = atomicAdd(A.ticket, 1ULL);
         t = __shfl_sync(FULL, t, 0);
-        if ((int64_t)t >= A.ntasks) return;
+        const int64_t nt = __ldg(A.ntasks);
+        if ((int64_t)t >= nt) return;
         if (ld_volatile_s32(A.status) != 0) return;
-        const int64_t ti = A.ntasks - 1 - (int64_t)t;
+        const int64_t ti = nt - 1 - (int64_t)t;
         const int2 tk = A.tasks[ti];
         const int i = tk.x, ch = tk.y;
         const int64_t c0 = A.colptr[i], c1 = A.colptr[i + 1];
@@ -542,6 +591,15 @@ __global__ void __launch_bounds__(256, KC_SOLVE_MINB) bwd_solve_pair_k(SolveArgs
         const unsigned nch = m <= 0 ? 1u : (unsigned)((m + A.rpt - 1) / A.rpt);
         const int64_t qs = c0 + 1 + (int64_t)ch * A.rpt;
         const int nq = (int)(min(c1, qs + A.rpt) - qs);
+        // what finishes a column of one chunk, fetched before the waits
+        int r = pair_rhs<NR>(lane);
+        bool wr = pair_writer<NR>(lane);
+        float2 yi = make_float2(0.f, 0.f);
+        double di = 0.0;
+        if constexpr (NR <= KC_SOLVE_EARLY) {
+            if (wr) yi = A.yf[(int64_t)i * NR + r];
+            di = A.diag[i];
+        }
         float s[PL::NRL], c[PL::NRL];
 #pragma unroll
         for (int r = 0; r < PL::NRL; ++r) s[r] = c[r] = 0.f;
@@ -554,31 +612,29 @@ __global__ void __launch_bounds__(256, KC_SOLVE_MINB) bwd_solve_pair_k(SolveArgs
                 jj[u] = q < nq ? __ldg(&A.rowidx[qs + q]) : -1;
                 w[u] = q < nq ? __ldg(&A.val[__ldg(&A.slot[qs + q])]) : 0.f;
             }
-            if (!points_ready<D>(A.ready, jj, A.status, A.spin_limit)) {
+            if (!__all_sync(FULL, gather_pair_add<NR, D>(A.xf, jj, w, block, s, c, A.status, A.spin_limit))) {
                 if (lane == 0) atomicCAS(A.status, 0, DEV_TIMEOUT);
                 return;
             }
-            gather_pair_add<NR, D>(A.xf, jj, w, block, s, c);
         }
         double sum = reduce_scatter_pair<NR>(s, c, lane);
-        bool wr = pair_writer<NR>(lane);
-        int r = pair_rhs<NR>(lane);
         bool finish = true;
         if (nch > 1) {
             if (wr) A.acc[ti * NR + r] = sum;
             finish = combine_chunks<NR>(A.acc, A.gcnt, A.cnt, i, ti, ch, nch, lane, sum);
             wr = lane < NR;  // the combined sums: right-hand side lane % NR
             r = lane % NR;
+            if constexpr (NR <= KC_SOLVE_EARLY) yi = A.yf[(int64_t)i * NR + r];
         }
-        if (finish) {
-            if (wr) {
-                double di = A.diag[i];
-                if (!(di > 0.0)) di = A.diag_fallback;
-                const double xi = (value_of(A.yf[(int64_t)i * NR + r]) - sum) / di;
-                A.xf[(int64_t)i * NR + r] = pair_of(xi);
-                A.x[(int64_t)i * NR + r] = xi;
+        if (finish && wr) {
+            if constexpr (NR > KC_SOLVE_EARLY) {
+                yi = A.yf[(int64_t)i * NR + r];
+                di = A.diag[i];
             }
-            publish_ready(&A.ready[i], lane);
+            if (!(di > 0.0)) di = A.diag_fallback;
+            const double xi = (value_of(yi) - sum) / di;
+            st_value((unsigned long long*)A.xf + (int64_t)i * NR + r, word_of(pair_of(xi)));
+            A.x[(int64_t)i * NR + r] = xi;
         }
     }
 }
@@ -611,11 +667,20 @@ __global__ void from_point_major_k(const double* __restrict__ xp, const int32_t*
 
 kc_status solver_init(Solver& S, const kc_pattern* P, int nrhs_cap, const kc_opts* o, Arena& A, cudaStream_t s) {
     S.P = P;
-    S.rpt = (o && o->rows_per_task > 0) ? o->rows_per_task : KC_SOLVE_ROWS;
+    S.rpt = (o && o->rows_per_task > 0) ? o->rows_per_task : 0;
+    if (S.rpt == 0) {
+        // Few right-hand sides and more chunks per level than resident warps: longer
+        // chunks, so that a column has fewer sums to combine (2^20 points, rho = 3,
+        // one right-hand side: 128 rows 7.9 ms, 256 6.7, 512 6.7; 16 right-hand
+        // sides: 12.1, 12.4, 13.9).
+        S.rpt = KC_SOLVE_ROWS;
+        const int64_t warps = (int64_t)sm_count() * 32;
+        if (nrhs_cap <= 4 && tasks_bound(P, KC_SOLVE_ROWS) > warps * (P->depth > 0 ? P->depth : 1)) S.rpt = 2 * KC_SOLVE_ROWS;
+    }
     if (o && o->spin_limit_cycles > 0) S.spin = o->spin_limit_cycles;
-    KC_TRY(build_tasks(P, S.rpt, A, s, &S.tasks, nullptr, &S.ntasks));
+    KC_TRY(build_tasks(P, S.rpt, A, s, &S.tasks, &S.ntasks_dev, nullptr));
+    S.ntasks = tasks_bound(P, S.rpt);
     S.nrhs_cap = nrhs_cap;
-    KC_TRY(A.get(&S.ready, P->N));
     KC_TRY(A.get(&S.cnt, P->N));
     KC_TRY(A.get(&S.acc, S.ntasks * nrhs_cap));
     KC_TRY(A.get(&S.gcnt, S.ntasks));
@@ -630,22 +695,34 @@ kc_status solver_init(Solver& S, const kc_pattern* P, int nrhs_cap, const kc_opt
 // the status word is checked by solver_check.
 template <typename T, int NR>
 static kc_status solve_launch(Solver& S, SolveArgs<T> a, int nrhs, cudaStream_t s) {
+    constexpr bool PAIR = std::is_same<T, float>::value;
     const kc_pattern* P = S.P;
-    const int grid = sm_count() * 8;
-    KC_CUDA(cudaMemsetAsync(S.ready, 0, sizeof(int) * P->N, s));
+    // CTAs of 8 warps: as many as fit, and no more than about KC_SOLVE_WAVES
+    // warps per row (column chunk) of a dependency level; the rows go out in level
+    // order, so further warps would only wait and poll.
+    auto launch = [&](void (*kfn)(SolveArgs<T>), int64_t items) -> kc_status {
+        int per_sm = 0;
+        KC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kfn, 256, 0));
+        const double want = KC_SOLVE_WAVES * (double)items / (double)(P->depth > 0 ? P->depth : 1);
+        const int64_t full = (int64_t)sm_count() * (per_sm > 0 ? per_sm : 1);
+        const int64_t ctas = (int64_t)(want / 8.0) + 1;
+        ::kc::note_launch(), kfn<<<(unsigned)(ctas < full ? ctas : full), 256, 0, s>>>(a);
+        KC_CUDA(cudaGetLastError());
+        return KC_OK;
+    };
+    const size_t words = sizeof(unsigned long long) * (size_t)P->N * NR;
+    KC_CUDA(cudaMemsetAsync(S.y, 0xff, words, s));  // unset
+    KC_CUDA(cudaMemsetAsync(PAIR ? (void*)S.xf : (void*)a.x, 0xff, words, s));
     KC_CUDA(cudaMemsetAsync(S.ticket, 0, 2 * sizeof(unsigned long long), s));
     KC_CUDA(cudaMemsetAsync(S.status, 0, sizeof(int), s));
-    a.ticket = S.ticket;
-    if constexpr (std::is_same<T, float>::value) ::kc::note_launch(), fwd_solve_pair_k<NR><<<grid, 256, 0, s>>>(a);
-    else ::kc::note_launch(), fwd_solve_k<T, NR><<<grid, 256, 0, s>>>(a);
-    KC_CUDA(cudaGetLastError());
-    KC_CUDA(cudaMemsetAsync(S.ready, 0, sizeof(int) * P->N, s));
     KC_CUDA(cudaMemsetAsync(S.cnt, 0, sizeof(unsigned) * P->N, s));
     KC_CUDA(cudaMemsetAsync(S.gcnt, 0, sizeof(unsigned) * S.ntasks, s));
+    a.ticket = S.ticket;
+    if constexpr (PAIR) KC_TRY(launch(fwd_solve_pair_k<NR>, P->N));
+    else KC_TRY(launch(fwd_solve_k<T, NR>, P->N));
     a.ticket = S.ticket + 1;
-    if constexpr (std::is_same<T, float>::value) ::kc::note_launch(), bwd_solve_pair_k<NR><<<grid, 256, 0, s>>>(a);
-    else ::kc::note_launch(), bwd_solve_k<T, NR><<<grid, 256, 0, s>>>(a);
-    KC_CUDA(cudaGetLastError());
+    if constexpr (PAIR) KC_TRY(launch(bwd_solve_pair_k<NR>, S.ntasks));
+    else KC_TRY(launch(bwd_solve_k<T, NR>, S.ntasks));
     return KC_OK;
 }
 
@@ -684,7 +761,7 @@ static SolveArgs<T> solve_args(Solver& S, const T* val, const double* diag, doub
     a.slot = P->slot;
     a.order = P->order;
     a.tasks = S.tasks;
-    a.ntasks = S.ntasks;
+    a.ntasks = S.ntasks_dev;
     a.rpt = S.rpt;
     a.val = val;
     a.diag = diag;
@@ -697,7 +774,6 @@ static SolveArgs<T> solve_args(Solver& S, const T* val, const double* diag, doub
     a.acc = S.acc;
     a.cnt = S.cnt;
     a.gcnt = S.gcnt;
-    a.ready = S.ready;
     a.status = S.status;
     a.spin_limit = S.spin;
     return a;

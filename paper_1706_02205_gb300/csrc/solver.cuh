@@ -7,9 +7,9 @@ namespace kc {
 struct Solver {
     const kc_pattern* P = nullptr;
     int2* tasks = nullptr;
-    int64_t ntasks = 0;
+    const int64_t* ntasks_dev = nullptr;  // tasks of the backward solve
+    int64_t ntasks = 0;                   // at most
     int rpt = 64;
-    int* ready = nullptr;
     unsigned* cnt = nullptr;
     unsigned* gcnt = nullptr;
     double* acc = nullptr;
@@ -21,6 +21,7 @@ struct Solver {
     long long spin = 4000000000LL;
 };
 
+int64_t tasks_bound(const kc_pattern* P, int rpt);
 kc_status build_tasks(const kc_pattern* P, int rpt, Arena& A, cudaStream_t s, int2** tasks_out,
                       const int64_t** count_out, int64_t* ntasks_out, bool adaptive = false);
 kc_status solver_init(Solver& S, const kc_pattern* P, int nrhs_cap, const kc_opts* o, Arena& A, cudaStream_t s);
