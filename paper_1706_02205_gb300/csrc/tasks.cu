@@ -20,25 +20,68 @@ namespace kc {
 constexpr int TK_THREADS = 256;
 constexpr int TK_WARPS = TK_THREADS / 32;
 
+// Lane layout of the products: an entry's NS vectors are split over P lanes of
+// NSL each, so a warp works on 32 / P entries at a time and a lane keeps NSL
+// sums.  With one entry per lane and NS sums each, the butterflies at the end of
+// a row (5 NS additions a lane) took as long as its products: the FP64 pipe (two
+// lanes a clock and SM) bounds these kernels.  Measured at 2^20 points, rho = 3,
+// FP32 form, 16 vectors, L L^T v: 27.0 -> 13.2 ms, of which the FP64 pipe takes 9.6.
 template <int NS>
-__device__ __forceinline__ void gather_fma(double (&acc)[NS], double w, const double* __restrict__ z, int64_t k) {
-    const double* p = z + k * NS;
+struct MvLayout {
+    static constexpr int NSL = NS < 4 ? NS : 4;
+    static constexpr int P = NS / NSL;
+    static constexpr int EL = 32 / P;  // entries at a time
+};
+
+// acc[r] += w v[k * NS + part + r] over 32 entries of the row (column), entry
+// t held by lane t (w = 0 past its end, k then anything valid)
+template <int NS>
+__device__ __forceinline__ void block_fma(double (&acc)[MvLayout<NS>::NSL], int k, double w, int cnt,
+                                          const double* __restrict__ v, int lane) {
+    using ML = MvLayout<NS>;
+    const int el = lane / ML::P, part = (lane % ML::P) * ML::NSL;
 #pragma unroll
-    for (int r = 0; r < NS; ++r) acc[r] = fma(w, __ldg(p + r), acc[r]);
+    for (int t0 = 0; t0 < 32; t0 += ML::EL) {
+        const int kk = ML::P == 1 ? k : __shfl_sync(0xffffffffu, k, t0 + el);
+        const double ww = ML::P == 1 ? w : __shfl_sync(0xffffffffu, w, t0 + el);
+        if (t0 + el < cnt) {
+            const double* p = v + (int64_t)kk * NS + part;
+            if constexpr (ML::NSL == 1) {
+                acc[0] = fma(ww, __ldg(p), acc[0]);
+            } else {
+#pragma unroll
+                for (int r = 0; r < ML::NSL; r += 2) {
+                    const double2 x = __ldg((const double2*)(p + r));
+                    acc[r] = fma(ww, x.x, acc[r]);
+                    acc[r + 1] = fma(ww, x.y, acc[r + 1]);
+                }
+            }
+        }
+    }
 }
 
-// lanes 0..NS-1 write y[j*NS + r] = (warp total of acc[r]) + dj * z[j*NS + r]
+// The warp's total of one vector: a reduce-scatter over the lanes of one part
+// (the sums a lane keeps halve, then plain sums).  The lane ends with the total
+// of vector `r`; `writer` is true in one lane per vector.
 template <int NS>
-__device__ __forceinline__ void finish_row(double (&acc)[NS], double dj, const double* __restrict__ z, int64_t j,
-                                           double* __restrict__ y) {
-    const int lane = lane_id();
-    double mine = 0.0;
+__device__ __forceinline__ double warp_total(double (&acc)[MvLayout<NS>::NSL], int lane, int& r, bool& writer) {
+    using ML = MvLayout<NS>;
+    r = (lane % ML::P) * ML::NSL;
+    int o = 16;
 #pragma unroll
-    for (int r = 0; r < NS; ++r) {
-        const double t = warp_sum(acc[r]);  // butterfly: every lane holds the same bits
-        if (lane == r) mine = t;
+    for (int h = ML::NSL / 2; h >= 1; h >>= 1, o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int q = 0; q < h; ++q) {
+            const double send = up ? acc[q] : acc[q + h], keep = up ? acc[q + h] : acc[q];
+            acc[q] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+        if (up) r += h;
     }
-    if (lane < NS) y[j * NS + lane] = fma(dj, z[j * NS + lane], mine);
+    writer = (lane & (2 * o - 1) & ~(ML::P - 1)) == 0;
+#pragma unroll
+    for (; o >= ML::P; o >>= 1) acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], o);
+    return acc[0];
 }
 
 // y = L z: row j of L is col/val[rowptr[j] .. rowptr[j+1]-1), the diagonal last
@@ -50,13 +93,21 @@ __global__ void __launch_bounds__(TK_THREADS) l_rows_k(const int64_t* __restrict
                                                        const double* __restrict__ z, double* __restrict__ y) {
     const int64_t j = (int64_t)blockIdx.x * TK_WARPS + (threadIdx.x >> 5);
     if (j >= N) return;
-    double acc[NS];
-#pragma unroll
-    for (int r = 0; r < NS; ++r) acc[r] = 0.0;
-    const int64_t e1 = rowptr[j + 1] - 1;
-#pragma unroll 4
-    for (int64_t e = rowptr[j] + lane_id(); e < e1; e += 32) gather_fma<NS>(acc, (double)__ldg(&val[e]), z, __ldg(&col[e]));
-    finish_row<NS>(acc, diag[j], z, j, y);
+    const int lane = lane_id();
+    double acc[MvLayout<NS>::NSL] = {};
+    const int64_t e0 = rowptr[j];
+    const int n = (int)(rowptr[j + 1] - 1 - e0);
+#pragma unroll (NS <= 2 ? 4 : 2)
+    for (int t = 0; t < n; t += 32) {
+        const bool in = t + lane < n;
+        const int k = in ? __ldg(&col[e0 + t + lane]) : 0;
+        const double w = in ? (double)__ldg(&val[e0 + t + lane]) : 0.0;
+        block_fma<NS>(acc, k, w, n - t, z, lane);
+    }
+    int r;
+    bool writer;
+    const double s = warp_total<NS>(acc, lane, r, writer);
+    if (writer) y[j * NS + r] = fma(diag[j], z[j * NS + r], s);
 }
 
 // y = L^T v: column i of L is rowidx[colptr[i] .. colptr[i+1]), the diagonal
@@ -95,23 +146,22 @@ __global__ void __launch_bounds__(TK_THREADS) lt_chunks_k(const int64_t* __restr
     const int64_t k = c - off[i];
     const int64_t q0 = colptr[i] + 1 + k * LT_CHUNK;
     const int64_t q1 = min(colptr[i + 1], q0 + LT_CHUNK);
-    double acc[NS];
-#pragma unroll
-    for (int r = 0; r < NS; ++r) acc[r] = 0.0;
-#pragma unroll 4
-    for (int64_t q = q0 + lane_id(); q < q1; q += 32)
-        gather_fma<NS>(acc, (double)__ldg(&val[__ldg(&slot[q])]), v, __ldg(&rowidx[q]));
-    if (off[i + 1] - off[i] == 1) {
-        finish_row<NS>(acc, diag[i], v, i, y);
-    } else {
-        const int lane = lane_id();
-        double mine = 0.0;
-#pragma unroll
-        for (int r = 0; r < NS; ++r) {
-            const double t = warp_sum(acc[r]);
-            if (lane == r) mine = t;
-        }
-        if (lane < NS) part[c * NS + lane] = mine;
+    const int lane = lane_id();
+    double acc[MvLayout<NS>::NSL] = {};
+    const int n = (int)(q1 - q0);
+#pragma unroll (NS <= 2 ? 4 : 2)
+    for (int t = 0; t < n; t += 32) {
+        const bool in = t + lane < n;
+        const int j = in ? __ldg(&rowidx[q0 + t + lane]) : 0;
+        const double w = in ? (double)__ldg(&val[__ldg(&slot[q0 + t + lane])]) : 0.0;
+        block_fma<NS>(acc, j, w, n - t, v, lane);
+    }
+    int r;
+    bool writer;
+    const double s = warp_total<NS>(acc, lane, r, writer);
+    if (writer) {
+        if (off[i + 1] - off[i] == 1) y[(int64_t)i * NS + r] = fma(diag[i], v[(int64_t)i * NS + r], s);
+        else part[c * NS + r] = s;
     }
 }
 
