@@ -3,14 +3,16 @@
 // The refined solve is CG on the dense Theta (task (2) of Section 1) with the
 // factor as preconditioner, M = L L^T (Section 4.3 suggests CG preconditioned
 // with the factor).  Theta is never stored: Theta v is evaluated from the
-// coordinates, FP64 throughout, O(N^2) per product.  The masked matrix Theta
-// restricted to S is not positive definite in general, so it is not used as
-// the CG operator.
+// coordinates to FP64 accuracy, O(N^2) per product: for the closed-form Matern
+// kernels by split entries on the tensor cores (dense.cu), for the other
+// covariance functions in FP64 below.  The masked matrix Theta restricted to S
+// is not positive definite in general, so it is not used as the CG operator.
 //
 // a9's error check uses the same dense product with FP32 entries and
 // compensated (Dot2) tile sums combined in FP64.
-#include "solver.cuh"
 #include "covariance.cuh"
+#include "dense.cuh"
+#include "solver.cuh"
 
 namespace kc {
 
@@ -219,9 +221,11 @@ struct CgOperator {
     const double* x_ord = nullptr;
     int d = 0;
     KernelParams kp{};
+    DenseSplit split{};  // closed-form kernels: entries and vectors split (dense.cu)
     SparseOp M{};
     kc_status apply(int64_t N, const double* v, double* y, int ns, cudaStream_t s) const {
         if (M.arp) return sparse_pos_mv(M, N, v, y, ns, s);
+        if (split.vf) return dense_theta_split(split, x_ord, N, d, kp, v, y, ns, s);
         return dense_theta_f64(x_ord, N, d, kp, v, y, ns, s);
     }
 };
@@ -271,6 +275,7 @@ static kc_status refine_core(const kc_pattern* P, CgOperator& op, double fb, int
     while (ns < nrhs) ns <<= 1;  // padded slot count (extra columns stay zero)
     Solver S;
     KC_TRY(solver_init(S, P, ns, o, A, s));
+    if (!op.M.arp && op.kp.nu_code <= 2) KC_TRY(dense_split_init(op.split, N, ns, A, s));
     const int64_t n = N * ns;
     double *bp, *xs, *r, *z, *p, *q, *partial, *sc;
     int* active;
