@@ -44,24 +44,45 @@ kc_status scratch_alloc(void** p, size_t bytes, cudaStream_t s);
 kc_status scratch_trim(int64_t keep_bytes);
 
 // Stream-ordered scratch: every buffer is freed (cudaFreeAsync) when the
-// arena goes out of scope, after the work enqueued before that point.
+// arena goes out of scope, after the work enqueued before that point.  Small
+// buffers (up to a quarter of ARENA_CHUNK) are cut from chunks, because every
+// allocation and release is a driver call of some microseconds (more once a
+// process has used many streams) and a call on a few thousand points asks for
+// dozens of buffers of some KB.
+constexpr size_t ARENA_CHUNK = 4u << 20;
 struct Arena {
     cudaStream_t s;
     static constexpr int CAP = 128;
     void* ptrs[CAP];
     int n = 0;
+    unsigned char* chunk = nullptr;  // the rest of the current chunk
+    size_t left = 0;
     explicit Arena(cudaStream_t st) : s(st) {}
     ~Arena() {
         for (int i = n - 1; i >= 0; --i) cudaFreeAsync(ptrs[i], s);
     }
+    kc_status raw(void** out, size_t bytes) {
+        if (n == CAP) return fail(KC_ENOMEM, "scratch arena full");
+        KC_TRY(scratch_alloc(out, bytes, s));
+        ptrs[n++] = *out;
+        return KC_OK;
+    }
     template <typename T>
     kc_status get(T** out, size_t count) {
-        if (n == CAP) return fail(KC_ENOMEM, "scratch arena full");
+        const size_t bytes = (count * sizeof(T) + 255) / 256 * 256 + (count == 0 ? 256 : 0);
         void* p = nullptr;
-        size_t bytes = count * sizeof(T);
-        if (bytes == 0) bytes = 16;
-        KC_TRY(scratch_alloc(&p, bytes, s));
-        ptrs[n++] = p;
+        if (bytes > ARENA_CHUNK / 4) {
+            KC_TRY(raw(&p, bytes));
+        } else {
+            if (left < bytes) {
+                KC_TRY(raw(&p, ARENA_CHUNK));
+                chunk = (unsigned char*)p;
+                left = ARENA_CHUNK;
+            }
+            p = chunk;
+            chunk += bytes;
+            left -= bytes;
+        }
         *out = (T*)p;
         return KC_OK;
     }

@@ -121,12 +121,13 @@ kc_status bbox(const double* x, int64_t N, int d, double* lo, double* hi, Arena&
 // (the first three raw coordinates are an arbitrary projection of it).
 kc_status grid_coords(const double* x, int64_t N, int d, Arena& A, cudaStream_t s, const double** gx, int* gs);
 
-// Bounding box over all d <= 32 axes (host out), for the float copies used by
-// the FP32 distance screens; E = the largest extent.
+// Bounding box over all d <= 32 axes (host out; the low corner also for the float
+// copies used by the FP32 distance screens); E = the largest extent.  KC_EINVAL if
+// a coordinate is not finite.  One pass and one wait of the host.
 constexpr int MAXD = 32;
 struct Origin {
     double lo[MAXD];
 };
-kc_status bbox_all(const double* x, int64_t N, int d, Origin* lo, double* E, Arena& A, cudaStream_t s);
+kc_status points_bounds(const double* x, int64_t N, int d, Origin* lo, Origin* hi, double* E, Arena& A, cudaStream_t s);
 
 }  // namespace kc

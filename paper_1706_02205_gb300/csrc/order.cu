@@ -20,11 +20,19 @@
 //
 // Rounds run in bands of keys: with vmax the largest undecided v, the band
 // holds the undecided points with v >= vmax/4 (KC_ORDER_BAND); only band points can dominate
-// band points, so the dominance search uses a grid of band points with cell
-// size sqrt(vmax).  The updates scan a fixed fine grid of all points.
+// band points, so the dominance search uses a grid of band points with cells of
+// a quarter of sqrt(vmax) (more where the points are too few for that), whose
+// largest points alone are searched for where a cell holds several.  The updates
+// scan a fixed fine grid of all points.  All bands run in one cooperative launch.
 // Finally the points are sorted by (v descending, index ascending).
+//
+// Bound by latency: about 50 rounds of dependent scans, each between grid
+// barriers.  Measured (before: a dozen launches and two waits of the host per
+// round): 2^20 points of a jittered grid 16.0 -> 12.2 ms, 250,007 points of a
+// swiss roll in R^20 22.4 -> 18.6 (34 -> 18.7 in a process that has used many
+// streams, where every launch costs more), 131,071 points of the cube 13.3 ->
+// 9.5, 100,003 in the square 9.2 -> 5.8, 2000 4.6 -> 1.7.
 #include <algorithm>
-#include <chrono>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -33,24 +41,6 @@
 #include "grid.cuh"
 
 namespace kc {
-
-__global__ void finite_check_k(const double* __restrict__ x, int64_t n, int* __restrict__ bad) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n && !isfinite(x[i])) atomicExch(bad, 1);
-}
-
-kc_status check_finite(const double* x, int64_t n, Arena& A, cudaStream_t s) {
-    int* bad;
-    KC_TRY(A.get(&bad, 1));
-    KC_CUDA(cudaMemsetAsync(bad, 0, sizeof(int), s));
-    ::kc::note_launch(), finite_check_k<<<blocks_for(n, 256), 256, 0, s>>>(x, n, bad);
-    KC_CUDA(cudaGetLastError());
-    int h = 0;
-    KC_CUDA(cudaMemcpyAsync(&h, bad, sizeof(int), cudaMemcpyDeviceToHost, s));
-    KC_CUDA(cudaStreamSynchronize(s));
-    if (h) return fail(KC_EINVAL, "points must be finite");
-    return KC_OK;
-}
 
 // out[q] = rows ids[q] of the n x w array a
 __global__ void gather_rows_k(const double* __restrict__ a, int w, const int32_t* __restrict__ ids, int64_t n,
@@ -81,237 +71,6 @@ __global__ void ord_init_k(const double* __restrict__ x, int d, const int32_t* _
     }
 }
 
-// max of v2 over undecided points and their count
-__global__ void ord_vmax_k(const double* __restrict__ v2, const int* __restrict__ stat, int64_t N,
-                           unsigned long long* __restrict__ vmax_bits, unsigned long long* __restrict__ count) {
-    unsigned long long m = 0, c = 0;
-    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < N; q += (int64_t)gridDim.x * blockDim.x)
-        if (stat[q] == 0) {
-            m = max(m, (unsigned long long)__double_as_longlong(v2[q]));
-            c++;
-        }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-        c += __shfl_xor_sync(0xffffffffu, c, o);
-    }
-    if (lane_id() == 0) {
-        atomicMax(vmax_bits, m);
-        atomicAdd(count, c);
-    }
-}
-
-__global__ void ord_band_k(const double* __restrict__ v2, const int* __restrict__ stat, int64_t N, double T,
-                           int32_t* __restrict__ blist, unsigned long long* __restrict__ nb) {
-    int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (q < N && stat[q] == 0 && v2[q] >= T) blist[atomicAdd(nb, 1ULL)] = (int32_t)q;
-}
-
-// per band cell: the largest squared distance (as bits) of its undecided band
-// points, -1 if none; a dominance scan skips the cells whose largest value is
-// below its own (no point of larger key there)
-__global__ void ord_cellmax_k(const int32_t* __restrict__ bsorted, const int64_t* __restrict__ bstart,
-                              int64_t ncells, const double* __restrict__ v2, const int* __restrict__ stat,
-                              long long* __restrict__ cmax) {
-    const int64_t cidx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (cidx >= ncells) return;
-    long long m = -1;
-    const long long* __restrict__ v2b = (const long long*)v2;
-    for (int64_t f = bstart[cidx]; f < bstart[cidx + 1]; ++f) {
-        const int p = bsorted[f];
-        if (stat[p] == 0) m = max(m, v2b[p]);
-    }
-    cmax[cidx] = m;
-}
-
-#ifndef KC_DOM_BUDGET
-#define KC_DOM_BUDGET 256
-#endif
-constexpr int DOM_THREAD_BUDGET = KC_DOM_BUDGET;
-
-// One thread per band point: is it dominant?  Most band points meet a
-// dominator among their first candidates; a point whose scan would go past
-// DOM_THREAD_BUDGET candidates (an undominated point has to look at every
-// band point within sqrt(v)) is handed, undecided, to ord_dominance_warp_k.
-__global__ void ord_dominance_k(Grid gb, const int32_t* __restrict__ bsorted, const int64_t* __restrict__ bstart,
-                                int64_t nb, const double* __restrict__ xg, int d, const int32_t* __restrict__ idg,
-                                const double* __restrict__ v2, const int* __restrict__ stat, double T,
-                                int32_t* __restrict__ sel, unsigned long long* __restrict__ nsel,
-                                unsigned long long* __restrict__ nactive, const float* __restrict__ xgf,
-                                float delta, const long long* __restrict__ cmax, const double* __restrict__ gxg,
-                                int gs, int32_t* __restrict__ hard, unsigned long long* __restrict__ nhard) {
-    int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= nb) return;
-    const int q = bsorted[e];
-    if (stat[q] != 0) return;
-    const double vq = v2[q];
-    if (!(vq >= T)) return;
-    const long long bq = __double_as_longlong(vq);
-    const long long* __restrict__ v2b = (const long long*)v2;
-    atomicAdd(nactive, 1ULL);
-    const double* xq = xg + (int64_t)q * d;
-    const float rq = sqrtf((float)vq);
-    const int idq = idg[q];
-    const double R = sqrt(vq);
-    // Scan the band grid ring by ring outward from q's cell, so a dominated
-    // point usually meets a dominator within the first rings; ring r holds no
-    // point closer than (r-1) cells.
-    const int dg = gb.dg;
-    int c[3] = {0, 0, 0};
-    int maxr = 0;
-    for (int t = 0; t < dg; ++t) {
-        c[t] = cell_coord(gb, gxg[(int64_t)q * gs + t], t);
-        maxr = max(maxr, span_for(gb, R, t));
-    }
-    bool dom = true;
-    int budget = DOM_THREAD_BUDGET;  // candidates this thread examines before handing q to a warp
-    for (int r = 0; r <= maxr && dom; ++r) {
-        if (r >= 2 && (double)(r - 1) * gb.c > R) break;
-        const int z0 = dg > 2 ? max(0, c[2] - r) : 0, z1 = dg > 2 ? min(gb.n[2] - 1, c[2] + r) : 0;
-        const int y0 = dg > 1 ? max(0, c[1] - r) : 0, y1 = dg > 1 ? min(gb.n[1] - 1, c[1] + r) : 0;
-        for (int cz = z0; cz <= z1 && dom; ++cz)
-            for (int cy = y0; cy <= y1 && dom; ++cy) {
-                const bool edge = r == 0 || (dg > 2 && abs(cz - c[2]) == r) || (dg > 1 && abs(cy - c[1]) == r);
-                const int64_t base = ((int64_t)cz * gb.n[1] + cy) * gb.n[0];
-                // the cells of this ring in the row: all of [c-r, c+r] on an edge row, else the two ends
-                int seg[2][2];
-                int nseg = 0;
-                if (edge) {
-                    seg[0][0] = max(0, c[0] - r);
-                    seg[0][1] = min(gb.n[0] - 1, c[0] + r);
-                    nseg = 1;
-                } else {
-                    if (c[0] - r >= 0) {
-                        seg[nseg][0] = seg[nseg][1] = c[0] - r;
-                        ++nseg;
-                    }
-                    if (c[0] + r <= gb.n[0] - 1) {
-                        seg[nseg][0] = seg[nseg][1] = c[0] + r;
-                        ++nseg;
-                    }
-                }
-                for (int sg = 0; sg < nseg && dom; ++sg)
-                    for (int cx = seg[sg][0]; cx <= seg[sg][1] && dom; ++cx) {
-                        if (cmax[base + cx] < bq) continue;  // no larger key in this cell
-                        const int64_t f0 = bstart[base + cx], f1 = bstart[base + cx + 1];
-                        if (f1 - f0 > budget) {  // too many candidates left for one thread
-                            hard[atomicAdd(nhard, 1ULL)] = q;
-                            return;
-                        }
-                        budget -= (int)(f1 - f0);
-                        for (int64_t f = f0; f < f1; ++f) {
-                            const int p = bsorted[f];
-                            if (p == q || stat[p] != 0) continue;
-                            const long long bp = v2b[p];
-                            if (bp > bq || (bp == bq && idg[p] < idq)) {
-                                if (xgf && screen_f32(xgf + (int64_t)p * d, xgf + (int64_t)q * d, d, rq, delta) == 0)
-                                    continue;  // surely farther than sqrt(vq)
-                                if (dist2_exact(xg + (int64_t)p * d, xq, d) < vq) {
-                                    dom = false;
-                                    break;
-                                }
-                            }
-                        }
-                    }
-            }
-    }
-    if (dom) sel[atomicAdd(nsel, 1ULL)] = q;
-}
-
-// The points the threads handed over, one warp each (grid-stride over the
-// list): the same scan in the same ring and cell order, a cell's points 32 at
-// a time, so a long scan costs a 32nd of a serial one (with a thread per
-// point those few scans were the whole duration of a round).
-__global__ void ord_dominance_warp_k(Grid gb, const int32_t* __restrict__ hard,
-                                     const unsigned long long* __restrict__ nhard, const int64_t* __restrict__ bstart,
-                                     const int32_t* __restrict__ bsorted, const double* __restrict__ xg, int d,
-                                     const int32_t* __restrict__ idg, const double* __restrict__ v2,
-                                     const int* __restrict__ stat, int32_t* __restrict__ sel,
-                                     unsigned long long* __restrict__ nsel, const float* __restrict__ xgf, float delta,
-                                     const long long* __restrict__ cmax, const double* __restrict__ gxg, int gs) {
-    const int lane = lane_id();
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int64_t nh = (int64_t)*nhard;
-    for (int64_t e = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; e < nh; e += nw) {
-        const int q = hard[e];
-        const double vq = v2[q];
-        const long long bq = __double_as_longlong(vq);
-        const long long* __restrict__ v2b = (const long long*)v2;
-        const double* xq = xg + (int64_t)q * d;
-        const float rq = sqrtf((float)vq);
-        const int idq = idg[q];
-        const double R = sqrt(vq);
-        const int dg = gb.dg;
-        int c[3] = {0, 0, 0};
-        int maxr = 0;
-        for (int t = 0; t < dg; ++t) {
-            c[t] = cell_coord(gb, gxg[(int64_t)q * gs + t], t);
-            maxr = max(maxr, span_for(gb, R, t));
-        }
-        bool dom = true;  // uniform across the warp
-        for (int r = 0; r <= maxr && dom; ++r) {
-            if (r >= 2 && (double)(r - 1) * gb.c > R) break;
-            const int z0 = dg > 2 ? max(0, c[2] - r) : 0, z1 = dg > 2 ? min(gb.n[2] - 1, c[2] + r) : 0;
-            const int y0 = dg > 1 ? max(0, c[1] - r) : 0, y1 = dg > 1 ? min(gb.n[1] - 1, c[1] + r) : 0;
-            for (int cz = z0; cz <= z1 && dom; ++cz)
-                for (int cy = y0; cy <= y1 && dom; ++cy) {
-                    const bool edge = r == 0 || (dg > 2 && abs(cz - c[2]) == r) || (dg > 1 && abs(cy - c[1]) == r);
-                    const int64_t base = ((int64_t)cz * gb.n[1] + cy) * gb.n[0];
-                    int seg[2][2];
-                    int nseg = 0;
-                    if (edge) {
-                        seg[0][0] = max(0, c[0] - r);
-                        seg[0][1] = min(gb.n[0] - 1, c[0] + r);
-                        nseg = 1;
-                    } else {
-                        if (c[0] - r >= 0) {
-                            seg[nseg][0] = seg[nseg][1] = c[0] - r;
-                            ++nseg;
-                        }
-                        if (c[0] + r <= gb.n[0] - 1) {
-                            seg[nseg][0] = seg[nseg][1] = c[0] + r;
-                            ++nseg;
-                        }
-                    }
-                    for (int sg = 0; sg < nseg && dom; ++sg)
-                        for (int cx = seg[sg][0]; cx <= seg[sg][1] && dom; ++cx) {
-                            if (cmax[base + cx] < bq) continue;  // no larger key in this cell
-                            const int64_t f0 = bstart[base + cx], f1 = bstart[base + cx + 1];
-                            for (int64_t fb = f0; fb < f1 && dom; fb += 32) {
-                                bool hit = false;
-                                const int64_t f = fb + lane;
-                                if (f < f1) {
-                                    const int p = bsorted[f];
-                                    if (p != q && stat[p] == 0) {
-                                        const long long bp = v2b[p];
-                                        if (bp > bq || (bp == bq && idg[p] < idq)) {
-                                            const bool far = xgf && screen_f32(xgf + (int64_t)p * d, xgf + (int64_t)q * d,
-                                                                               d, rq, delta) == 0;
-                                            hit = !far && dist2_exact(xg + (int64_t)p * d, xq, d) < vq;
-                                        }
-                                    }
-                                }
-                                if (__any_sync(0xffffffffu, hit)) dom = false;
-                            }
-                        }
-                }
-        }
-        if (dom && lane == 0) sel[atomicAdd(nsel, 1ULL)] = q;
-    }
-}
-
-// ---- greedy steps for the coarsest points: each step selects the argmax of
-// the previous step's per-block candidates and pushes it to every point.
-constexpr int GREEDY_BLOCKS_PER_SM = 4;
-#ifndef KC_GREEDY_STEPS
-#define KC_GREEDY_STEPS 256
-#endif
-constexpr int64_t GREEDY_STEPS = KC_GREEDY_STEPS;  // coarsest points selected one at a time
-// A band holds the undecided points with v >= KC_ORDER_BAND * (largest v).
-#ifndef KC_ORDER_BAND
-#define KC_ORDER_BAND 0.25
-#endif
-
 // Keys compare on the bit patterns of the squared distances: for v >= 0
 // (and +inf) IEEE doubles order like their bits as integers, and integer
 // compares stay off the GB300's small FP64 pipe.
@@ -321,37 +80,313 @@ __device__ __forceinline__ bool key_above(double va, int ia, double vb, int ib) 
     return a > b || (a == b && ia < ib);
 }
 
-// per-block best (v2 desc, original index asc) over undecided points; cand_g = -1 if none
-__device__ void block_best(double v, int id, int g, double* sv, int* si, int* sg, double* out_v, int* out_i,
-                           int* out_g) {
-    for (int o = 16; o > 0; o >>= 1) {
-        double v2o = __shfl_xor_sync(0xffffffffu, v, o);
-        int i2 = __shfl_xor_sync(0xffffffffu, id, o);
-        int g2 = __shfl_xor_sync(0xffffffffu, g, o);
-        if (g2 >= 0 && (g < 0 || key_above(v2o, i2, v, id))) {
-            v = v2o;
-            id = i2;
-            g = g2;
+#ifndef KC_DOM_BUDGET
+#define KC_DOM_BUDGET 32
+#endif
+constexpr int DOM_THREAD_BUDGET = KC_DOM_BUDGET;
+
+// What the band rounds read and write.  v2 and stat change between the phases of
+// one launch: they go without __restrict__, so that they are never read through
+// the non-coherent path.
+struct BandArgs {
+    int64_t N;
+    int d, gs;
+    Grid g0;                            // fine grid of all points
+    const int64_t* __restrict__ cstart;  // its cells
+    const double* __restrict__ xg;      // coordinates in grid order
+    const float* __restrict__ xgf;      // float copy minus the box corner
+    const double* __restrict__ gxg;     // grid coordinates (stride gs)
+    const int4* __restrict__ pcell;     // a point's cell on the fine grid
+    const int32_t* __restrict__ idg;
+    float delta;
+    double* v2;
+    int* stat;
+    int32_t *blist, *bcell, *bsorted, *bcnt, *bstart, *hard, *sel;
+    long long* cmax;
+    int32_t* champ;                     // the cell's undecided point of largest key (dense bands)
+    int32_t* wit;                       // a point that dominated it, -1: none yet
+    double* wd;                         // and its squared distance
+    int* part;                          // scan: one sum per block
+    struct BandCtl* ctl;
+    double lo[3], hi[3];
+    long long limit;
+};
+// Counters: of a band by its parity, of a round modulo 3 (reset two phases before their next use).
+struct BandCtl {
+    unsigned long long vmax[2];
+    unsigned open[2], nb[2], occ[2];
+    unsigned nsel[3], nact[3], nhard[3];
+    unsigned bar, gen;
+    int status, rounds;
+};
+
+// Band grid: cells a quarter of the largest search radius, at most about 2 nb of
+// them (any grid gives the same order).
+__device__ __noinline__ void band_grid(const BandArgs& A, double vmax, int64_t nb, Grid& g) {
+    g.dg = A.g0.dg;
+    g.c = g.inv_c = 1.0;
+    g.n[0] = g.n[1] = g.n[2] = 1;
+    g.ncells = 1;
+    double vol = 1.0, emax = 0.0, ext[3] = {0.0, 0.0, 0.0};
+    int nz = 0;
+    for (int t = 0; t < g.dg; ++t) {
+        g.lo[t] = A.lo[t];
+        ext[t] = A.hi[t] - A.lo[t];
+        if (ext[t] > 0.0) {
+            vol *= ext[t];
+            ++nz;
+        }
+        emax = fmax(emax, ext[t]);
+    }
+    if (!(emax > 0.0)) return;
+    const int64_t most = 2 * nb + 1;
+    const double q = vol / (double)most;
+    double c = nz == 1 ? q : nz == 2 ? sqrt(q) : cbrt(q);
+    c = fmax(c, 0.25 * sqrt(vmax));
+    for (int step = 0; step < 4096; ++step) {
+        int64_t tot = 1;
+        bool fits = c > 0.0;
+        for (int t = 0; t < g.dg && fits; ++t) {
+            const double f = floor(ext[t] / c) + 1.0;
+            if (!(f <= 1e6)) fits = false;
+            else {
+                g.n[t] = (int)f;
+                tot *= g.n[t];
+                fits = tot <= most;
+            }
+        }
+        if (fits) {
+            g.ncells = tot;
+            g.c = c;
+            g.inv_c = 1.0 / c;
+            return;
+        }
+        c = c > 0.0 ? c * 1.25 : emax * 1e-6;
+    }
+    g.n[0] = g.n[1] = g.n[2] = 1;  // a degenerate box: one cell
+    g.ncells = 1;
+    g.c = 2.0 * emax;
+    g.inv_c = 1.0 / g.c;
+}
+
+// Cells to either side of a point's own that cover sqrt(v) on the grid g, by FP32
+// arithmetic with slack (a larger box is as good) where float holds v.
+__device__ __forceinline__ int span_of_v(const Grid& g, double v, float inv_c, int t) {
+    if (!(v > 1e-30 && v < 1e30 && inv_c > 1e-30f && inv_c < 1e30f)) return span_for(g, sqrt(v), t);
+    const float f = sqrtf((float)v) * inv_c * (1.0f + 1e-5f) + 1e-5f;
+    return f > (float)g.n[t] ? g.n[t] : min(g.n[t], (int)f + 1);
+}
+
+// Does the undecided band point p dominate q (larger key, closer than sqrt(vq))?
+// Its squared distance if it does, else infinity.
+__device__ __forceinline__ double dominates(const BandArgs& A, int p, int q, double vq, float rq, int idq) {
+    if (p == q || A.stat[p] != 0) return INFINITY;
+    if (!key_above(A.v2[p], A.idg[p], vq, idq)) return INFINITY;
+    if (screen_f32(A.xgf + (int64_t)p * A.d, A.xgf + (int64_t)q * A.d, A.d, rq, A.delta) == 0) return INFINITY;
+    const double dd = dist2_exact(A.xg + (int64_t)p * A.d, A.xg + (int64_t)q * A.d, A.d);
+    return dd < vq ? dd : INFINITY;
+}
+
+// A point that dominates the undecided band point q, with its squared distance
+// in wd; -1: none, q is dominant.  One thread scans the band grid ring by ring
+// outward from q's cell: most points meet a dominator within the first rings
+// (ring r holds no point closer than (r-1) cells).  It gives up (-2) when the
+// scan would go past DOM_THREAD_BUDGET candidates: an undominated point has to look at every band point within sqrt(v), which is a
+// warp's work.
+__device__ __forceinline__ int dominator_thread(const BandArgs& A, const Grid& gb, int q, double vq, double& wd) {
+    const long long bq = vbits(vq);
+    const float rq = sqrtf((float)vq);
+    const int idq = A.idg[q];
+    const double R = sqrt(vq);
+    const int dg = gb.dg;
+    int c[3] = {0, 0, 0};
+    int maxr = 0;
+    for (int t = 0; t < dg; ++t) {
+        c[t] = cell_coord(gb, A.gxg[(int64_t)q * A.gs + t], t);
+        maxr = max(maxr, span_for(gb, R, t));
+    }
+    int budget = DOM_THREAD_BUDGET;
+    for (int r = 0; r <= maxr; ++r) {
+        if (r >= 2 && (double)(r - 1) * gb.c > R) break;
+        const int z0 = dg > 2 ? max(0, c[2] - r) : 0, z1 = dg > 2 ? min(gb.n[2] - 1, c[2] + r) : 0;
+        const int y0 = dg > 1 ? max(0, c[1] - r) : 0, y1 = dg > 1 ? min(gb.n[1] - 1, c[1] + r) : 0;
+        for (int cz = z0; cz <= z1; ++cz)
+            for (int cy = y0; cy <= y1; ++cy) {
+                // the cells of this ring in the row: all of [c-r, c+r] on an edge row, else the two ends
+                const bool edge = r == 0 || (dg > 2 && abs(cz - c[2]) == r) || (dg > 1 && abs(cy - c[1]) == r);
+                const int64_t base = ((int64_t)cz * gb.n[1] + cy) * gb.n[0];
+                const int step = edge ? 1 : 2 * r;
+                for (int cx = c[0] - r; cx <= c[0] + r; cx += step) {
+                    if (cx < 0 || cx >= gb.n[0]) continue;
+                    if (A.cmax[base + cx] < bq) continue;  // no larger key in this cell
+                    const int f0 = A.bstart[base + cx], f1 = A.bstart[base + cx + 1];
+                    if (f1 - f0 > budget) return -2;
+                    budget -= f1 - f0;
+                    for (int f = f0; f < f1; ++f) {
+                        const int p = A.bsorted[f];
+                        const double dd = dominates(A, p, q, vq, rq, idq);
+                        if (dd < vq) {
+                            wd = dd;
+                            return p;
+                        }
+                    }
+                }
+            }
+    }
+    return -1;
+}
+
+// Lane whose range [inc - len, inc) holds m, from the inclusive sums inc of the lanes' lengths
+// (m past the last: any lane).
+__device__ __forceinline__ int which_row(int inc, int m) {
+    int row = 0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+        if (__shfl_sync(0xffffffffu, inc, row + o - 1) <= m) row += o;
+    return row;
+}
+
+// The same by a warp, a lane per cell of the box around q.  (With the warp on
+// one cell at a time the cells of a box were a chain of dependent loads.)
+template <bool DENSE>
+__device__ __forceinline__ int dominator_warp(const BandArgs& A, const Grid& gb, int q, double vq, double& wd) {
+    constexpr int SCAN = 4;
+    const unsigned FULL = 0xffffffffu;
+    const int lane = lane_id();
+    const long long bq = vbits(vq);
+    const float rq = sqrtf((float)vq);
+    const int idq = A.idg[q];
+    const double R = sqrt(vq);
+    int lo[3] = {0, 0, 0}, n[3] = {1, 1, 1};
+    for (int t = 0; t < gb.dg; ++t) {
+        const int c = cell_coord(gb, A.gxg[(int64_t)q * A.gs + t], t), sp = span_for(gb, R, t);
+        lo[t] = max(0, c - sp);
+        n[t] = min(gb.n[t] - 1, c + sp) - lo[t] + 1;
+    }
+    const int cells = n[0] * n[1] * n[2];
+    auto cell_at = [&](int t) {
+        const int row = t / n[0];
+        return ((int64_t)(lo[2] + row / n[1]) * gb.n[1] + lo[1] + row % n[1]) * gb.n[0] + lo[0] + t % n[0];
+    };
+    if constexpr (DENSE) {  // the cells' largest points first: they dominate nearly whatever is dominated
+        for (int t0 = 0; t0 < cells; t0 += 32) {
+            int p = -1;
+            double dd = INFINITY;
+            if (t0 + lane < cells) {
+                const int64_t cell = cell_at(t0 + lane);
+                if (A.cmax[cell] >= bq) {
+                    p = A.champ[cell];  // there is one: its value is at least vq, so at least T
+                    dd = dominates(A, p, q, vq, rq, idq);
+                }
+            }
+            const unsigned hits = __ballot_sync(FULL, dd < vq);
+            if (hits) {
+                wd = __shfl_sync(FULL, dd, __ffs(hits) - 1);
+                return __shfl_sync(FULL, p, __ffs(hits) - 1);
+            }
         }
     }
-    const int w = threadIdx.x >> 5;
-    if (lane_id() == 0) {
-        sv[w] = v;
-        si[w] = id;
-        sg[w] = g;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int q = 1; q < (int)(blockDim.x >> 5); ++q)
-            if (sg[q] >= 0 && (g < 0 || key_above(sv[q], si[q], v, id))) {
-                v = sv[q];
-                id = si[q];
-                g = sg[q];
+    // then all points of the cells with a larger key, batches of 32 cells: their
+    // points go to the lanes in one sequence, four at a time so that their loads overlap
+    for (int t0 = 0; t0 < cells; t0 += 32) {
+        int f0 = 0, len = 0;
+        if (t0 + lane < cells) {
+            const int64_t cell = cell_at(t0 + lane);
+            if (A.cmax[cell] >= bq) {
+                f0 = A.bstart[cell];
+                len = A.bstart[cell + 1] - f0;
             }
-        *out_v = v;
-        *out_i = id;
-        *out_g = g;
+        }
+        int inc = len;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int up = __shfl_up_sync(FULL, inc, o);
+            if (lane >= o) inc += up;
+        }
+        const int total = __shfl_sync(FULL, inc, 31);
+        for (int m0 = 0; m0 < total; m0 += 32 * SCAN) {
+            int p[SCAN];
+#pragma unroll
+            for (int u = 0; u < SCAN; ++u) {
+                const int m = m0 + 32 * u + lane;
+                const int row = which_row(inc, m);
+                const int f = __shfl_sync(FULL, f0, row) + m - __shfl_sync(FULL, inc - len, row);
+                p[u] = m < total ? A.bsorted[f] : -1;
+            }
+            double v[SCAN];
+            int st[SCAN];
+#pragma unroll
+            for (int u = 0; u < SCAN; ++u) {
+                v[u] = p[u] >= 0 ? A.v2[p[u]] : 0.0;
+                st[u] = p[u] >= 0 ? A.stat[p[u]] : 1;
+            }
+            double dd = INFINITY;
+            int hit = -1;
+#pragma unroll
+            for (int u = 0; u < SCAN; ++u)
+                if (hit < 0 && st[u] == 0 && vbits(v[u]) >= bq) {
+                    dd = dominates(A, p[u], q, vq, rq, idq);
+                    if (dd < vq) hit = p[u];
+                }
+            const unsigned hits = __ballot_sync(FULL, hit >= 0);
+            if (hits) {
+                wd = __shfl_sync(FULL, dd, __ffs(hits) - 1);
+                return __shfl_sync(FULL, hit, __ffs(hits) - 1);
+            }
+        }
     }
+    return -1;
+}
+
+// one slot of a list per calling thread, by one atomic per group of threads
+__device__ __forceinline__ unsigned list_slot(unsigned* n) {
+    const unsigned m = __activemask();
+    const int leader = __ffs(m) - 1;
+    unsigned base = 0;
+    if (lane_id() == leader) base = atomicAdd(n, (unsigned)__popc(m));
+    return __shfl_sync(m, base, leader) + __popc(m & ((1u << lane_id()) - 1u));
+}
+
+// ---- greedy steps for the coarsest points: each step selects the argmax of
+// the previous step's per-block candidates and pushes it to every point.
+constexpr int GREEDY_THREADS = 1024;
+#ifndef KC_GREEDY_STEPS
+#define KC_GREEDY_STEPS 256
+#endif
+constexpr int64_t GREEDY_STEPS = KC_GREEDY_STEPS;  // coarsest points selected one at a time
+// A band holds the undecided points with v >= KC_ORDER_BAND * (largest v).
+#ifndef KC_ORDER_BAND
+#define KC_ORDER_BAND 0.25
+#endif
+
+// the better of two candidates (v2 desc, original index asc; g < 0: none)
+struct Cand {
+    double v;
+    int i, g;
+    __device__ __forceinline__ void take(double vo, int io, int go) {
+        if (go >= 0 && (g < 0 || key_above(vo, io, v, i))) {
+            v = vo;
+            i = io;
+            g = go;
+        }
+    }
+    __device__ __forceinline__ void warp_best() { best_of<16>(); }
+    template <int FROM>
+    __device__ __forceinline__ void best_of() {
+#pragma unroll
+        for (int o = FROM; o > 0; o >>= 1)
+            take(__shfl_xor_sync(0xffffffffu, v, o), __shfl_xor_sync(0xffffffffu, i, o), __shfl_xor_sync(0xffffffffu, g, o));
+    }
+};
+// the block's best candidate, in every thread (sh: 32 entries)
+__device__ __forceinline__ Cand block_best(Cand c, Cand* sh) {
+    c.warp_best();
+    __syncthreads();  // sh is free
+    if (lane_id() == 0) sh[threadIdx.x >> 5] = c;
+    __syncthreads();
+    c = lane_id() < (int)(blockDim.x >> 5) ? sh[lane_id()] : Cand{0.0, 0, -1};
+    c.warp_best();
+    return c;
 }
 
 // A grid-wide barrier for a cooperative launch (every block resident): the
@@ -389,129 +424,395 @@ __device__ bool grid_barrier(unsigned* count, unsigned* gen, int* status, long l
     return ok != 0;
 }
 
-// All greedy steps in one cooperative launch: phase 0 leaves every block's
-// candidate (no winner yet); phase k >= 1 takes the winner of phase k-1's
-// candidates (every block computes the same), marks it, pushes it to the
-// block's points and leaves the block's new candidate.  The candidates
-// alternate between two buffers; a grid barrier separates the phases.
-__global__ void ord_greedy_loop_k(const double* __restrict__ xg, int d, const int32_t* __restrict__ idg,
-                                  double* __restrict__ v2, int* __restrict__ stat, int64_t N, int64_t steps,
-                                  double* pv0, int* pi0, int* pg0, double* pv1, int* pi1, int* pg1,
-                                  const float* __restrict__ xgf, float delta, unsigned* bar, int* status,
-                                  long long limit) {
-    __shared__ double sv[32];
-    __shared__ int si[32], sg[32];
-    __shared__ double s_wv;
-    __shared__ int s_wi, s_wg;
-    const int nin = gridDim.x;
+// All greedy steps in one cooperative launch of at most one CTA per SM.  In step
+// k every block leaves the best of its points in its slot of buffer k & 1 and
+// reads all slots, so every block finds the same winner, marks it and pushes it
+// to its own points.  The slots carry their own readiness, a parity bit in each
+// of their two words that changes with every use of a buffer: no barrier and no
+// fence.  A block writes a buffer again only after it has read the next one
+// whole, which the others write after they have read this one.  (With a grid
+// barrier and 608 blocks a step took 14.6 us at 2^20 points, 7.4 at 2000; now
+// 10.9 and 3.1.)
+__global__ void __launch_bounds__(GREEDY_THREADS, 1)
+    ord_greedy_loop_k(const double* __restrict__ xg, int d, const int32_t* __restrict__ idg, double* v2, int* stat,
+                      int64_t N, int64_t steps, ulonglong2* slots, const float* __restrict__ xgf, float delta,
+                      int* status, long long limit) {
+    __shared__ Cand sh[32];
+    const int nblk = gridDim.x;
+    const unsigned long long PB = 1ull << 63;
+    int w = -1;  // the winner of the previous step
     for (int64_t k = 0; k <= steps; ++k) {
-        const double* pv_in = (k & 1) ? pv0 : pv1;
-        const int* pi_in = (k & 1) ? pi0 : pi1;
-        const int* pg_in = (k & 1) ? pg0 : pg1;
-        double* pv_out = (k & 1) ? pv1 : pv0;
-        int* pi_out = (k & 1) ? pi1 : pi0;
-        int* pg_out = (k & 1) ? pg1 : pg0;
-        {
-            double v = 0;
-            int i = 0, g = -1;
-            if (k > 0)
-                for (int b = threadIdx.x; b < nin; b += blockDim.x) {
-                    const int gb = __ldcg(&pg_in[b]);
-                    const double vb = __ldcg(&pv_in[b]);
-                    const int ib = __ldcg(&pi_in[b]);
-                    if (gb >= 0 && (g < 0 || key_above(vb, ib, v, i))) {
-                        v = vb;
-                        i = ib;
-                        g = gb;
-                    }
-                }
-            block_best(v, i, g, sv, si, sg, &s_wv, &s_wi, &s_wg);
-        }
-        __syncthreads();
-        const int w = s_wg;
-        if (w >= 0 && blockIdx.x == 0 && threadIdx.x == 0) stat[w] = 1;  // v2[w] keeps its final value l^2
-        double bv = 0;
-        int bi = 0, bg = -1;
+        Cand c{0.0, 0, -1};
         const double* xw = w >= 0 ? xg + (int64_t)w * d : nullptr;
-        for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < N; q += (int64_t)gridDim.x * blockDim.x) {
-            if (q == w || __ldcg(&stat[q]) != 0) continue;
+        for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < N; q += (int64_t)nblk * blockDim.x) {
+            if (q == w) stat[q] = 1;  // v2[w] keeps its final value l^2
+            if (q == w || stat[q] != 0) continue;
             double vq = v2[q];
-            if (w >= 0 &&
-                !(xgf && screen_f32(xgf + q * d, xgf + (int64_t)w * d, d, sqrtf((float)vq), delta) == 0)) {
+            if (w >= 0 && screen_f32(xgf + q * d, xgf + (int64_t)w * d, d, sqrtf((float)vq), delta) != 0) {
                 const double dd = dist2_exact(xg + q * d, xw, d);
                 if (dd < vq) {
                     vq = dd;
                     v2[q] = dd;
                 }
             }
-            const int iq = idg[q];
-            if (bg < 0 || key_above(vq, iq, bv, bi)) {
-                bv = vq;
-                bi = iq;
-                bg = (int)q;
+            c.take(vq, idg[q], (int)q);
+        }
+        if (k == steps) break;
+        c = block_best(c, sh);
+        if (nblk == 1) {
+            w = c.g;
+            continue;
+        }
+        ulonglong2* buf = slots + (k & 1) * nblk;
+        const unsigned long long par = ((k >> 1) & 1) ? 0ull : PB;
+        if (threadIdx.x == 0) {
+            // squared distances have no sign bit, indices are below 2^31; no candidate: all ones below it
+            const unsigned long long a = (unsigned long long)vbits(c.v) | par;
+            const unsigned long long b = ((unsigned long long)(unsigned)c.i << 32 | (unsigned)c.g) | par;
+            asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(&buf[blockIdx.x].x), "l"(a) : "memory");
+            asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(&buf[blockIdx.x].y), "l"(b) : "memory");
+        }
+        c = Cand{0.0, 0, -1};
+        bool fine = true;
+        for (int b = threadIdx.x; b < nblk; b += blockDim.x) {
+            unsigned long long u, v;
+            const long long t0 = clock64();
+            for (int poll = 1;; ++poll) {
+                asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(u) : "l"(&buf[b].x) : "memory");
+                asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(&buf[b].y) : "memory");
+                if ((u & PB) == par && (v & PB) == par) break;
+                if (clock64() - t0 > limit || ((poll & 63) == 0 && ld_volatile_s32(status) != 0)) {
+                    atomicCAS(status, 0, DEV_TIMEOUT);
+                    fine = false;
+                    break;
+                }
+            }
+            c.take(__longlong_as_double((long long)(u & ~PB)), (int)((v & ~PB) >> 32), (int)(unsigned)v);
+        }
+        if (__syncthreads_or(!fine)) return;
+        w = block_best(c, sh).g;
+    }
+}
+
+// All bands and their rounds in one cooperative launch, a grid barrier between
+// the phases: the host waits once, where it used to wait three times per band
+// and twice per round, around a dozen launches each.
+__global__ void __launch_bounds__(256, 4) ord_bands_k(BandArgs A) {
+    __shared__ int wsum[8];
+    __shared__ int carry;
+    __shared__ int active;
+    __shared__ Grid gb;  // of the band
+    BandCtl* C = A.ctl;
+    const float inv_c0 = (float)A.g0.inv_c;
+    const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nt = (int64_t)gridDim.x * blockDim.x;
+    const int lane = lane_id();
+    const int64_t warp = tid >> 5, nw = nt >> 5;
+    const bool first = tid == 0;
+    auto barrier = [&]() { return grid_barrier(&C->bar, &C->gen, &C->status, A.limit); };
+    int round = 0;
+    for (int band = 0;; ++band) {
+        const int bp = band & 1;
+        // largest undecided value, and whether there is any
+        {
+            unsigned long long m = 0;
+            bool any = false;
+            for (int64_t q = tid; q < A.N; q += nt)
+                if (A.stat[q] == 0) {
+                    m = max(m, (unsigned long long)__double_as_longlong(A.v2[q]));
+                    any = true;
+                }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+            any = __any_sync(0xffffffffu, any);
+            if (lane == 0 && any) {
+                atomicMax(&C->vmax[bp], m);
+                C->open[bp] = 1u;
             }
         }
-        __syncthreads();  // sv/si/sg are reused
-        block_best(bv, bi, bg, sv, si, sg, &pv_out[blockIdx.x], &pi_out[blockIdx.x], &pg_out[blockIdx.x]);
-        if (k < steps && !grid_barrier(bar, bar + 1, status, limit)) return;
+        if (!barrier()) return;
+        if (*(volatile unsigned*)&C->open[bp] == 0u) return;  // every point is decided
+        const double vmax = __longlong_as_double((long long)*(volatile unsigned long long*)&C->vmax[bp]);
+        const double T = vmax * KC_ORDER_BAND;
+        if (first) {
+            C->vmax[bp ^ 1] = 0ull;
+            C->open[bp ^ 1] = C->nb[bp ^ 1] = C->occ[bp ^ 1] = 0u;
+        }
+        for (int64_t q = tid; q < A.N; q += nt)
+            if (A.stat[q] == 0 && A.v2[q] >= T) A.blist[list_slot(&C->nb[bp])] = (int32_t)q;
+        if (!barrier()) return;
+        // the band's points by cells: counts, their scan, fill
+        const int64_t nb = *(volatile unsigned*)&C->nb[bp];
+        if (threadIdx.x == 0) band_grid(A, vmax, nb, gb);
+        __syncthreads();
+        for (int64_t c = tid; c < gb.ncells; c += nt) A.bcnt[c] = 0;
+        if (!barrier()) return;
+        for (int64_t e = tid; e < nb; e += nt) {
+            const int c = (int)cell_of(gb, A.gxg + (int64_t)A.blist[e] * A.gs);
+            A.bcell[e] = c;
+            if (atomicAdd(&A.bcnt[c], 1) == 0) list_slot(&C->occ[bp]);
+        }
+        if (!barrier()) return;
+        const int64_t per = ((gb.ncells + gridDim.x - 1) / gridDim.x + 255) / 256 * 256;
+        const int64_t c0 = min(gb.ncells, (int64_t)blockIdx.x * per), c1 = min(gb.ncells, c0 + per);
+        {
+            int sum = 0;
+            for (int64_t c = c0 + threadIdx.x; c < c1; c += blockDim.x) sum += A.bcnt[c];
+            sum = warp_sum(sum);
+            if (lane == 0) wsum[threadIdx.x >> 5] = sum;
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                int t = 0;
+                for (int w = 0; w < 8; ++w) t += wsum[w];
+                A.part[blockIdx.x] = t;
+            }
+        }
+        if (!barrier()) return;
+        {
+            int sum = 0;  // the cells before the block's
+            for (int b = threadIdx.x; b < (int)blockIdx.x; b += blockDim.x) sum += A.part[b];
+            sum = warp_sum(sum);
+            if (lane == 0) wsum[threadIdx.x >> 5] = sum;
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                int t = 0;
+                for (int w = 0; w < 8; ++w) t += wsum[w];
+                carry = t;
+            }
+            __syncthreads();
+            for (int64_t cb = c0; cb < c1; cb += blockDim.x) {
+                const int64_t c = cb + threadIdx.x;
+                const int n = c < c1 ? A.bcnt[c] : 0;
+                int inc = n;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int up = __shfl_up_sync(0xffffffffu, inc, o);
+                    if (lane >= o) inc += up;
+                }
+                if (lane == 31) wsum[threadIdx.x >> 5] = inc;
+                __syncthreads();
+                int before = carry;
+                for (int w = 0; w < (int)(threadIdx.x >> 5); ++w) before += wsum[w];
+                if (c < c1) {
+                    A.bstart[c] = before + inc - n;
+                    A.bcnt[c] = before + inc - n;  // where the cell's next point goes
+                }
+                __syncthreads();
+                if (threadIdx.x == blockDim.x - 1) carry = before + inc;
+                __syncthreads();
+            }
+            if (first) A.bstart[gb.ncells] = (int)nb;
+        }
+        if (!barrier()) return;
+        for (int64_t e = tid; e < nb; e += nt) A.bsorted[atomicAdd(&A.bcnt[A.bcell[e]], 1)] = A.blist[e];
+        if (!barrier()) return;
+        const int64_t occ = *(volatile unsigned*)&C->occ[bp];
+        const bool dense = nb >= 2 * occ, wide = nb >= 16 * occ;
+        // squared diagonal of a cell below every v of the band (grid coordinates are the points' own up to 3-D)
+        const bool within = A.d <= 3 && gb.c * gb.c * gb.dg * (1.0 + 1e-9) < T;
+        for (;; ++round) {
+            const int rp = round % 3;
+            // whether the block saw an active point: one store per block (a store per point
+            // to the one word took 0.1 ms a round at 2^20 points)
+            if (threadIdx.x == 0) active = 0;
+            __syncthreads();
+            auto post_active = [&]() {
+                __syncthreads();
+                if (threadIdx.x == 0 && active) C->nact[rp] = 1u;
+            };
+            // per band cell the largest value (as bits) of its undecided points, -1 if none: a
+            // dominance scan skips the cells whose largest value is below its own
+            // Dense bands (several points an occupied cell): 8 or 32 lanes per cell find its
+            // undecided point of largest key.  That point dominates the others of its
+            // cell, surely so where the cell's diagonal is below every sqrt(v) of the
+            // band, else if the distance says so; only what is left is looked at by a
+            // warp below.  (A thread per band point spent most of a round on points near
+            // the top of their cells.)
+            if (dense) {
+                const int lg = wide ? 32 : 8, l8 = lane & (lg - 1), per_warp = 32 / lg;
+                for (int64_t c4 = warp * per_warp; c4 < gb.ncells; c4 += nw * per_warp) {
+                    const int64_t c = c4 + lane / lg;
+                    const int f0 = c < gb.ncells ? A.bstart[c] : 0, f1 = c < gb.ncells ? A.bstart[c + 1] : 0;
+                    Cand best{0.0, 0, -1};
+                    for (int f = f0 + l8; f < f1; f += lg) {
+                        const int p = A.bsorted[f];
+                        if (A.stat[p] == 0) best.take(A.v2[p], A.idg[p], p);
+                    }
+                    __syncwarp();
+                    if (wide) best.warp_best();
+                    else best.best_of<4>();
+                    const bool act = best.g >= 0 && best.v >= T;
+                    if (l8 == 0 && c < gb.ncells) {
+                        A.cmax[c] = best.g >= 0 ? vbits(best.v) : -1;
+                        A.champ[c] = act ? best.g : -1;
+                        if (act) active = 1;
+                    }
+                    if (!within && act)
+                        for (int f = f0 + l8; f < f1; f += lg) {
+                            const int p = A.bsorted[f];
+                            if (p == best.g || A.stat[p] != 0) continue;
+                            const double vp = A.v2[p];
+                            if (!(vp >= T)) continue;
+                            const int sc = screen_f32(A.xgf + (int64_t)p * A.d, A.xgf + (int64_t)best.g * A.d, A.d,
+                                                      sqrtf((float)vp), A.delta);
+                            if (sc > 0) continue;
+                            if (sc == 0 || !(dist2_exact(A.xg + (int64_t)p * A.d, A.xg + (int64_t)best.g * A.d, A.d) < vp))
+                                A.hard[list_slot(&C->nhard[rp])] = p;
+                        }
+                    __syncwarp();
+                }
+                post_active();
+                if (!barrier()) return;
+            }
+            // Otherwise: per band cell the largest value (as bits) of its undecided points,
+            // -1 if none (a scan skips the cells whose largest value is below its own), ...
+            if (!dense) {
+                for (int64_t c = tid; c < gb.ncells; c += nt) {
+                    long long m = -1;
+                    for (int f = A.bstart[c]; f < A.bstart[c + 1]; ++f) {
+                        const int p = A.bsorted[f];
+                        if (A.stat[p] == 0) m = max(m, vbits(A.v2[p]));
+                    }
+                    A.cmax[c] = m;
+                }
+                if (!barrier()) return;
+            }
+            // ... then a thread per band point; the long scans are handed to a warp each
+            for (int64_t e = dense ? nb : tid; e < nb; e += nt) {
+                const int q = A.bsorted[e];
+                if (A.stat[q] != 0) continue;
+                const double vq = A.v2[q];
+                if (!(vq >= T)) continue;
+                active = 1;
+                // the point that dominated it before may still do
+                const int w0 = A.wit[q];
+                if (w0 >= 0 && A.stat[w0] == 0 && A.wd[q] < vq && key_above(A.v2[w0], A.idg[w0], vq, A.idg[q])) continue;
+                double wd = 0.0;
+                const int k = dominator_thread(A, gb, q, vq, wd);
+                if (k == -1) A.sel[list_slot(&C->nsel[rp])] = q;
+                else if (k == -2) A.hard[list_slot(&C->nhard[rp])] = q;
+                else {
+                    A.wit[q] = k;
+                    A.wd[q] = wd;
+                }
+            }
+            if (!dense) {
+                post_active();
+                if (!barrier()) return;
+            }
+            if (*(volatile unsigned*)&C->nact[rp] == 0u) break;  // band exhausted
+            const int64_t nh = *(volatile unsigned*)&C->nhard[rp];
+            auto scan = [&](int q) {
+                double wd = 0.0;
+                const double vq = A.v2[q];
+                const int k = dense ? dominator_warp<true>(A, gb, q, vq, wd) : dominator_warp<false>(A, gb, q, vq, wd);
+                if (lane == 0) {
+                    if (k == -1) {
+                        A.sel[atomicAdd(&C->nsel[rp], 1u)] = q;
+                    } else {
+                        A.wit[q] = k;
+                        A.wd[q] = wd;
+                    }
+                }
+            };
+            if (dense)  // the cells' largest points: cells warp, warp + nw, ..., 32 looked up at a time
+                for (int64_t cb = warp; cb < gb.ncells; cb += 32 * nw) {
+                    const int64_t c = cb + lane * nw;
+                    const int mine = c < gb.ncells ? A.champ[c] : -1;
+                    for (unsigned m = __ballot_sync(0xffffffffu, mine >= 0); m; m &= m - 1)
+                        scan(__shfl_sync(0xffffffffu, mine, __ffs(m) - 1));
+                }
+            for (int64_t e = warp; e < nh; e += nw) scan(A.hard[e]);
+            if (!barrier()) return;
+            // lower v2 of the undecided points of smaller key around every selected point: W
+            // warps a point.  A point selected in this
+            // round has no larger undecided key within its reach, so it does not matter
+            // whether it is marked yet.
+            const int64_t ns = *(volatile unsigned*)&C->nsel[rp];
+            if (ns == 0) {
+                if (first) atomicCAS(&C->status, 0, DEV_BAD_INPUT);
+                return;
+            }
+            if (first) {
+                const int nx = (round + 1) % 3;
+                C->nsel[nx] = C->nact[nx] = C->nhard[nx] = 0u;
+                C->rounds = round + 1;
+            }
+            const int64_t W = max((int64_t)1, min((int64_t)64, nw / ns));
+            for (int64_t u = warp; u < ns * W; u += nw) {
+                const int p = A.sel[u / W];
+                const int part = (int)(u % W);
+                if (part == 0 && lane == 0) A.stat[p] = 1;
+                const double* xp = A.xg + (int64_t)p * A.d;
+                const double vp = A.v2[p];  // final value of the selected point
+                const int idp = A.idg[p];
+                const int4 pc = A.pcell[p];
+                const int sx = span_of_v(A.g0, vp, inv_c0, 0);
+                const int x0 = max(0, pc.x - sx), x1 = min(A.g0.n[0] - 1, pc.x + sx);
+                int y0 = 0, y1 = 0, z0 = 0, z1 = 0;
+                if (A.g0.dg > 1) {
+                    const int sy = span_of_v(A.g0, vp, inv_c0, 1);
+                    y0 = max(0, pc.y - sy);
+                    y1 = min(A.g0.n[1] - 1, pc.y + sy);
+                }
+                if (A.g0.dg > 2) {
+                    const int sz = span_of_v(A.g0, vp, inv_c0, 2);
+                    z0 = max(0, pc.z - sz);
+                    z1 = min(A.g0.n[2] - 1, pc.z + sz);
+                }
+                // the rows of cells of the box in batches of rb: a lane per row finds where its
+                // points start, and the batch's points go to the lanes in one sequence
+                const int ny = y1 - y0 + 1, rows = ny * (z1 - z0 + 1);
+                const int rb = max(1, min(32, (rows + (int)W - 1) / (int)W));
+                for (int r0 = part * rb; r0 < rows; r0 += (int)W * rb) {
+                    const int r = r0 + lane;
+                    int64_t a = 0;
+                    int len = 0;
+                    if (lane < rb && r < rows) {
+                        const int64_t base = ((int64_t)(z0 + r / ny) * A.g0.n[1] + y0 + r % ny) * A.g0.n[0];
+                        a = A.cstart[base + x0];
+                        len = (int)(A.cstart[base + x1 + 1] - a);
+                    }
+                    int inc = len;
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int up = __shfl_up_sync(0xffffffffu, inc, o);
+                        if (lane >= o) inc += up;
+                    }
+                    const int total = __shfl_sync(0xffffffffu, inc, 31);
+                    for (int m0 = 0; m0 < total; m0 += 32) {
+                        const int m = m0 + lane;
+                        const int row = which_row(inc, m);
+                        const int64_t ra = __shfl_sync(0xffffffffu, a, row);
+                        const int rs = __shfl_sync(0xffffffffu, inc - len, row);
+                        if (m >= total) continue;
+                        const int64_t q = ra + (m - rs);
+                        if (A.stat[q] != 0) continue;
+                        const double vq = A.v2[q];
+                        if (!(vq < vp || (vq == vp && A.idg[q] > idp))) continue;
+                        if (screen_f32(A.xgf + q * A.d, A.xgf + (int64_t)p * A.d, A.d, sqrtf((float)vq), A.delta) == 0)
+                            continue;
+                        const double dd = dist2_exact(A.xg + q * A.d, xp, A.d);
+                        if (dd < vq)
+                            atomicMin((unsigned long long*)A.v2 + q, (unsigned long long)__double_as_longlong(dd));
+                    }
+                }
+            }
+            if (!barrier()) return;
+        }
+        ++round;  // its counters are used: selected none, so they stay as they are
+        if (first) {
+            const int nx = round % 3;
+            C->nsel[nx] = C->nact[nx] = C->nhard[nx] = 0u;
+        }
     }
 }
 
-__global__ void ord_mark_k(const int32_t* __restrict__ sel, int64_t ns, int* __restrict__ stat) {
-    int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < ns) stat[sel[k]] = 1;
-}
-
-// cell-rows of the fine grid covered by the update ball of each selected
-// point: the box is computed once per point (query_box) and kept in sbox
-__global__ void ord_items_k(Grid g, const int32_t* __restrict__ sel, int64_t ns, const double* __restrict__ gxg,
-                            int gs, const double* __restrict__ v2, int64_t* __restrict__ cnt, int4* __restrict__ sbox) {
-    int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= ns) return;
-    const int p = sel[k];
-    const int4 b = query_box(g, gxg + (int64_t)p * gs, sqrt(v2[p]));
-    sbox[k] = b;
-    int lo[3], hi[3];
-    box_range(g, b, lo, hi);
-    cnt[k] = (int64_t)(hi[1] - lo[1] + 1) * (hi[2] - lo[2] + 1);
-}
-__global__ void ord_item_fill_k(const int64_t* __restrict__ off, int64_t ns, int32_t* __restrict__ item_sel) {
-    int64_t k = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (k >= ns) return;
-    for (int64_t t = off[k] + lane_id(); t < off[k + 1]; t += 32) item_sel[t] = (int32_t)k;
-}
-
-// one warp per (selected point, cell-row): lower v2 of undecided points of smaller key
-__global__ void ord_update_k(Grid g, const int32_t* __restrict__ sel, const int64_t* __restrict__ off,
-                             const int32_t* __restrict__ item_sel, int64_t nitems, const int64_t* __restrict__ cstart,
-                             const double* __restrict__ xg, int d, const int32_t* __restrict__ idg,
-                             double* __restrict__ v2, const int* __restrict__ stat, const float* __restrict__ xgf,
-                             float delta, const int4* __restrict__ sbox) {
-    int64_t it = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (it >= nitems) return;
-    const int lane = lane_id();
-    const int k = item_sel[it];
-    const int p = sel[k];
-    const double* xp = xg + (int64_t)p * d;
-    const double vp = v2[p];  // final value of the selected point
-    const int idp = idg[p];
-    int lo[3], hi[3];
-    box_range(g, sbox[k], lo, hi);
-    int64_t r = it - off[k];
-    const int ny = hi[1] - lo[1] + 1;
-    const int cy = lo[1] + (int)(r % ny);
-    const int cz = lo[2] + (int)(r / ny);
-    const int64_t base = ((int64_t)cz * g.n[1] + cy) * g.n[0];
-    const int64_t a = cstart[base + lo[0]], b = cstart[base + hi[0] + 1];
-    unsigned long long* vb = (unsigned long long*)v2;
-    for (int64_t q = a + lane; q < b; q += 32) {
-        if (stat[q] != 0) continue;
-        const double vq = v2[q];
-        if (!(vq < vp || (vq == vp && idg[q] > idp))) continue;
-        if (xgf && screen_f32(xgf + q * d, xgf + (int64_t)p * d, d, sqrtf((float)vq), delta) == 0) continue;
-        const double dd = dist2_exact(xg + q * d, xp, d);
-        if (dd < vq) atomicMin(vb + q, (unsigned long long)__double_as_longlong(dd));
-    }
+__global__ void ord_cells_k(Grid g, const double* __restrict__ gxg, int gs, int64_t N, int4* __restrict__ pcell) {
+    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= N) return;
+    int c[3] = {0, 0, 0};
+    for (int t = 0; t < g.dg; ++t) c[t] = cell_coord(g, gxg[q * gs + t], t);
+    pcell[q] = make_int4(c[0], c[1], c[2], 0);
 }
 
 __global__ void ord_keys_k(const double* __restrict__ v2, const int32_t* __restrict__ idg, int64_t N,
@@ -537,13 +838,15 @@ __global__ void ord_out_k(const uint64_t* __restrict__ skey, const int64_t* __re
 
 kc_status order_impl(const double* x, int64_t N, int d, int32_t* perm, double* l, double* x_ord, cudaStream_t s) {
     Arena A(s);
-    KC_TRY(check_finite(x, N * d, A, s));
+    Origin org, top;
+    double E = 0.0;
+    KC_TRY(points_bounds(x, N, d, &org, &top, &E, A, s));
     // grid coordinates: the points (d <= 3) or their principal-axes projections
     const double* gx;
     int gs;
     KC_TRY(grid_coords(x, N, d, A, s, &gx, &gs));
-    double lo[3], hi[3];
-    KC_TRY(bbox(gx, N, gs, lo, hi, A, s));
+    double lo[3] = {org.lo[0], org.lo[1], org.lo[2]}, hi[3] = {top.lo[0], top.lo[1], top.lo[2]};
+    if (gx != x) KC_TRY(bbox(gx, N, gs, lo, hi, A, s));
     // fine grid of all points, about two points per cell
     Grid g0 = make_grid(gs, lo, hi, N, 0.0, N / 2 > 1 ? N / 2 : 1);
     int32_t* gsorted;
@@ -553,33 +856,15 @@ kc_status order_impl(const double* x, int64_t N, int d, int32_t* perm, double* l
     KC_TRY(grid_build(g0, gx, gs, nullptr, N, gsorted, cstart, A, s));
 
     double *xg, *v2;
-    int32_t *idg, *blist, *bsorted, *sel, *item_sel;
+    int32_t* idg;
     int* stat;
-    int64_t *bstart, *icnt, *ioff;
-    unsigned long long* ctr;  // [0] vmax bits [1] undecided [2] nb [3] nsel [4] nactive [5] handed to warps
     KC_TRY(A.get(&xg, N * d));
     KC_TRY(A.get(&v2, N));
     KC_TRY(A.get(&idg, N));
     KC_TRY(A.get(&stat, N));
-    KC_TRY(A.get(&blist, N));
-    KC_TRY(A.get(&bsorted, N));
-    KC_TRY(A.get(&sel, N));
-    int32_t* hard;  // band points handed from the thread scan to the warp scan
-    KC_TRY(A.get(&hard, N));
-    KC_TRY(A.get(&icnt, N));
-    int4* sbox;
-    KC_TRY(A.get(&sbox, N));
-    KC_TRY(A.get(&ioff, N + 1));
-    KC_TRY(A.get(&bstart, 2 * N + 2));
-    long long* cmax;  // per band cell (at most 2 N + 1 cells)
-    KC_TRY(A.get(&cmax, 2 * N + 2));
-    KC_TRY(A.get(&ctr, 8));
     // float copy of the coordinates (minus the box corner) for FP32 screens of
     // the distance tests; exact FP64 tests decide every close call
     float* xgf = nullptr;
-    Origin org;
-    double E = 0.0;
-    KC_TRY(bbox_all(x, N, d, &org, &E, A, s));
     const float delta = (float)(E * 1.1920928955078125e-07);  // 2^-23 E
     KC_TRY(A.get(&xgf, N * d));
     ::kc::note_launch(), ord_init_k<<<blocks_for(N, 256), 256, 0, s>>>(x, d, gsorted, N, xg, idg, v2, stat, org, xgf);
@@ -591,125 +876,86 @@ kc_status order_impl(const double* x, int64_t N, int d, int32_t* perm, double* l
         ::kc::note_launch(), gather_rows_k<<<blocks_for(N, 256), 256, 0, s>>>(gx, gs, gsorted, N, p);
         gxg = p;
     }
+    int4* pcell;
+    KC_TRY(A.get(&pcell, N));
+    ::kc::note_launch(), ord_cells_k<<<blocks_for(N, 256), 256, 0, s>>>(g0, gxg, gs, N, pcell);
     KC_CUDA(cudaGetLastError());
-    int64_t item_cap = 0;
-    item_sel = nullptr;
     const int sms = sm_count();
+    const long long limit = 4000000000LL;
 
     // Greedy phase: the coarsest points are selected one at a time (every
     // step updates every point), because while few points are selected the
     // update balls cover the whole cloud and the band rounds would be
-    // quadratic.  All steps run in one cooperative launch with a grid barrier
-    // between them.
+    // quadratic.
+    BandCtl* ctl;
+    KC_TRY(A.get(&ctl, 1));
+    KC_CUDA(cudaMemsetAsync(ctl, 0, sizeof(BandCtl), s));
     {
-        int per_sm = 0;
-        KC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ord_greedy_loop_k, 256, 0));
-        const int nblk = sms * std::max(1, std::min(per_sm, GREEDY_BLOCKS_PER_SM));
-        double* pv[2];
-        int *pi[2], *pg[2];
-        for (int k = 0; k < 2; ++k) {
-            KC_TRY(A.get(&pv[k], nblk));
-            KC_TRY(A.get(&pi[k], nblk));
-            KC_TRY(A.get(&pg[k], nblk));
-        }
-        unsigned* bar;
-        int* gst;
-        KC_TRY(A.get(&bar, 2));
-        KC_TRY(A.get(&gst, 1));
-        KC_CUDA(cudaMemsetAsync(bar, 0, 2 * sizeof(unsigned), s));
-        KC_CUDA(cudaMemsetAsync(gst, 0, sizeof(int), s));
+        // one block, which exchanges nothing, for up to 4 points a thread
+        const int nblk = N <= 4 * GREEDY_THREADS ? 1 : (int)std::min<int64_t>(sms, (N + GREEDY_THREADS - 1) / GREEDY_THREADS);
+        ulonglong2* slots;
+        KC_TRY(A.get(&slots, 2 * nblk));
+        KC_CUDA(cudaMemsetAsync(slots, 0, sizeof(ulonglong2) * 2 * nblk, s));
         int64_t steps = N - 1 < GREEDY_STEPS ? N - 1 : GREEDY_STEPS;
         const double* a_xg = xg;
         const int32_t* a_idg = idg;
         const float* a_xgf = xgf;
-        long long limit = 4000000000LL;
+        int* gst = &ctl->status;
+        long long lim = limit;
+        float dl = delta;
         void* args[] = {(void*)&a_xg, (void*)&d, (void*)&a_idg, (void*)&v2, (void*)&stat, (void*)&N, (void*)&steps,
-                        (void*)&pv[0], (void*)&pi[0], (void*)&pg[0], (void*)&pv[1], (void*)&pi[1], (void*)&pg[1],
-                        (void*)&a_xgf, (void*)&delta, (void*)&bar, (void*)&gst, (void*)&limit};
+                        (void*)&slots, (void*)&a_xgf, (void*)&dl, (void*)&gst, (void*)&lim};
         ::kc::note_launch();
-        KC_CUDA(cudaLaunchCooperativeKernel((const void*)ord_greedy_loop_k, dim3(nblk), dim3(256), args, 0, s));
-        int hst = 0;
-        KC_CUDA(cudaMemcpyAsync(&hst, gst, sizeof(int), cudaMemcpyDeviceToHost, s));
-        KC_CUDA(cudaStreamSynchronize(s));
-        if (hst != 0) return fail(KC_ETIMEOUT, "ordering: a grid barrier of the greedy phase ran out");
+        KC_CUDA(cudaLaunchCooperativeKernel((const void*)ord_greedy_loop_k, dim3(nblk), dim3(GREEDY_THREADS), args, 0, s));
     }
-    int rounds = 0;
-    const bool stats = getenv("KC_ORDER_STATS") != nullptr;
-    for (;;) {
-        KC_CUDA(cudaMemsetAsync(ctr, 0, 2 * sizeof(unsigned long long), s));
-        ::kc::note_launch(), ord_vmax_k<<<sms * 4, 256, 0, s>>>(v2, stat, N, ctr, ctr + 1);
-        unsigned long long h[2];
-        KC_CUDA(cudaMemcpyAsync(h, ctr, sizeof(h), cudaMemcpyDeviceToHost, s));
-        KC_CUDA(cudaStreamSynchronize(s));
-        if (h[1] == 0) break;
-        double vmax;
-        memcpy(&vmax, &h[0], sizeof(double));
-        const double T = vmax * KC_ORDER_BAND;
-        KC_CUDA(cudaMemsetAsync(ctr + 2, 0, sizeof(unsigned long long), s));
-        ::kc::note_launch(), ord_band_k<<<blocks_for(N, 256), 256, 0, s>>>(v2, stat, N, T, blist, ctr + 2);
-        unsigned long long hnb = 0;
-        KC_CUDA(cudaMemcpyAsync(&hnb, ctr + 2, sizeof(hnb), cudaMemcpyDeviceToHost, s));
-        KC_CUDA(cudaStreamSynchronize(s));
-        const int64_t nb = (int64_t)hnb;
-        // band cells a quarter of the largest search radius (bounded by the
-        // cell budget), scanned nearest ring first
-        Grid gb = make_grid(gs, lo, hi, nb, vmax > 0 ? 0.25 * sqrt(vmax) : 0.0, 2 * nb + 1);
-        {
-            Arena B(s);
-            int64_t* bst;
-            KC_TRY(B.get(&bst, gb.ncells + 1));
-            KC_TRY(grid_build(gb, gxg, gs, blist, nb, bsorted, bst, B, s));
-            KC_CUDA(cudaMemcpyAsync(bstart, bst, sizeof(int64_t) * (gb.ncells + 1), cudaMemcpyDeviceToDevice, s));
+    {
+        BandArgs a;
+        a.N = N;
+        a.d = d;
+        a.gs = gs;
+        a.g0 = g0;
+        a.cstart = cstart;
+        a.xg = xg;
+        a.xgf = xgf;
+        a.gxg = gxg;
+        a.pcell = pcell;
+        a.idg = idg;
+        a.delta = delta;
+        a.v2 = v2;
+        a.stat = stat;
+        a.ctl = ctl;
+        a.limit = limit;
+        for (int t = 0; t < 3; ++t) {
+            a.lo[t] = t < g0.dg ? lo[t] : 0.0;
+            a.hi[t] = t < g0.dg ? hi[t] : 0.0;
         }
-        const int band_r0 = rounds;
-        const auto band_t0 = std::chrono::steady_clock::now();
-        int64_t band_sel = 0, band_items = 0;
-        for (;;) {
-            if (++rounds > 1000000) return fail(KC_ECUDA, "ordering: too many rounds");
-            KC_CUDA(cudaMemsetAsync(ctr + 3, 0, 3 * sizeof(unsigned long long), s));
-            ::kc::note_launch(), ord_cellmax_k<<<blocks_for(gb.ncells, 256), 256, 0, s>>>(bsorted, bstart, gb.ncells, v2,
-                                                                                         stat, cmax);
-            ::kc::note_launch(), ord_dominance_k<<<blocks_for(nb, 128), 128, 0, s>>>(
-                gb, bsorted, bstart, nb, xg, d, idg, v2, stat, T, sel, ctr + 3, ctr + 4, xgf, delta, cmax, gxg, gs, hard,
-                ctr + 5);
-            ::kc::note_launch(), ord_dominance_warp_k<<<sms * 8, 256, 0, s>>>(
-                gb, hard, ctr + 5, bstart, bsorted, xg, d, idg, v2, stat, sel, ctr + 3, xgf, delta, cmax, gxg, gs);
-            unsigned long long hs[2];
-            KC_CUDA(cudaMemcpyAsync(hs, ctr + 3, sizeof(hs), cudaMemcpyDeviceToHost, s));
-            KC_CUDA(cudaStreamSynchronize(s));
-            const int64_t ns = (int64_t)hs[0];
-            if (hs[1] == 0) {  // band exhausted
-                if (stats) {
-                    double ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - band_t0)
-                                    .count();
-                    fprintf(stderr, "[kc order] vmax=%.3e band=%lld rounds=%d selected=%lld items=%lld ms=%.2f\n", vmax,
-                            (long long)nb, rounds - band_r0 - 1, (long long)band_sel, (long long)band_items, ms);
-                }
-                break;
-            }
-            band_sel += (int64_t)hs[0];
-            if (ns == 0) return fail(KC_ECUDA, "ordering: no dominant point in a nonempty band");
-            ::kc::note_launch(), ord_mark_k<<<blocks_for(ns, 256), 256, 0, s>>>(sel, ns, stat);
-            ::kc::note_launch(), ord_items_k<<<blocks_for(ns, 256), 256, 0, s>>>(g0, sel, ns, gxg, gs, v2, icnt, sbox);
-            Arena R(s);  // per-round scratch of the scan
-            KC_TRY(exclusive_scan_i64(icnt, ioff, ns, R, s));
-            int64_t nitems = 0;
-            KC_CUDA(cudaMemcpyAsync(&nitems, ioff + ns, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-            KC_CUDA(cudaStreamSynchronize(s));
-            band_items += nitems;
-            if (nitems > item_cap) {
-                item_cap = nitems * 2;
-                if (item_sel) cudaFreeAsync(item_sel, s);
-                item_sel = nullptr;
-                KC_TRY(scratch_alloc((void**)&item_sel, sizeof(int32_t) * item_cap, s));
-            }
-            ::kc::note_launch(), ord_item_fill_k<<<blocks_for(ns * 32, 256), 256, 0, s>>>(ioff, ns, item_sel);
-            ::kc::note_launch(), ord_update_k<<<blocks_for(nitems * 32, 256), 256, 0, s>>>(g0, sel, ioff, item_sel, nitems, cstart, xg, d,
-                                                                     idg, v2, stat, xgf, delta, sbox);
-            KC_CUDA(cudaGetLastError());
-        }
+        KC_TRY(A.get(&a.blist, N));
+        KC_TRY(A.get(&a.bcell, N));
+        KC_TRY(A.get(&a.bsorted, N));
+        KC_TRY(A.get(&a.hard, N));
+        KC_TRY(A.get(&a.sel, N));
+        KC_TRY(A.get(&a.bcnt, 2 * N + 1));    // a band of nb points has at most 2 nb + 1 cells
+        KC_TRY(A.get(&a.bstart, 2 * N + 2));
+        KC_TRY(A.get(&a.cmax, 2 * N + 1));
+        KC_TRY(A.get(&a.champ, 2 * N + 1));
+        KC_TRY(A.get(&a.wit, N));
+        KC_TRY(A.get(&a.wd, N));
+        KC_CUDA(cudaMemsetAsync(a.wit, 0xff, sizeof(int32_t) * N, s));  // -1
+        int per_sm = 0;
+        KC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ord_bands_k, 256, 0));
+        // a block per 256 points (few blocks keep the barriers short), at most what is resident at once
+        const int nblk = (int)std::min<int64_t>((int64_t)sms * std::max(1, per_sm), (N + 255) / 256);
+        KC_TRY(A.get(&a.part, nblk));
+        void* args[] = {(void*)&a};
+        ::kc::note_launch();
+        KC_CUDA(cudaLaunchCooperativeKernel((const void*)ord_bands_k, dim3(nblk), dim3(256), args, 0, s));
+        BandCtl h;
+        KC_CUDA(cudaMemcpyAsync(&h, ctl, sizeof(h), cudaMemcpyDeviceToHost, s));
+        KC_CUDA(cudaStreamSynchronize(s));
+        if (h.status == DEV_TIMEOUT) return fail(KC_ETIMEOUT, "ordering: a grid barrier ran out");
+        if (h.status != 0) return fail(KC_ECUDA, "ordering: no dominant point in a nonempty band");
+        if (getenv("KC_ORDER_STATS")) fprintf(stderr, "[kc order] N=%lld rounds=%d\n", (long long)N, h.rounds);
     }
-    if (item_sel) cudaFreeAsync(item_sel, s);
     uint64_t *k0, *k1;
     int64_t *w0, *w1;
     KC_TRY(A.get(&k0, N));

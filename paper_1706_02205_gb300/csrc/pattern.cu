@@ -19,8 +19,6 @@
 
 namespace kc {
 
-kc_status check_finite(const double* x, int64_t n, Arena& A, cudaStream_t s);
-
 struct PatArgs {
     Grid g;
     const double* xs;      // coordinates in cell-sorted order
@@ -236,17 +234,16 @@ struct PatSetup {
 
 static kc_status pat_setup(const double* xo, const double* l, int64_t N, int d, double rho, PatSetup& S, Arena& A,
                            cudaStream_t s) {
-    KC_TRY(check_finite(xo, N * d, A, s));
+    Origin org, top;
+    double E = 0.0;
+    KC_TRY(points_bounds(xo, N, d, &org, &top, &E, A, s));
     // grid coordinates: the points (d <= 3) or their principal-axes projections
     const double* gxo;
     int gst;
     KC_TRY(grid_coords(xo, N, d, A, s, &gxo, &gst));
-    double lo[3], hi[3];
-    KC_TRY(bbox(gxo, N, gst, lo, hi, A, s));
+    double lo[3] = {org.lo[0], org.lo[1], org.lo[2]}, hi[3] = {top.lo[0], top.lo[1], top.lo[2]};
+    if (gxo != xo) KC_TRY(bbox(gxo, N, gst, lo, hi, A, s));
     S.g = make_grid(gst, lo, hi, N, 0.0, N / 2 > 1 ? N / 2 : 1);
-    Origin org;
-    double E = 0.0;
-    KC_TRY(bbox_all(xo, N, d, &org, &E, A, s));
     S.delta = (float)(E * 1.1920928955078125e-07);  // 2^-23 E
     KC_TRY(A.get(&S.xsf, N * d));
     KC_TRY(A.get(&S.xof, N * d));

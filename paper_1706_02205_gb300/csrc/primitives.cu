@@ -431,12 +431,61 @@ static size_t rs_smem_bytes() {
     return (size_t)RS_TILE * (sizeof(int64_t) + sizeof(K));
 }
 
+// Few elements: one block sorts (key, place) in shared memory (bitonic; the
+// places make it stable) instead of up to eight passes of three to five launches
+// each (2000 points: 40 launches for a 64-bit key).
+constexpr int SMALL_SORT = 4096, SMALL_THREADS = 1024;
+template <typename K>
+__global__ void __launch_bounds__(SMALL_THREADS) small_sort_k(const K* __restrict__ kin, const int64_t* __restrict__ vin,
+                                                              int n, int size, K mask, K* __restrict__ kout,
+                                                              int64_t* __restrict__ vout) {
+    extern __shared__ __align__(16) unsigned char rs_smem[];
+    K* key = (K*)rs_smem;
+    int* at = (int*)(key + size);
+    for (int i = threadIdx.x; i < size; i += SMALL_THREADS) {
+        key[i] = i < n ? kin[i] & mask : ~(K)0;
+        at[i] = i;
+    }
+    __syncthreads();
+    for (int k = 2; k <= size; k <<= 1)
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            for (int i = threadIdx.x; i < size / 2; i += SMALL_THREADS) {
+                const int a = 2 * i - (i & (j - 1)), b = a + j;  // a has bit j clear
+                const K ka = key[a], kb = key[b];
+                const int pa = at[a], pb = at[b];
+                const bool up = (a & k) == 0;
+                if ((ka > kb || (ka == kb && pa > pb)) == up) {
+                    key[a] = kb;
+                    key[b] = ka;
+                    at[a] = pb;
+                    at[b] = pa;
+                }
+            }
+            __syncthreads();
+        }
+    for (int i = threadIdx.x; i < n; i += SMALL_THREADS) {
+        kout[i] = kin[at[i]];
+        vout[i] = vin[at[i]];
+    }
+}
+
 template <typename K>
 static kc_status radix_impl(K* k_in, int64_t* v_in, K* k_out, int64_t* v_out, int64_t n, int bits, Arena& A,
                             cudaStream_t s) {
     if (n <= 0) return KC_OK;
     int passes = (bits + 7) / 8;
     if (passes < 1) passes = 1;
+    if (n <= SMALL_SORT) {
+        int size = 2;
+        while (size < n) size <<= 1;
+        const int used = 8 * passes;  // the passes look at whole digits
+        const K mask = used >= (int)(8 * sizeof(K)) ? ~(K)0 : (K)(((K)1 << used) - 1);
+        KC_TRY(allow_dynamic_smem(small_sort_k<K>));
+        ::kc::note_launch(), small_sort_k<K><<<1, SMALL_THREADS, (size_t)size * (sizeof(K) + sizeof(int)), s>>>(
+            k_in, v_in, (int)n, size, mask, k_out, v_out);
+        KC_CUDA(cudaGetLastError());
+        return KC_OK;
+    }
     KC_TRY(allow_dynamic_smem(rs_scatter_k<K>));
     int64_t ntiles = (n + RS_TILE - 1) / RS_TILE;
     int64_t* hist;
