@@ -389,7 +389,7 @@ def supernodal_leg(args, l, xo, pat0, kern):
 TRAFFIC_CAPTURE = {"sources": ("paper_1706_02205_gb300/csrc/factor.cu", "paper_1706_02205_gb300/csrc/common.cuh",
                                "paper_1706_02205_gb300/csrc/grid.cuh", "paper_1706_02205_gb300/csrc/covariance.cuh",
                                "paper_1706_02205_gb300/csrc/ichol.cuh"),
-                   "sha256": "397f406122c62d11937429fe71d13763dae76d28bf69e16afe548ec0d7b9a2ce",
+                   "sha256": "5c6ca620da909072c99ab964eed0538f310757cfce89986468f1c1c723f72731",
                    "dram_per_algorithmic_byte": (26.960658 + 0.946831) / 26.387813}
 
 

@@ -199,7 +199,7 @@ __global__ void __launch_bounds__(256) bounds_k(const double* __restrict__ x, in
 }
 
 kc_status points_bounds(const double* x, int64_t N, int d, Origin* lo, Origin* hi, double* E, Arena& A,
-                        cudaStream_t s) {
+                        cudaStream_t s, bool* finite) {
     if (d > MAXD) return fail(KC_EINVAL, "d must be <= 32");
     constexpr int W = 2 * MAXD + 1, MOST = 152;
     const int nb = (int)std::min<int64_t>(MOST, (N * d + 255) / 256);
@@ -213,8 +213,10 @@ kc_status points_bounds(const double* x, int64_t N, int d, Origin* lo, Origin* h
     KC_CUDA(cudaMemcpyAsync(h.data(), part, sizeof(unsigned long long) * h.size(), cudaMemcpyDeviceToHost, s));
     KC_CUDA(cudaStreamSynchronize(s));
     double e = 0.0;
-    for (int b = 0; b < nb; ++b)
-        if (h[(size_t)b * W + 2 * MAXD]) return fail(KC_EINVAL, "points must be finite");
+    bool ok = true;
+    for (int b = 0; b < nb; ++b) ok = ok && !h[(size_t)b * W + 2 * MAXD];
+    if (finite) *finite = ok;
+    else if (!ok) return fail(KC_EINVAL, "points must be finite");
     for (int t = 0; t < MAXD; ++t) lo->lo[t] = hi->lo[t] = 0.0;
     for (int t = 0; t < d; ++t) {
         unsigned long long mn = ~0ull, mx = 0ull;

@@ -123,11 +123,12 @@ kc_status grid_coords(const double* x, int64_t N, int d, Arena& A, cudaStream_t 
 
 // Bounding box over all d <= 32 axes (host out; the low corner also for the float
 // copies used by the FP32 distance screens); E = the largest extent.  KC_EINVAL if
-// a coordinate is not finite.  One pass and one wait of the host.
+// a coordinate is not finite, unless `finite` is given to say so.  One pass and one wait of the host.
 constexpr int MAXD = 32;
 struct Origin {
     double lo[MAXD];
 };
-kc_status points_bounds(const double* x, int64_t N, int d, Origin* lo, Origin* hi, double* E, Arena& A, cudaStream_t s);
+kc_status points_bounds(const double* x, int64_t N, int d, Origin* lo, Origin* hi, double* E, Arena& A, cudaStream_t s,
+                        bool* finite = nullptr);
 
 }  // namespace kc

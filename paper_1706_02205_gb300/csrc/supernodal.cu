@@ -24,7 +24,7 @@
 // index order).  Rounds are host-driven launches, so no kernel waits.
 #include <algorithm>
 
-#include "common.cuh"
+#include "grid.cuh"
 
 namespace kc {
 
@@ -35,6 +35,31 @@ constexpr int SN_MAX_ROUNDS = 1 << 20;
 enum : int8_t { SN_UNDEC = 0, SN_IN = 1, SN_OUT = 2 };
 
 __device__ __forceinline__ double sn_R(double rl1, int k) { return ldexp(rl1, -k); }
+
+// The test d(a, b) <= R_k over the pattern's entries, most of them far from the
+// radius: an FP32 screen on copies of the points minus their box's corner
+// decides those, and only what it cannot tell takes the FP64 distance and its
+// root.  The FP64 pipe bounds the exact test (two FMA a clock and SM): over the
+// 188.7 M entries of the 2^20 grid (rho = 3) a pass of sn_pairs_k took 7.2 ms
+// with it alone and 2.6 with the screen, one of sn_conflicts_k 1.53 and 1.07.
+struct SnPoints {
+    const double* x;
+    const float* xf;  // NULL: exact tests only
+    int d;
+    float delta;      // bound of the error of a coordinate difference of xf
+};
+__global__ void sn_float_k(const double* __restrict__ x, int64_t N, int d, Origin org, float* __restrict__ xf) {
+    const int64_t m = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (m < N)
+        for (int t = 0; t < d; ++t) xf[m * d + t] = (float)(x[m * d + t] - org.lo[t]);
+}
+__device__ __forceinline__ bool sn_within(const SnPoints& X, int64_t a, int64_t b, double R) {
+    if (X.xf) {
+        const int sc = screen_f32(X.xf + a * X.d, X.xf + b * X.d, X.d, (float)R, X.delta);
+        if (sc >= 0) return sc != 0;
+    }
+    return sqrt(dist2_exact(X.x + a * X.d, X.x + b * X.d, X.d)) <= R;
+}
 
 __global__ void sn_level_k(const double* __restrict__ l, int64_t N, int32_t* __restrict__ lev) {
     const int64_t m = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -54,7 +79,7 @@ __global__ void sn_level_k(const double* __restrict__ l, int64_t N, int32_t* __r
 // cnt_l[i] += 1 for each earlier conflict i); mode 1 fills list[off[m] ..]
 // with the earlier conflicts first, then, from the other side, the later
 // ones (their order within the list is immaterial).
-__global__ void sn_conflicts_k(const double* __restrict__ x, int d, const int64_t* __restrict__ rowptr,
+__global__ void sn_conflicts_k(SnPoints X, const int64_t* __restrict__ rowptr,
                                const int32_t* __restrict__ col, const int32_t* __restrict__ lev, int64_t N,
                                double rl1, int mode, int32_t* __restrict__ cnt_e, int32_t* __restrict__ cnt_l,
                                const int64_t* __restrict__ off, int32_t* __restrict__ fill_l,
@@ -64,7 +89,6 @@ __global__ void sn_conflicts_k(const double* __restrict__ x, int d, const int64_
     const int lane = lane_id();
     const int k = lev[m];
     const double R = sn_R(rl1, k);
-    const double* xm = x + m * d;
     int64_t w = mode ? off[m] : 0;
     int ne = 0;
     const int64_t a0 = rowptr[m], a1 = rowptr[m + 1] - 1;  // row m without its diagonal
@@ -74,7 +98,7 @@ __global__ void sn_conflicts_k(const double* __restrict__ x, int d, const int64_
         int32_t i = -1;
         if (e < a1) {
             i = col[e];
-            hit = lev[i] == k && sqrt(dist2_exact(xm, x + (int64_t)i * d, d)) <= R;
+            hit = lev[i] == k && sn_within(X, m, i, R);
         }
         const unsigned b = __ballot_sync(0xffffffffu, hit);
         if (hit) {
@@ -147,15 +171,16 @@ __global__ void sn_assign_k(const double* __restrict__ x, int d, const int64_t* 
 
 // supernode pairs: for each pattern entry (b, a), a < b, with dist <= R_k(a),
 // the unordered pair of their supernodes; plus (A, A) for every supernode.
-// mode 0 counts per row, mode 1 fills at off[b].
-__global__ void sn_pairs_k(const double* __restrict__ x, int d, const int64_t* __restrict__ rowptr,
+// mode 0 counts per row, mode 1 fills at off[b].  A pair that an earlier lane
+// of the same 32 entries names is left out (the sort's unique pass would drop
+// it; the radix sorts of the construction took 5.7 ms and take 3.1).
+__global__ void sn_pairs_k(SnPoints X, const int64_t* __restrict__ rowptr,
                            const int32_t* __restrict__ col, const int32_t* __restrict__ lev,
                            const int32_t* __restrict__ node, int64_t N, double rl1, int B, int mode,
                            int32_t* __restrict__ cnt, const int64_t* __restrict__ off, uint64_t* __restrict__ keys) {
     const int64_t b = (int64_t)blockIdx.x * SN_WARPS + (threadIdx.x >> 5);
     if (b >= N) return;
     const int lane = lane_id();
-    const double* xb = x + b * d;
     const uint32_t nb = (uint32_t)node[b];
     int64_t w = mode ? off[b] : 0;
     int n = 0;
@@ -164,12 +189,15 @@ __global__ void sn_pairs_k(const double* __restrict__ x, int d, const int64_t* _
         const int64_t e = e0 + lane;
         bool hit = false;
         uint64_t key = 0;
+        uint32_t na = 0;
         if (e < a1) {
             const int32_t a = col[e];
-            hit = sqrt(dist2_exact(xb, x + (int64_t)a * d, d)) <= sn_R(rl1, lev[a]);
-            const uint32_t na = (uint32_t)node[a];
+            hit = sn_within(X, b, a, sn_R(rl1, lev[a]));
+            na = (uint32_t)node[a];
             key = na < nb ? ((uint64_t)na << B | nb) : ((uint64_t)nb << B | na);
         }
+        const unsigned same = __match_any_sync(0xffffffffu, hit ? na : 0x80000000u | (uint32_t)lane);
+        hit = hit && lane == __ffs(same) - 1;
         const unsigned bal = __ballot_sync(0xffffffffu, hit);
         if (mode && hit) keys[w + __popc(bal & ((1u << lane) - 1))] = key;
         w += __popc(bal);
@@ -334,16 +362,35 @@ static kc_status sync_read(const void* dev, void* host, size_t bytes, cudaStream
     return KC_OK;
 }
 
+// The points and their float copies; exact tests only where the extent E leaves
+// float's normal range (or is not finite), so that neither the copies nor the
+// squares of their differences over- or underflow.
+static kc_status sn_points(const double* x, int64_t N, int d, SnPoints& X, Arena& A, cudaStream_t s) {
+    X = SnPoints{x, nullptr, d, 0.f};
+    if (d > MAXD) return KC_OK;
+    Origin lo, hi;
+    double E = 0.0;
+    bool finite = true;
+    KC_TRY(points_bounds(x, N, d, &lo, &hi, &E, A, s, &finite));
+    if (!finite || !(E > 1e-12 && E < 1e15)) return KC_OK;
+    float* xf;
+    KC_TRY(A.get(&xf, N * d));
+    note_launch(), sn_float_k<<<blocks_for(N, 256), 256, 0, s>>>(x, N, d, lo, xf);
+    KC_CUDA(cudaGetLastError());
+    X.xf = xf;
+    X.delta = (float)(E * 1.1920928955078125e-07);  // 2^-23 E
+    return KC_OK;
+}
+
 // the unique supernode pairs of the pattern
-static kc_status sn_pairs(const double* x, int d, const kc_pattern* P, double rl1, SnState& S, Arena& A,
-                          cudaStream_t s) {
+static kc_status sn_pairs(const SnPoints& X, const kc_pattern* P, double rl1, SnState& S, Arena& A, cudaStream_t s) {
     const int64_t N = P->N;
     int32_t* cnt;
     int64_t* off;
     KC_TRY(A.get(&cnt, N));
     KC_TRY(A.get(&off, N + 1));
-    note_launch(), sn_pairs_k<<<blocks_for(N, SN_WARPS), SN_THREADS, 0, s>>>(x, d, P->rowptr, P->col, S.lev, S.node,
-                                                                            N, rl1, S.B, 0, cnt, nullptr, nullptr);
+    note_launch(), sn_pairs_k<<<blocks_for(N, SN_WARPS), SN_THREADS, 0, s>>>(X, P->rowptr, P->col, S.lev, S.node, N,
+                                                                            rl1, S.B, 0, cnt, nullptr, nullptr);
     KC_CUDA(cudaGetLastError());
     KC_TRY(exclusive_scan_i32_to_i64(cnt, off, N, A, s));
     int64_t total = 0;
@@ -354,8 +401,8 @@ static kc_status sn_pairs(const double* x, int d, const kc_pattern* P, double rl
     KC_TRY(A.get(&k1, total));
     KC_TRY(A.get(&v0, total));
     KC_TRY(A.get(&v1, total));
-    note_launch(), sn_pairs_k<<<blocks_for(N, SN_WARPS), SN_THREADS, 0, s>>>(x, d, P->rowptr, P->col, S.lev, S.node,
-                                                                            N, rl1, S.B, 1, cnt, off, k0);
+    note_launch(), sn_pairs_k<<<blocks_for(N, SN_WARPS), SN_THREADS, 0, s>>>(X, P->rowptr, P->col, S.lev, S.node, N,
+                                                                            rl1, S.B, 1, cnt, off, k0);
     KC_CUDA(cudaGetLastError());
     KC_CUDA(cudaMemsetAsync(v0, 0, sizeof(int64_t) * total, s));
     KC_TRY(radix_sort_u64_i64(k0, v0, k1, v1, total, 2 * S.B, A, s));
@@ -374,8 +421,8 @@ static kc_status sn_pairs(const double* x, int d, const kc_pattern* P, double rl
 }
 
 // levels, supernodes and the assignment (per maximin position)
-static kc_status sn_nodes(const double* x, int d, const double* l, const kc_pattern* P, double rl1, SnState& S,
-                          Arena& A, cudaStream_t s) {
+static kc_status sn_nodes(const SnPoints& X, const double* l, const kc_pattern* P, double rl1, SnState& S, Arena& A,
+                          cudaStream_t s) {
     const int64_t N = P->N;
     KC_TRY(A.get(&S.lev, N));
     KC_TRY(A.get(&S.state, N));
@@ -392,7 +439,7 @@ static kc_status sn_nodes(const double* x, int d, const double* l, const kc_patt
     KC_CUDA(cudaMemsetAsync(cnt_l, 0, sizeof(int32_t) * N, s));
     KC_CUDA(cudaMemsetAsync(fill_l, 0, sizeof(int32_t) * N, s));
     note_launch(), sn_conflicts_k<<<blocks_for(N, SN_WARPS), SN_THREADS, 0, s>>>(
-        x, d, P->rowptr, P->col, S.lev, N, rl1, 0, cnt_e, cnt_l, nullptr, nullptr, nullptr);
+        X, P->rowptr, P->col, S.lev, N, rl1, 0, cnt_e, cnt_l, nullptr, nullptr, nullptr);
     KC_CUDA(cudaGetLastError());
     note_launch(), sn_sum_k<<<blocks_for(N, 256), 256, 0, s>>>(cnt_e, cnt_l, N, cnt);
     KC_CUDA(cudaGetLastError());
@@ -401,7 +448,7 @@ static kc_status sn_nodes(const double* x, int d, const double* l, const kc_patt
     KC_TRY(sync_read(off + N, &total, sizeof(total), s));
     KC_TRY(A.get(&list, total));
     note_launch(), sn_conflicts_k<<<blocks_for(N, SN_WARPS), SN_THREADS, 0, s>>>(
-        x, d, P->rowptr, P->col, S.lev, N, rl1, 1, cnt_e, cnt_l, off, fill_l, list);
+        X, P->rowptr, P->col, S.lev, N, rl1, 1, cnt_e, cnt_l, off, fill_l, list);
     KC_CUDA(cudaGetLastError());
     KC_CUDA(cudaMemsetAsync(S.state, 0, N, s));
     unsigned long long* und;
@@ -416,7 +463,7 @@ static kc_status sn_nodes(const double* x, int d, const double* l, const kc_patt
         if (h == 0) break;
         if (++rounds > SN_MAX_ROUNDS) return fail(KC_ECUDA, "supernodal: independent-set rounds did not finish");
     }
-    note_launch(), sn_assign_k<<<blocks_for(N, 256), 256, 0, s>>>(x, d, off, cnt, list, S.state, N, S.node);
+    note_launch(), sn_assign_k<<<blocks_for(N, 256), 256, 0, s>>>(X.x, X.d, off, cnt, list, S.state, N, S.node);
     KC_CUDA(cudaGetLastError());
     return KC_OK;
 }
@@ -533,8 +580,10 @@ kc_status supernodal_impl(const double* x_ord, const double* l, int d, double rh
     Arena A(s);
     SnState S;
     while (S.B < 31 && ((int64_t)1 << S.B) < N) ++S.B;
-    KC_TRY(sn_nodes(x_ord, d, l, P, rl1, S, A, s));
-    KC_TRY(sn_pairs(x_ord, d, P, rl1, S, A, s));
+    SnPoints X;
+    KC_TRY(sn_points(x_ord, N, d, X, A, s));
+    KC_TRY(sn_nodes(X, l, P, rl1, S, A, s));
+    KC_TRY(sn_pairs(X, P, rl1, S, A, s));
     int32_t* color;
     KC_TRY(A.get(&color, N));
     KC_TRY(sn_colors(S, N, color, A, s));
