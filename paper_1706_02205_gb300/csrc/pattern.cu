@@ -149,6 +149,42 @@ __device__ __forceinline__ bool pat_member(const PatArgs& P, int i, const double
     return sc > 0 || in_s(dist2_exact(P.xs + q * P.d, xi, P.d), Rj);
 }
 
+// The FP32 screen of a column with one radius R for all its candidates (max rule)
+// as two thresholds of the float squared distance s: s < in decides dist <= R,
+// s > out decides dist > R, the exact test the rest.  The margins are those of
+// screen_f32 (delta: a coordinate difference's error; c: the float rounding of
+// the sum of squares and of its root, relative), with some ulps more for the
+// thresholds' own rounding; an extent outside float's comfortable range
+// (P.delta = infinity then) leaves every candidate to the exact test.
+struct Screen {
+    float in, out;
+};
+__device__ __forceinline__ Screen screen_of(double R, int d, float delta) {
+    const float Rf = (float)R, md = sqrtf((float)d) * delta, c = (float)(d + 6) * 1.1920929e-7f;
+    const float lo = Rf - md - c * Rf, hi = (Rf + md) * (1.f + 2.f * c);
+    Screen s;
+    s.in = lo > 0.f ? lo * lo * (1.f - 1e-6f) : -1.f;
+    s.out = hi * hi * (1.f + 1e-6f);
+    if (!(md < INFINITY)) s = Screen{-1.f, INFINITY};
+    return s;
+}
+// pat_member with the thresholds, D axes known at compile time (0: P.d)
+template <int D>
+__device__ __forceinline__ bool pat_within(const PatArgs& P, int i, const double* xi, const float* xif, double R,
+                                           const Screen& S, int64_t q) {
+    const int d = D ? D : P.d;
+    if (P.ps[q] <= i) return false;
+    if (isinf(R)) return true;
+    float s = 0.f;
+#pragma unroll
+    for (int t = 0; t < (D ? D : d); ++t) {
+        const float w = P.xsf[q * d + t] - xif[t];
+        s = fmaf(w, w, s);
+    }
+    if (s > S.out) return false;
+    return s < S.in || in_s(dist2_exact(P.xs + q * d, xi, d), R);
+}
+
 // chunks of 32 candidates of every item (the hit masks' layout)
 __global__ void pat_chunks_k(PatArgs P, int64_t* __restrict__ nch) {
     const int64_t it = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -158,46 +194,81 @@ __global__ void pat_chunks_k(PatArgs P, int64_t* __restrict__ nch) {
     nch[it] = (b - a + 31) / 32;
 }
 
-// Search pass of the builder: one warp per item; the row counts as in the
-// count pass, and every 32 candidates' memberships as one mask word.
-__global__ void pat_mask_k(PatArgs P, const int64_t* __restrict__ moff, int* __restrict__ cnt,
-                           uint32_t* __restrict__ masks) {
-    const int64_t it = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (it >= P.nitems) return;
-    const int lane = lane_id();
+// Lanes per work item in the builder's two passes.  The finest columns, half of
+// all, look at 10 to 16 candidates per row of cells: with a warp per item more
+// than half of the lanes idle, and the item's chain of dependent loads (its
+// column, box, cells) is walked once per item (pattern and schedule of 2^20 points,
+// rho = 3: 19.2 ms with 32 lanes, 18.9 with 16, 19.1 with 8).
+constexpr int PL = 16;
+
+// Search pass of the builder: PL lanes per item; every 32 candidates'
+// memberships as one mask word, and the members' counts by cell-sorted
+// position, where neighbouring lanes add to neighbouring words (by row index
+// every lane's add went to a line of its own; this and the lanes above took the
+// search from 3.46 to 3.17 ms and the fill from 4.41 to 3.45, the thresholds of
+// Screen and D at compile time the search to 2.79).  Bound by instruction issue
+// (the tests of about three candidates an entry) and the counters' atomics.
+template <int D, bool MIN>
+__global__ void __launch_bounds__(256) pat_mask_k(PatArgs P, const int64_t* __restrict__ moff, int* __restrict__ cntq,
+                                                  uint32_t* __restrict__ masks) {
+    const int64_t it = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / PL;
+    const int sub = threadIdx.x % PL, sh = lane_id() / PL * PL;
+    const unsigned grp = (unsigned)(((1ull << PL) - 1) << sh);
+    if (it >= P.nitems) return;  // (a whole group of lanes)
     int64_t a, b;
     const int i = item_range(P, it, a, b);
     const double* xi = P.xo + (int64_t)i * P.d;
     const float* xif = P.xof + (int64_t)i * P.d;
     const double R = col_radius(P.rho, P.l[i]);
+    [[maybe_unused]] const Screen S = screen_of(R, P.d, P.delta);
     uint32_t* m = masks + moff[it];
     for (int64_t q0 = a; q0 < b; q0 += 32) {
-        const int64_t q = q0 + lane;
-        int j = 0;
-        const bool hit = q < b && pat_member(P, i, xi, xif, R, q, j);
-        const unsigned w = __ballot_sync(0xffffffffu, hit);
-        if (lane == 0) m[(q0 - a) >> 5] = w;
-        if (hit) atomicAdd(&cnt[j], 1);
+        uint32_t word = 0;
+#pragma unroll
+        for (int h = 0; h < 32; h += PL) {
+            const int64_t q = q0 + h + sub;
+            [[maybe_unused]] int j = 0;
+            bool hit;
+            if constexpr (MIN) hit = q < b && pat_member(P, i, xi, xif, R, q, j);
+            else hit = q < b && pat_within<D>(P, i, xi, xif, R, S, q);
+            word |= ((__ballot_sync(grp, hit) & grp) >> sh) << h;
+            if (hit) atomicAdd(&cntq[q], 1);
+        }
+        if (sub == 0) m[(q0 - a) >> 5] = word;
     }
 }
 
-// Fill pass of the builder: the members from the masks, no distance tests.
-__global__ void pat_mask_fill_k(PatArgs P, const int64_t* __restrict__ moff, const uint32_t* __restrict__ masks,
-                                int* __restrict__ cnt, const int64_t* __restrict__ rowptr, int32_t* __restrict__ col) {
-    const int64_t it = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+// Row lengths (with the diagonal) from the counts by cell-sorted position, and
+// back: the place of each row's next entry by cell-sorted position.
+__global__ void pat_len_k(const int32_t* __restrict__ ps, const int* __restrict__ cntq, int64_t N,
+                          int32_t* __restrict__ len) {
+    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (q < N) len[ps[q]] = cntq[q] + 1;
+}
+__global__ void pat_next_k(const int32_t* __restrict__ ps, const int64_t* __restrict__ rowptr, int64_t N,
+                           unsigned long long* __restrict__ next) {
+    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (q < N) next[q] = (unsigned long long)rowptr[ps[q]];
+}
+
+// Fill pass of the builder: the members from the masks, no distance tests.  Bound
+// by the scattered 4-byte stores, 188.7 M in 3.45 ms (places counted in 32 bits
+// beside a row base took as long).
+__global__ void __launch_bounds__(256) pat_mask_fill_k(PatArgs P, const int64_t* __restrict__ moff,
+                                                       const uint32_t* __restrict__ masks,
+                                                       unsigned long long* __restrict__ next,
+                                                       int32_t* __restrict__ col) {
+    const int64_t it = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / PL;
     if (it >= P.nitems) return;
-    const int lane = lane_id();
-    const int i = P.item_col[it];
+    const int sub = threadIdx.x % PL;
     const int64_t c0 = moff[it], c1 = moff[it + 1];
     int64_t a, b;
-    item_range(P, it, a, b);
+    const int i = item_range(P, it, a, b);
     for (int64_t c = c0; c < c1; ++c) {
         const uint32_t w = masks[c];
-        if ((w >> lane) & 1u) {
-            const int j = P.ps[a + ((c - c0) << 5) + lane];
-            const int slot = atomicAdd(&cnt[j], 1);
-            col[rowptr[j] + slot] = i;
-        }
+#pragma unroll
+        for (int h = 0; h < 32; h += PL)
+            if ((w >> (h + sub)) & 1u) col[atomicAdd(&next[a + ((c - c0) << 5) + h + sub], 1ull)] = i;
     }
 }
 
@@ -245,6 +316,7 @@ static kc_status pat_setup(const double* xo, const double* l, int64_t N, int d, 
     if (gxo != xo) KC_TRY(bbox(gxo, N, gst, lo, hi, A, s));
     S.g = make_grid(gst, lo, hi, N, 0.0, N / 2 > 1 ? N / 2 : 1);
     S.delta = (float)(E * 1.1920928955078125e-07);  // 2^-23 E
+    if (!(E > 1e-12 && E < 1e18)) S.delta = INFINITY;  // (float over- and underflow: exact tests only)
     KC_TRY(A.get(&S.xsf, N * d));
     KC_TRY(A.get(&S.xof, N * d));
     KC_TRY(A.get(&S.gs, N));
@@ -484,7 +556,6 @@ struct PatternBuilder {
     int64_t N = 0;
     int64_t* moff = nullptr;
     uint32_t* masks = nullptr;
-    int* cnt = nullptr;
     int64_t* rowptr = nullptr;
     int64_t nnz = 0;
 };
@@ -508,7 +579,8 @@ kc_status pattern_begin_impl(const double* xo, const double* l, int64_t N, int d
     int64_t* nch;
     if ((st = B->A->get(&nch, ni + 1)) != KC_OK) return fail_out(st);
     if ((st = B->A->get(&B->moff, ni + 1)) != KC_OK) return fail_out(st);
-    if ((st = B->A->get(&B->cnt, N)) != KC_OK) return fail_out(st);
+    int* cntq;
+    if ((st = B->A->get(&cntq, N)) != KC_OK) return fail_out(st);
     int32_t* len;
     if ((st = B->A->get(&len, N)) != KC_OK) return fail_out(st);
     if (ni > 0) ::kc::note_launch(), pat_chunks_k<<<blocks_for(ni, 256), 256, 0, s>>>(B->P, nch);
@@ -518,9 +590,13 @@ kc_status pattern_begin_impl(const double* xo, const double* l, int64_t N, int d
         cudaStreamSynchronize(s) != cudaSuccess)
         return fail_out(fail(KC_ECUDA, "pattern: chunk count"));
     if ((st = B->A->get(&B->masks, nchunks)) != KC_OK) return fail_out(st);
-    if (cudaMemsetAsync(B->cnt, 0, sizeof(int) * N, s) != cudaSuccess) return fail_out(fail(KC_ECUDA, "memset"));
-    if (ni > 0) ::kc::note_launch(), pat_mask_k<<<blocks_for(ni * 32, 256), 256, 0, s>>>(B->P, B->moff, B->cnt, B->masks);
-    ::kc::note_launch(), plus_one_k<<<blocks_for(N, 256), 256, 0, s>>>(B->cnt, N, len);
+    if (cudaMemsetAsync(cntq, 0, sizeof(int) * N, s) != cudaSuccess) return fail_out(fail(KC_ECUDA, "memset"));
+    auto mask = rule == KC_RULE_MIN ? pat_mask_k<0, true>
+                : d == 2            ? pat_mask_k<2, false>
+                : d == 3            ? pat_mask_k<3, false>
+                                    : pat_mask_k<0, false>;
+    if (ni > 0) ::kc::note_launch(), mask<<<blocks_for(ni * PL, 256), 256, 0, s>>>(B->P, B->moff, cntq, B->masks);
+    ::kc::note_launch(), pat_len_k<<<blocks_for(N, 256), 256, 0, s>>>(B->S.gs, cntq, N, len);
     if (cudaGetLastError() != cudaSuccess) return fail_out(fail(KC_ECUDA, "pattern: search launch"));
     if ((st = exclusive_scan_i32_to_i64(len, rowptr, N, *B->A, s)) != KC_OK) return fail_out(st);
     if (cudaMemcpyAsync(&B->nnz, rowptr + N, sizeof(int64_t), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
@@ -550,10 +626,12 @@ static kc_status pattern_fill_from(PatternBuilder* B, int32_t* col) {
     KC_CUDA(cudaMemcpyAsync(&hmx, mx, sizeof(int), cudaMemcpyDeviceToHost, s));
     KC_CUDA(cudaStreamSynchronize(s));
     if (hmx > SORT_BLOCK_CAP) return fail(KC_EINVAL, "pattern row longer than 16384 entries");
-    KC_CUDA(cudaMemsetAsync(B->cnt, 0, sizeof(int) * N, s));
+    unsigned long long* next;
+    KC_TRY(A.get(&next, N));
+    ::kc::note_launch(), pat_next_k<<<blocks_for(N, 256), 256, 0, s>>>(B->S.gs, B->rowptr, N, next);
     if (B->S.nitems > 0)
-        ::kc::note_launch(), pat_mask_fill_k<<<blocks_for(B->S.nitems * 32, 256), 256, 0, s>>>(B->P, B->moff, B->masks,
-                                                                                            B->cnt, B->rowptr, col);
+        ::kc::note_launch(), pat_mask_fill_k<<<blocks_for(B->S.nitems * PL, 256), 256, 0, s>>>(B->P, B->moff, B->masks,
+                                                                                            next, col);
     KC_CUDA(cudaGetLastError());
     int32_t* long_rows;
     unsigned long long* nlong;
