@@ -263,7 +263,8 @@ __global__ void scan_tile_k(const Tin* __restrict__ in, int64_t n, const int64_t
     if (blockIdx.x == gridDim.x - 1 && threadIdx.x == SCAN_THREADS - 1) out[n] = run;
 }
 
-__global__ void scan_single_k(const int64_t* __restrict__ in, int64_t n, int64_t* __restrict__ out) {
+template <typename Tin>
+__global__ void scan_single_k(const Tin* __restrict__ in, int64_t n, int64_t* __restrict__ out) {
     // one block, sequential over chunks of 1024 (used for short arrays)
     __shared__ int64_t carry;
     __shared__ int64_t wsum[32];
@@ -271,7 +272,7 @@ __global__ void scan_single_k(const int64_t* __restrict__ in, int64_t n, int64_t
     __syncthreads();
     for (int64_t base = 0; base < n; base += blockDim.x) {
         int64_t i = base + threadIdx.x;
-        int64_t v = i < n ? in[i] : 0;
+        int64_t v = i < n ? (int64_t)in[i] : 0;
         int lane = lane_id(), w = threadIdx.x >> 5;
         int64_t incl = v;
         for (int o = 1; o < 32; o <<= 1) {
@@ -298,12 +299,17 @@ static kc_status scan_impl(const Tin* in, int64_t* out, int64_t n, Arena& A, cud
         return KC_OK;
     }
     int64_t nb = (n + SCAN_TILE - 1) / SCAN_TILE;
+    if (nb <= 2) {  // one launch instead of three (one block walks at most four rounds)
+        ::kc::note_launch(), scan_single_k<Tin><<<1, 1024, 0, s>>>(in, n, out);
+        KC_CUDA(cudaGetLastError());
+        return KC_OK;
+    }
     int64_t* bsum;
     int64_t* boff;
     KC_TRY(A.get(&bsum, nb));
     KC_TRY(A.get(&boff, nb + 1));
     ::kc::note_launch(), scan_reduce_k<Tin><<<(unsigned)nb, SCAN_THREADS, 0, s>>>(in, n, bsum);
-    if (nb <= 8192) ::kc::note_launch(), scan_single_k<<<1, 1024, 0, s>>>(bsum, nb, boff);
+    if (nb <= 8192) ::kc::note_launch(), scan_single_k<int64_t><<<1, 1024, 0, s>>>(bsum, nb, boff);
     else KC_TRY(scan_impl<int64_t>(bsum, boff, nb, A, s));
     ::kc::note_launch(), scan_tile_k<Tin><<<(unsigned)nb, SCAN_THREADS, 0, s>>>(in, n, boff, out);
     KC_CUDA(cudaGetLastError());
