@@ -64,6 +64,18 @@ constexpr int BF_MAXG = 8;       // columns per group at most
 #endif
 constexpr int BU = KC_BLOCK_BU;
 
+// Slots of the table of a prefix of P columns, 2^bits: a load factor of at most
+// 3/4, or 3/8 where shared memory allows (group_launch).  Probe loops run as long
+// as the slowest lane's, so the sparser table pays: 42.9 against 39.9 ms on the
+// 2^20 supernodal pattern (rho = 3, FP32 form; 3/16: 41.4).  Two-choice buckets,
+// without probe loops, took 48.7: their longer code, not the loops, then limits.
+constexpr int PT_DENSE = 4, PT_SPARSE = 8;
+__host__ __device__ __forceinline__ int table_bits(int P, int den) {
+    int hb = 5;
+    while (3 * ((int64_t)1 << hb) < (int64_t)den * P) ++hb;
+    return hb;
+}
+
 template <typename T>
 struct GroupArgs {
     int64_t N;
@@ -87,7 +99,7 @@ struct GroupArgs {
     unsigned long long* zero_piv;
     KernelParams kp;
     long long spin_limit;
-    int hbits;  // prefix table: 2^hbits slots
+    int hbits;  // prefix table: at most 2^hbits slots
     int pmax;   // longest shared prefix: rows of the value table
     int lanes;  // lanes per row
 };
@@ -128,6 +140,58 @@ __device__ __forceinline__ float fsub_dot(float v, float a, float b) { return fm
 template <>
 __device__ __forceinline__ double fsub_dot(double v, double a, double b) { return fma(-a, b, v); }
 
+// Acc<float> for two neighbouring columns in packed FP32 pairs: the same
+// operations, each rounded as there, at half the issue slots, and nested so that
+// the pairs past the group's last column are jumped over: 39.9 -> 37.4 ms on the
+// 2^20 supernodal pattern (all four pairs always: 38.3; the nesting without pairs:
+// 40.4).  A last odd column's partner holds zeros, whose sums stay zero.
+__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b) {
+    unsigned long long r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ unsigned long long sub2(unsigned long long a, unsigned long long b) {
+    unsigned long long r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ unsigned long long pack2(float a, float b) {
+    return (unsigned long long)__float_as_uint(b) << 32 | __float_as_uint(a);
+}
+struct PairEntry {
+    unsigned long long w, neg;  // (w, w), (-w, -w)
+    __device__ __forceinline__ explicit PairEntry(float x) : w(pack2(x, x)), neg(pack2(-x, -x)) {}
+};
+struct AccPair {
+    unsigned long long s = 0, c = 0;
+    __device__ __forceinline__ void add(const PairEntry& e, unsigned long long v) {
+        const unsigned long long p = mul2(e.w, v);
+        const unsigned long long ep = fma2(e.w, v, mul2(e.neg, v));  // w v - p
+        const unsigned long long ns = add2(s, p);
+        const unsigned long long z = sub2(ns, s);
+        const unsigned long long es = add2(sub2(s, sub2(ns, z)), sub2(p, z));
+        s = ns;
+        c = add2(c, add2(ep, es));
+    }
+    __device__ __forceinline__ void split(Acc<float>& a, Acc<float>& b) const {
+        a.s = __uint_as_float((unsigned)s);
+        a.c = __uint_as_float((unsigned)c);
+        b.s = __uint_as_float((unsigned)(s >> 32));
+        b.c = __uint_as_float((unsigned)(c >> 32));
+    }
+    __device__ __forceinline__ void split(Acc<double>&, Acc<double>&) const {}
+};
+
 template <typename T, int MM, bool GEN, int GC, int M4 = MM>
 __device__ __forceinline__ void group_rows(const GroupArgs<T>& A, int64_t qb, int64_t qe, int g0, int m,
                                            const unsigned long long* tab, int hb, const T* V, const T* Laa,
@@ -149,6 +213,8 @@ __device__ __forceinline__ void group_rows(const GroupArgs<T>& A, int64_t qb, in
         if (act && sub < m)
             th = theta_off<T, GEN>(A.kp, A.d, A.x + (int64_t)j * A.d, A.x + (int64_t)(g0 + sub) * A.d);
         Acc<T> acc[M4];
+        constexpr bool PAIRS = sizeof(T) == 4 && M4 == 8;
+        [[maybe_unused]] AccPair pair[PAIRS ? M4 / 2 : 1];
         if (act) {
             for (int64_t f0 = es + sub; f0 < e; f0 += (int64_t)BU * G) {
                 int k[BU];
@@ -164,13 +230,31 @@ __device__ __forceinline__ void group_rows(const GroupArgs<T>& A, int64_t qb, in
                     const int p = k[v] >= 0 ? prefix_find(tab, hb, k[v]) : -1;
                     if (p >= 0) {
                         const T* vp = V + (int64_t)p * MM;
+                        if constexpr (PAIRS) {
+                            const PairEntry e2(w[v]);
+                            const ulonglong2* vq = (const ulonglong2*)vp;
+                            ulonglong2 x = vq[0];
+                            pair[0].add(e2, x.x);
+                            if (m > 2) {
+                                pair[1].add(e2, x.y);
+                                if (m > 4) {
+                                    x = vq[1];
+                                    pair[2].add(e2, x.x);
+                                    if (m > 6) pair[3].add(e2, x.y);
+                                }
+                            }
+                        } else {
 #pragma unroll
-                        for (int u = 0; u < M4; ++u)
-                            if (u < m) acc[u].add(w[v], vp[u]);
+                            for (int u = 0; u < M4; ++u)
+                                if (u < m) acc[u].add(w[v], vp[u]);
+                        }
                     }
                 }
             }
         }
+        if constexpr (PAIRS)
+#pragma unroll
+            for (int u = 0; u < M4; u += 2) pair[u / 2].split(acc[u], acc[u + 1]);
 #pragma unroll
         for (int u = 0; u < M4; ++u)
             if (u < m) acc[u].group_reduce(G);
@@ -243,10 +327,9 @@ __global__ void __launch_bounds__(BF_THREADS, KC_BLOCK_MINB) ichol_group_k(Group
         }
         fence_acq_rel_gpu();  // acquire: the prefix values are visible from here on
 
-        // stage the prefix: table column -> position (sized to this prefix, load
-        // factor <= 3/4), values of the m rows
-        int hb = 5;
-        while (3 * (1 << hb) < 4 * P) ++hb;
+        // stage the prefix: table column -> position (sized to this prefix), values of
+        // the m rows
+        const int hb = min(A.hbits, table_bits(P, PT_SPARSE));
         for (int h = tid; h < (1 << hb); h += BF_THREADS) tab[h] = ~0ull;
         int64_t rs[MM];
 #pragma unroll
@@ -470,15 +553,29 @@ __global__ void grp_tasks_fill_k(const int32_t* __restrict__ gorder, const int64
 kc_status exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, Arena& A, cudaStream_t s);
 
 template <typename T, int MM, bool GEN>
-static kc_status group_launch(const GroupArgs<T>& a, cudaStream_t s) {
-    const size_t smem = sizeof(double) * (MM * (MM + 1) / 2 + MM) + sizeof(T) * (MM * MM + MM) + 16 + 16 +
-                        sizeof(unsigned long long) * ((size_t)1 << a.hbits) + sizeof(T) * (size_t)a.pmax * MM;
+static kc_status group_launch(GroupArgs<T> a, cudaStream_t s) {
     auto kfn = ichol_group_k<T, MM, GEN, 0>;
     if constexpr (sizeof(T) == 4)
         if (a.lanes == 8) kfn = ichol_group_k<T, MM, GEN, 8>;  // (the FP64 form measured no gain)
     KC_TRY(allow_dynamic_smem(kfn));
+    // the sparser table unless it costs resident CTAs (or does not fit)
+    size_t smem = 0;
     int per_sm = 0;
-    KC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kfn, BF_THREADS, smem));
+    for (int den : {PT_DENSE, PT_SPARSE}) {
+        const int hb = table_bits(a.pmax, den);
+        const size_t bytes = sizeof(double) * (MM * (MM + 1) / 2 + MM) + sizeof(T) * (MM * MM + MM) + 16 + 16 +
+                             sizeof(unsigned long long) * ((size_t)1 << hb) + sizeof(T) * (size_t)a.pmax * MM;
+        int n = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kfn, BF_THREADS, bytes) != cudaSuccess) {
+            if (den == PT_DENSE) return fail(KC_ECUDA, "grouped factor: occupancy");
+            (void)cudaGetLastError();
+            break;
+        }
+        if (n < per_sm || (den == PT_SPARSE && n < 1)) break;
+        per_sm = n;
+        smem = bytes;
+        a.hbits = hb;
+    }
     if (per_sm < 1) return fail(KC_EINVAL, "grouped factor: the prefix table exceeds an SM's shared memory");
     ::kc::note_launch(), kfn<<<sm_count() * per_sm, BF_THREADS, smem, s>>>(a);
     KC_CUDA(cudaGetLastError());
@@ -592,8 +689,6 @@ kc_status factor_blocked_impl(const kc_pattern* P, const double* x, int d, const
     KC_CUDA(cudaMemsetAsync(ticket, 0, sizeof(unsigned long long), s));
     KC_CUDA(cudaMemsetAsync(zp, 0, sizeof(unsigned long long), s));
     KC_CUDA(cudaMemsetAsync(status, 0, sizeof(int), s));
-    int hb = 5;
-    while (3 * (1 << hb) < 4 * std::max(hp, 1)) ++hb;  // load factor <= 3/4
     const int pm = std::max(hp, 1);
     cudaEvent_t e0, e1;
     KC_CUDA(cudaEventCreate(&e0));
@@ -603,11 +698,11 @@ kc_status factor_blocked_impl(const kc_pattern* P, const double* x, int d, const
     const bool gen = kp.nu_code > 2;
     if (prec == KC_FP64) {
         GroupArgs<double> a{N, d, x, P->rowptr, P->col, P->colptr, P->rowidx, P->slot, gstart, group_of, tasks, nt, rpt,
-                            (double*)val, diag, done, ticket, status, zp, kp, spin, hb, pm, lanes};
+                            (double*)val, diag, done, ticket, status, zp, kp, spin, 0, pm, lanes};
         st = gen ? group_launch<double, BF_MAXG, true>(a, s) : group_launch<double, BF_MAXG, false>(a, s);
     } else {
         GroupArgs<float> a{N, d, x, P->rowptr, P->col, P->colptr, P->rowidx, P->slot, gstart, group_of, tasks, nt, rpt,
-                           (float*)val, diag, done, ticket, status, zp, kp, spin, hb, pm, lanes};
+                           (float*)val, diag, done, ticket, status, zp, kp, spin, 0, pm, lanes};
         st = gen ? group_launch<float, BF_MAXG, true>(a, s) : group_launch<float, BF_MAXG, false>(a, s);
     }
     if (st != KC_OK) {
