@@ -378,17 +378,6 @@ struct Cand {
             take(__shfl_xor_sync(0xffffffffu, v, o), __shfl_xor_sync(0xffffffffu, i, o), __shfl_xor_sync(0xffffffffu, g, o));
     }
 };
-// the block's best candidate, in every thread (sh: 32 entries)
-__device__ __forceinline__ Cand block_best(Cand c, Cand* sh) {
-    c.warp_best();
-    __syncthreads();  // sh is free
-    if (lane_id() == 0) sh[threadIdx.x >> 5] = c;
-    __syncthreads();
-    c = lane_id() < (int)(blockDim.x >> 5) ? sh[lane_id()] : Cand{0.0, 0, -1};
-    c.warp_best();
-    return c;
-}
-
 // A grid-wide barrier for a cooperative launch (every block resident): the
 // last block to arrive resets the count and advances the generation; the
 // others poll the generation with backoff, at most `limit` cycles, after
@@ -424,73 +413,179 @@ __device__ bool grid_barrier(unsigned* count, unsigned* gen, int* status, long l
     return ok != 0;
 }
 
-// All greedy steps in one cooperative launch of at most one CTA per SM.  In step
-// k every block leaves the best of its points in its slot of buffer k & 1 and
-// reads all slots, so every block finds the same winner, marks it and pushes it
-// to its own points.  The slots carry their own readiness, a parity bit in each
-// of their two words that changes with every use of a buffer: no barrier and no
-// fence.  A block writes a buffer again only after it has read the next one
-// whole, which the others write after they have read this one.  (With a grid
-// barrier and 608 blocks a step took 14.6 us at 2^20 points, 7.4 at 2000; now
-// 10.9 and 3.1.)
+// A greedy step's candidates: the squared distance as its bits, which order like
+// the values (integer compares: the FP64 pipe takes 16 clocks for a warp's
+// compare), the point's original index and its place (g < 0: none).
+struct GreedyCand {
+    unsigned long long v;
+    int i, g;
+};
+__device__ __forceinline__ GreedyCand no_cand() { return GreedyCand{0ull, INT_MAX, -1}; }
+__device__ __forceinline__ void greedy_take(GreedyCand& c, unsigned long long v, int i, int g) {
+    if (v > c.v || (v == c.v && i < c.i)) c = GreedyCand{v, i, g};
+}
+// the best of the warp's candidates (largest v, then smallest i), in every lane
+__device__ __forceinline__ GreedyCand greedy_best(const GreedyCand& c) {
+    const unsigned FULL = 0xffffffffu;
+    const unsigned hi = (unsigned)(c.v >> 32), mh = __reduce_max_sync(FULL, hi);
+    const unsigned lo = hi == mh ? (unsigned)c.v : 0u, ml = __reduce_max_sync(FULL, lo);
+    const bool top = hi == mh && lo == ml;
+    const int mi = __reduce_min_sync(FULL, top ? c.i : INT_MAX);
+    const int src = __ffs(__ballot_sync(FULL, top && c.i == mi)) - 1;
+    return GreedyCand{(unsigned long long)mh << 32 | ml, mi, __shfl_sync(FULL, c.g, src)};
+}
+// a nonnegative double's bits as a float, rounded down (integer operations), but
+// not below float's smallest normal number
+__device__ __forceinline__ float float_below(unsigned long long v) {
+    const unsigned h = (unsigned)(v >> 32);
+    if (h < 897u << 20) return 1.1754944e-38f;
+    if (h >= 1151u << 20) return h >= 2047u << 20 ? INFINITY : 3.4028234e38f;
+    return __uint_as_float(((h - (896u << 20)) << 3) | ((unsigned)v >> 29));
+}
+
+// All greedy steps in one cooperative launch of at most one CTA per SM.  The points
+// lie in cell order, so stretches of 32 (or a small multiple) have small boxes; a
+// warp has up to 32 of them, the state of each, its box and its best candidate, in
+// a lane.  A step looks at a stretch's points only if the winner is one of them or
+// its distance from the box is not above the largest of their values, for
+// otherwise none can change.  Neighbouring stretches go to different blocks and
+// warps: a step takes as long as the warp with the most to look at, whose chains
+// of loads follow one another, and so a winner's surroundings are spread over all
+// the SMs.  Every block sends the best of its warps to a slot in every block's row
+// of buffer k & 1 and reads its own row, so every block finds the same winner
+// (with one slot a block that all poll, the polls crowd a few lines: 8.9 us a step).  The slots carry
+// their own readiness, a parity bit in each of their two words that changes with
+// every use of a buffer: no barrier and no fence.  A block writes a buffer again
+// only after it has read the next one whole, which the others write after they
+// have read this one.  The shared buffers alternate likewise: a warp writes one
+// again only after a block barrier that every warp reaches past its last read.
+// A step took 14.6 us at 2^20 points and 7.4 at 2000 with a grid barrier and 608
+// blocks, 10.9 and 3.1 with the slots but every point looked at and FP64
+// compares, and 4.8 and 2.1 now.
 __global__ void __launch_bounds__(GREEDY_THREADS, 1)
     ord_greedy_loop_k(const double* __restrict__ xg, int d, const int32_t* __restrict__ idg, double* v2, int* stat,
                       int64_t N, int64_t steps, ulonglong2* slots, const float* __restrict__ xgf, float delta,
                       int* status, long long limit) {
-    __shared__ Cand sh[32];
-    const int nblk = gridDim.x;
+    __shared__ GreedyCand sh[2][32], sx[2][32];
+    const int nblk = gridDim.x, lane = lane_id(), wrp = threadIdx.x >> 5;
+    const unsigned FULL = 0xffffffffu;
     const unsigned long long PB = 1ull << 63;
-    int w = -1;  // the winner of the previous step
-    for (int64_t k = 0; k <= steps; ++k) {
-        Cand c{0.0, 0, -1};
-        const double* xw = w >= 0 ? xg + (int64_t)w * d : nullptr;
-        for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < N; q += (int64_t)nblk * blockDim.x) {
-            if (q == w) stat[q] = 1;  // v2[w] keeps its final value l^2
-            if (q == w || stat[q] != 0) continue;
-            double vq = v2[q];
-            if (w >= 0 && screen_f32(xgf + q * d, xgf + (int64_t)w * d, d, sqrtf((float)vq), delta) != 0) {
-                const double dd = dist2_exact(xg + q * d, xw, d);
-                if (dd < vq) {
-                    vq = dd;
-                    v2[q] = dd;
+    const int64_t nw = (int64_t)nblk * (GREEDY_THREADS / 32);
+    // stretches of `per` points; lane j keeps the state of the warp's stretch j
+    const int64_t per = 32 * ((N + 1024 * nw - 1) / (1024 * nw)), ns = (N + per - 1) / per;
+    const int64_t gw = (int64_t)wrp * nblk + blockIdx.x;
+    const int mine = ns > gw ? (int)((ns - gw + nw - 1) / nw) : 0;  // the warp's stretches, at most 32
+    const int da = min(d, 3);
+    float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};  // box, first three axes
+    for (int j = 0; j < mine; ++j) {
+        const int64_t q0 = (gw + j * nw) * per, q1 = min(N, q0 + per);
+#pragma unroll
+        for (int t = 0; t < 3; ++t)
+            if (t < da) {
+                float a = INFINITY, b = -INFINITY;
+                for (int64_t q = q0 + lane; q < q1; q += 32) {
+                    const float u = xgf[q * d + t];
+                    a = fminf(a, u);
+                    b = fmaxf(b, u);
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) {
+                    a = fminf(a, __shfl_xor_sync(FULL, a, o));
+                    b = fmaxf(b, __shfl_xor_sync(FULL, b, o));
+                }
+                if (lane == j) {
+                    lo[t] = a;
+                    hi[t] = b;
                 }
             }
-            c.take(vq, idg[q], (int)q);
+    }
+    const int64_t own = (gw + lane * nw) * per;  // the lane's stretch
+    GreedyCand best = no_cand();                 // of the lane's stretch
+    float reach = 0.f;                           // not below the largest value of the lane's stretch
+    int64_t w = -1;                              // the winner of the previous step
+    for (int64_t k = 0; k <= steps; ++k) {
+        bool look = lane < mine;
+        if (look && w >= 0 && (w < own || w >= own + per)) {
+            float s = 0.f;  // not above the squared distance of the winner from the box
+#pragma unroll
+            for (int t = 0; t < 3; ++t)
+                if (t < da) {
+                    const float u = xgf[w * d + t];
+                    const float g = fmaxf(lo[t] - u, u - hi[t]) * (1.f - 1e-6f) - delta;
+                    if (g > 0.f) s = fmaf(g, g, s);
+                }
+            look = !(s * (1.f - 1e-5f) > reach);
+        }
+        for (unsigned todo = __ballot_sync(FULL, look); todo; todo &= todo - 1) {
+            const int j = __ffs(todo) - 1;
+            const int64_t q0 = (gw + j * nw) * per, q1 = min(N, q0 + per);
+            GreedyCand c = no_cand();
+            for (int64_t q = q0 + lane; q < q1; q += 32) {
+                unsigned long long vq = (unsigned long long)__double_as_longlong(v2[q]);
+                const int at = idg[q];
+                if (q == w) stat[q] = 1;  // v2[w] keeps its final value l^2
+                if (q == w || stat[q] != 0) continue;
+                if (w >= 0 && screen_f32(xgf + q * d, xgf + w * d, d, sqrtf(float_below(vq)), delta) != 0) {
+                    const double dd = dist2_exact(xg + q * d, xg + w * d, d);
+                    const unsigned long long u = (unsigned long long)__double_as_longlong(dd);
+                    if (u < vq) {
+                        vq = u;
+                        v2[q] = dd;
+                    }
+                }
+                greedy_take(c, vq, at, (int)q);
+            }
+            c = greedy_best(c);
+            if (lane == j) {
+                best = c;
+                reach = __uint_as_float(__float_as_uint(float_below(c.v)) + (c.v < 0x7ff0000000000000ull));
+            }
         }
         if (k == steps) break;
-        c = block_best(c, sh);
-        if (nblk == 1) {
-            w = c.g;
-            continue;
+        {
+            const GreedyCand c = greedy_best(best);
+            if (lane == 0) sh[k & 1][wrp] = c;
         }
-        ulonglong2* buf = slots + (k & 1) * nblk;
-        const unsigned long long par = ((k >> 1) & 1) ? 0ull : PB;
-        if (threadIdx.x == 0) {
-            // squared distances have no sign bit, indices are below 2^31; no candidate: all ones below it
-            const unsigned long long a = (unsigned long long)vbits(c.v) | par;
-            const unsigned long long b = ((unsigned long long)(unsigned)c.i << 32 | (unsigned)c.g) | par;
-            asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(&buf[blockIdx.x].x), "l"(a) : "memory");
-            asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(&buf[blockIdx.x].y), "l"(b) : "memory");
-        }
-        c = Cand{0.0, 0, -1};
-        bool fine = true;
-        for (int b = threadIdx.x; b < nblk; b += blockDim.x) {
-            unsigned long long u, v;
-            const long long t0 = clock64();
-            for (int poll = 1;; ++poll) {
-                asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(u) : "l"(&buf[b].x) : "memory");
-                asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(&buf[b].y) : "memory");
-                if ((u & PB) == par && (v & PB) == par) break;
-                if (clock64() - t0 > limit || ((poll & 63) == 0 && ld_volatile_s32(status) != 0)) {
-                    atomicCAS(status, 0, DEV_TIMEOUT);
-                    fine = false;
-                    break;
-                }
+        __syncthreads();
+        GreedyCand c = greedy_best(sh[k & 1][lane]);
+        if (nblk > 1) {
+            ulonglong2* buf = slots + (k & 1) * nblk * nblk;
+            const unsigned long long par = ((k >> 1) & 1) ? 0ull : PB;
+            if (threadIdx.x < nblk) {
+                ulonglong2* to = buf + threadIdx.x * nblk + blockIdx.x;
+                // squared distances have no sign bit, indices are below 2^31; no candidate: all ones below it
+                const unsigned long long a = c.v | par;
+                const unsigned long long b = ((unsigned long long)(unsigned)c.i << 32 | (unsigned)c.g) | par;
+                asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(to), "l"(a), "l"(b) : "memory");
             }
-            c.take(__longlong_as_double((long long)(u & ~PB)), (int)((v & ~PB) >> 32), (int)(unsigned)v);
+            bool fine = true;
+            if (32 * wrp < nblk) {
+                c = no_cand();
+                const int b = threadIdx.x;
+                if (b < nblk) {
+                    unsigned long long u, v;
+                    const long long t0 = clock64();
+                    for (int poll = 1;; ++poll) {
+                        asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];"
+                                     : "=l"(u), "=l"(v)
+                                     : "l"(&buf[blockIdx.x * nblk + b])
+                                     : "memory");
+                        if ((u & PB) == par && (v & PB) == par) break;
+                        if (clock64() - t0 > limit || ((poll & 63) == 0 && ld_volatile_s32(status) != 0)) {
+                            atomicCAS(status, 0, DEV_TIMEOUT);
+                            fine = false;
+                            break;
+                        }
+                    }
+                    c = GreedyCand{u & ~PB, (int)((v & ~PB) >> 32), (int)(unsigned)v};
+                }
+                c = greedy_best(c);
+            }
+            if (lane == 0) sx[k & 1][wrp] = 32 * wrp < nblk ? c : no_cand();
+            if (__syncthreads_or(!fine)) return;
+            c = greedy_best(sx[k & 1][lane]);
         }
-        if (__syncthreads_or(!fine)) return;
-        w = block_best(c, sh).g;
+        w = c.g;
     }
 }
 
@@ -865,7 +960,8 @@ kc_status order_impl(const double* x, int64_t N, int d, int32_t* perm, double* l
     // float copy of the coordinates (minus the box corner) for FP32 screens of
     // the distance tests; exact FP64 tests decide every close call
     float* xgf = nullptr;
-    const float delta = (float)(E * 1.1920928955078125e-07);  // 2^-23 E
+    // 2^-23 E; infinite, so that only exact tests decide, where floats could over- or underflow
+    const float delta = E > 1e-12 && E < 1e18 ? (float)(E * 1.1920928955078125e-07) : INFINITY;
     KC_TRY(A.get(&xgf, N * d));
     ::kc::note_launch(), ord_init_k<<<blocks_for(N, 256), 256, 0, s>>>(x, d, gsorted, N, xg, idg, v2, stat, org, xgf);
     // grid coordinates in grid order
@@ -894,8 +990,8 @@ kc_status order_impl(const double* x, int64_t N, int d, int32_t* perm, double* l
         // one block, which exchanges nothing, for up to 4 points a thread
         const int nblk = N <= 4 * GREEDY_THREADS ? 1 : (int)std::min<int64_t>(sms, (N + GREEDY_THREADS - 1) / GREEDY_THREADS);
         ulonglong2* slots;
-        KC_TRY(A.get(&slots, 2 * nblk));
-        KC_CUDA(cudaMemsetAsync(slots, 0, sizeof(ulonglong2) * 2 * nblk, s));
+        KC_TRY(A.get(&slots, 2 * nblk * nblk));
+        KC_CUDA(cudaMemsetAsync(slots, 0, sizeof(ulonglong2) * 2 * nblk * nblk, s));
         int64_t steps = N - 1 < GREEDY_STEPS ? N - 1 : GREEDY_STEPS;
         const double* a_xg = xg;
         const int32_t* a_idg = idg;
