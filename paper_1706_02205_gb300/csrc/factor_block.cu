@@ -145,11 +145,6 @@ __device__ __forceinline__ double fsub_dot(double v, double a, double b) { retur
 // the pairs past the group's last column are jumped over: 39.9 -> 37.4 ms on the
 // 2^20 supernodal pattern (all four pairs always: 38.3; the nesting without pairs:
 // 40.4).  A last odd column's partner holds zeros, whose sums stay zero.
-__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b) {
-    unsigned long long r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
 __device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
     unsigned long long r;
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
@@ -175,13 +170,15 @@ struct PairEntry {
 struct AccPair {
     unsigned long long s = 0, c = 0;
     __device__ __forceinline__ void add(const PairEntry& e, unsigned long long v) {
-        const unsigned long long p = mul2(e.w, v);
-        const unsigned long long ep = fma2(e.w, v, mul2(e.neg, v));  // w v - p
+        // p = w v rounded, by an FMA: a packed multiplication whose product goes into
+        // additions alone is fused with them, its rounding lost, whatever its .rn
+        const unsigned long long p = fma2(e.w, v, 0x8000000080000000ull);  // + (-0, -0)
+        const unsigned long long em = fma2(e.neg, v, p);                   // p - w v
         const unsigned long long ns = add2(s, p);
         const unsigned long long z = sub2(ns, s);
         const unsigned long long es = add2(sub2(s, sub2(ns, z)), sub2(p, z));
         s = ns;
-        c = add2(c, add2(ep, es));
+        c = add2(c, sub2(es, em));
     }
     __device__ __forceinline__ void split(Acc<float>& a, Acc<float>& b) const {
         a.s = __uint_as_float((unsigned)s);

@@ -40,3 +40,20 @@ def test_full_pattern_residual(N, prec):
     bar = 8 * (N + 1) * 2.0**-53 * 2.0 if prec == kc.FP64 else 2.0**-24 * 2.0 * 8
     assert float((L @ L.T - A).abs().max()) <= bar
     assert np.allclose(diag.cpu().numpy(), L.diagonal().cpu().numpy(), rtol=2.0**-23, atol=0)
+
+
+@pytest.mark.parametrize("seed", [411, 412, 413])
+def test_compensated_sums_do_not_depend_on_their_split(seed):
+    """FP32 form, 8 and 32 lanes a row: the sums of at most 64 products agree to
+    about 64 u^2, so the stored entries round alike but for one in 2^16; sums
+    without the compensation would differ in a large part of them."""
+    N = 64
+    x = torch.from_numpy(inputs.uniform(N, 3, seed=seed)).to(DEV)
+    n = torch.arange(N, device=DEV)
+    rowptr = torch.cat([torch.zeros(1, dtype=torch.int64, device=DEV), torch.cumsum(n + 1, 0)])
+    _, col = torch.tril_indices(N, N, device=DEV)
+    pat = kc.schedule(rowptr, col.to(torch.int32), x)
+    kern = kc.Kernel(0.5, 0.5, 1.0, 0.01)
+    a, _, _ = kc.factor_blocked(pat, x, kern, kc.FP32_FORM)
+    b, _, _ = kc.factor_blocked(pat, x, kern, kc.FP32_FORM, opts=kc.kc_opts(lanes_per_row=32))
+    assert float((a != b).double().mean()) <= 0.01
