@@ -19,7 +19,7 @@
 // p its value is already below d2(p,q).
 //
 // Rounds run in bands of keys: with vmax the largest undecided v, the band
-// holds the undecided points with v >= vmax/4 (KC_ORDER_BAND); only band points can dominate
+// holds the undecided points with v >= KC_ORDER_BAND vmax; only band points can dominate
 // band points, so the dominance search uses a grid of band points with cells of
 // a quarter of sqrt(vmax) (more where the points are too few for that), whose
 // largest points alone are searched for where a cell holds several.  The updates
@@ -28,10 +28,10 @@
 //
 // Bound by latency: about 50 rounds of dependent scans, each between grid
 // barriers.  Measured (before: a dozen launches and two waits of the host per
-// round): 2^20 points of a jittered grid 16.0 -> 12.2 ms, 250,007 points of a
-// swiss roll in R^20 22.4 -> 18.6 (34 -> 18.7 in a process that has used many
-// streams, where every launch costs more), 131,071 points of the cube 13.3 ->
-// 9.5, 100,003 in the square 9.2 -> 5.8, 2000 4.6 -> 1.7.
+// round): 2^20 points of a jittered grid 16.0 -> 8.4 ms, 250,007 points of a
+// swiss roll in R^20 22.4 -> 16.2 (34 in a process that has used many streams,
+// where every launch costs more), 131,071 points of the cube 13.3 -> 7.6, 100,003
+// in the square 9.2 -> 3.7, 2000 4.6 -> 1.2.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -108,6 +108,7 @@ struct BandArgs {
     double* wd;                         // and its squared distance
     int* part;                          // scan: one sum per block
     struct BandCtl* ctl;
+    unsigned* flags;  // of the grid barrier
     double lo[3], hi[3];
     long long limit;
 };
@@ -116,7 +117,7 @@ struct BandCtl {
     unsigned long long vmax[2];
     unsigned open[2], nb[2], occ[2];
     unsigned nsel[3], nact[3], nhard[3];
-    unsigned bar, gen;
+    unsigned bar;
     int status, rounds;
 };
 
@@ -348,15 +349,18 @@ __device__ __forceinline__ unsigned list_slot(unsigned* n) {
 }
 
 // ---- greedy steps for the coarsest points: each step selects the argmax of
-// the previous step's per-block candidates and pushes it to every point.
+// the previous step's per-block candidates and pushes it to the points near it.
+// 64, 96, 128, 256 and 512 of them: 10.1, 9.0, 9.0, 9.35 and 9.5 ms for the ordering
+// of 2^20 points, 3.52, 3.53, 3.49, 3.70 and 4.0 for the path of 2000 (all at a
+// band of 0.25; at 0.16 and 128 steps 8.8 and 3.43, at 0.4 9.0 and 3.75).
 constexpr int GREEDY_THREADS = 1024;
 #ifndef KC_GREEDY_STEPS
-#define KC_GREEDY_STEPS 256
+#define KC_GREEDY_STEPS 128
 #endif
 constexpr int64_t GREEDY_STEPS = KC_GREEDY_STEPS;  // coarsest points selected one at a time
 // A band holds the undecided points with v >= KC_ORDER_BAND * (largest v).
 #ifndef KC_ORDER_BAND
-#define KC_ORDER_BAND 0.25
+#define KC_ORDER_BAND 0.16
 #endif
 
 // the better of two candidates (v2 desc, original index asc; g < 0: none)
@@ -378,34 +382,38 @@ struct Cand {
             take(__shfl_xor_sync(0xffffffffu, v, o), __shfl_xor_sync(0xffffffffu, i, o), __shfl_xor_sync(0xffffffffu, g, o));
     }
 };
-// A grid-wide barrier for a cooperative launch (every block resident): the
-// last block to arrive resets the count and advances the generation; the
-// others poll the generation with backoff, at most `limit` cycles, after
-// which (or when another block has failed) the status word is set and false
-// returned.
-__device__ bool grid_barrier(unsigned* count, unsigned* gen, int* status, long long limit) {
-    __shared__ int ok;
+// A grid-wide barrier for a cooperative launch (every block resident).  Blocks
+// arrive at one counter, which only grows; the last of a phase tells every block
+// at a word in a sector of its own (a single word that all poll was slower:
+// 10.6 against 9.35 ms for the ordering of 2^20 points, 25.4 against 24.6 for
+// the 250,007 of a swiss roll).  A wait is at most `limit` cycles; after that, or when
+// another block has failed, the status word is set and false returned.
+// `phase`: the barriers passed so far, kept by the caller (all threads).
+constexpr int BAR_STRIDE = 8;  // words between the blocks' flags
+__device__ bool grid_barrier(unsigned* count, unsigned* flags, unsigned& phase, int* status, long long limit) {
+    __shared__ int ok, last;
     __syncthreads();
+    ++phase;
     if (threadIdx.x == 0) {
         ok = 1;
-        const unsigned g = ld_acquire_u32(gen);
         fence_acq_rel_gpu();  // this block's writes before its arrival
-        if (atomicAdd(count, 1u) == gridDim.x - 1) {
-            *count = 0u;
-            fence_acq_rel_gpu();
-            red_release_add_u32(gen, 1u);
-        } else {
-            const long long t0 = clock64();
-            unsigned ns = 32;
-            while (ld_acquire_u32(gen) == g) {
-                if (clock64() - t0 > limit || ld_volatile_s32(status) != 0) {
-                    atomicCAS(status, 0, DEV_TIMEOUT);
-                    ok = 0;
-                    break;
-                }
-                __nanosleep(ns);
-                if (ns < 256) ns <<= 1;
+        last = atomicAdd(count, 1u) == phase * gridDim.x - 1u;
+        fence_acq_rel_gpu();  // acquire (the last block): the others' writes
+    }
+    __syncthreads();
+    if (last) {
+        for (unsigned b = threadIdx.x; b < gridDim.x; b += blockDim.x)
+            asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(flags + b * BAR_STRIDE), "r"(phase) : "memory");
+    } else if (threadIdx.x == 0) {
+        const unsigned* mine = flags + blockIdx.x * BAR_STRIDE;
+        const long long t0 = clock64();
+        for (int poll = 1; ld_acquire_u32(mine) != phase; ++poll) {
+            if (clock64() - t0 > limit || ((poll & 63) == 0 && ld_volatile_s32(status) != 0)) {
+                atomicCAS(status, 0, DEV_TIMEOUT);
+                ok = 0;
+                break;
             }
+            if (poll > 8) __nanosleep(32);
         }
         fence_acq_rel_gpu();  // acquire: the other blocks' writes
     }
@@ -603,7 +611,8 @@ __global__ void __launch_bounds__(256, 4) ord_bands_k(BandArgs A) {
     const int lane = lane_id();
     const int64_t warp = tid >> 5, nw = nt >> 5;
     const bool first = tid == 0;
-    auto barrier = [&]() { return grid_barrier(&C->bar, &C->gen, &C->status, A.limit); };
+    unsigned phase = 0;
+    auto barrier = [&]() { return grid_barrier(&C->bar, A.flags, phase, &C->status, A.limit); };
     int round = 0;
     for (int band = 0;; ++band) {
         const int bp = band & 1;
@@ -1042,6 +1051,8 @@ kc_status order_impl(const double* x, int64_t N, int d, int32_t* perm, double* l
         // a block per 256 points (few blocks keep the barriers short), at most what is resident at once
         const int nblk = (int)std::min<int64_t>((int64_t)sms * std::max(1, per_sm), (N + 255) / 256);
         KC_TRY(A.get(&a.part, nblk));
+        KC_TRY(A.get(&a.flags, nblk * BAR_STRIDE));
+        KC_CUDA(cudaMemsetAsync(a.flags, 0, sizeof(unsigned) * nblk * BAR_STRIDE, s));
         void* args[] = {(void*)&a};
         ::kc::note_launch();
         KC_CUDA(cudaLaunchCooperativeKernel((const void*)ord_bands_k, dim3(nblk), dim3(256), args, 0, s));

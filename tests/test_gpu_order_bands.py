@@ -30,7 +30,9 @@ def int_grid(side, d, seed):
 
 
 CASES = [
-    ("uniform257", lambda: inputs.uniform(257, 2, seed=1)),  # one band round after 256 greedy steps
+    ("uniform129", lambda: inputs.uniform(129, 2, seed=21)),  # the greedy steps select all but the first
+    ("uniform130", lambda: inputs.uniform(130, 2, seed=22)),  # one point is left to a band
+    ("uniform257", lambda: inputs.uniform(257, 2, seed=1)),
     ("uniform258", lambda: inputs.uniform(258, 2, seed=2)),
     ("uniform4096", lambda: inputs.uniform(4096, 2, seed=3)),
     ("uniform4097", lambda: inputs.uniform(4097, 2, seed=4)),
