@@ -9,10 +9,10 @@
 //
 // Column-centric search: column i looks at the points within rho*l[i] of
 // x_i (a superset for the min rule) through a fine grid of all points, one
-// warp per (column, row of grid cells); the points of consecutive cells are
-// contiguous in the cell-sorted order.  A count pass gives the row lengths,
-// a fill pass scatters the column indices with atomics, and a sort of each
-// row (bitonic, in shared memory) restores ascending order.
+// warp (half a warp in the builder) per (column, row of grid cells); the points
+// of consecutive cells are contiguous in the cell-sorted order.  A count pass
+// gives the row lengths, a fill pass scatters the column indices with atomics,
+// and a sort of each row (bitonic, in registers) restores ascending order.
 #include <cmath>
 
 #include "grid.cuh"
