@@ -376,8 +376,8 @@ __device__ __forceinline__ bool task_stage(const FactorArgs<T>& A, const Team<TE
 #pragma unroll
             for (int u = 0; u < DEPS; ++u)
                 if (kk[u] >= 0) sq.add(vv[u], vv[u]);
-            if (!ok) break;
         }
+        if (!ok) break;  // (a later round's wait must not hide it)
     }
     if constexpr (TEAM) {
         if (!ok || !placed) atomicOr(&tm.ctl->bad, ok ? 2 : 1);
