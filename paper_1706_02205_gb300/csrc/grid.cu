@@ -322,7 +322,9 @@ static void jacobi_eigen(int d, double* a, double* v) {
     }
 }
 
-kc_status grid_coords(const double* x, int64_t N, int d, Arena& A, cudaStream_t s, const double** gx, int* gs) {
+kc_status grid_coords(const double* x, int64_t N, int d, Arena& A, cudaStream_t s, const double** gx, int* gs,
+                      double* beyond) {
+    if (beyond) *beyond = 0.0;
     if (d <= 3) {
         *gx = x;
         *gs = d;
@@ -355,6 +357,15 @@ kc_status grid_coords(const double* x, int64_t N, int d, Arena& A, cudaStream_t 
         for (int k = 0; k < d; ++k) nrm += vec[k * d + idx[t]] * vec[k * d + idx[t]];
         nrm = std::sqrt(nrm);  // 1 up to rounding; renormalised so |v_t| <= 1 holds
         for (int k = 0; k < MAXD; ++k) ax.v[t][k] = k < d ? vec[k * d + idx[t]] / (nrm * (1.0 + 1e-14)) : 0.0;
+    }
+    if (beyond) {
+        double all = 0.0, rest = 0.0;
+        for (int i = 0; i < d; ++i) {
+            const double c = std::max(0.0, cov[idx[i] * d + idx[i]]);
+            all += c;
+            if (i >= 3) rest += c;
+        }
+        if (all > 0.0) *beyond = rest / all;
     }
     double* out;
     KC_TRY(A.get(&out, (size_t)N * 3));

@@ -119,7 +119,9 @@ kc_status bbox(const double* x, int64_t N, int d, double* lo, double* hi, Arena&
 // by no more than their distance and every search box stays exact; for data
 // near a low-dimensional subspace they keep the boxes as tight as the data
 // (the first three raw coordinates are an arbitrary projection of it).
-kc_status grid_coords(const double* x, int64_t N, int d, Arena& A, cudaStream_t s, const double** gx, int* gs);
+// *beyond: the share of the points' variance outside these axes (0 for d <= 3).
+kc_status grid_coords(const double* x, int64_t N, int d, Arena& A, cudaStream_t s, const double** gx, int* gs,
+                      double* beyond = nullptr);
 
 // Bounding box over all d <= 32 axes (host out; the low corner also for the float
 // copies used by the FP32 distance screens); E = the largest extent.  KC_EINVAL if

@@ -29,9 +29,11 @@
 // Bound by latency: about 50 rounds of dependent scans, each between grid
 // barriers.  Measured (before: a dozen launches and two waits of the host per
 // round): 2^20 points of a jittered grid 16.0 -> 8.4 ms, 250,007 points of a
-// swiss roll in R^20 22.4 -> 16.2 (34 in a process that has used many streams,
+// swiss roll in R^20 22.4 -> 15.6 (34 in a process that has used many streams,
 // where every launch costs more), 131,071 points of the cube 13.3 -> 7.6, 100,003
-// in the square 9.2 -> 3.7, 2000 4.6 -> 1.2.
+// in the square 9.2 -> 3.7, 2000 4.6 -> 1.2; 60,000 points of the cube in R^20 320 ->
+// 256, 100,003 in R^8 154 -> 147, 5000 in R^20 16.1 -> 10.7; 100,000 points with heavy
+// tails (most of them in a few cells) 1170 -> 1155.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -50,6 +52,27 @@ __global__ void gather_rows_k(const double* __restrict__ a, int w, const int32_t
         for (int t = 0; t < w; ++t) out[q * w + t] = a[(int64_t)ids[q] * w + t];
 }
 
+// Floats of a point's row of the float copy: past three axes rows are filled up
+// with zeros to whole 16 bytes, so that a screen reads them by 16-byte loads
+// (a warp's 32 rows by single floats take a trip to L1 per float and line).
+__host__ __device__ __forceinline__ int row_floats(int d) { return d <= 3 ? d : (d + 3) & ~3; }
+// screen_f32 on such rows (HIGH: d > 3): the same sum (the filling adds zeros) and decision
+template <bool HIGH>
+__device__ __forceinline__ int screen_rows(const float* a, const float* b, int d, float Rf, float delta) {
+    if constexpr (!HIGH) return screen_f32(a, b, d, Rf, delta);
+    float s = 0.f;
+    for (int t = 0; t < d; t += 4) {
+        const float4 u = *(const float4*)(a + t), v = *(const float4*)(b + t);
+        const float w0 = u.x - v.x, w1 = u.y - v.y, w2 = u.z - v.z, w3 = u.w - v.w;
+        s = fmaf(w3, w3, fmaf(w2, w2, fmaf(w1, w1, fmaf(w0, w0, s))));
+    }
+    const float dist = sqrtf(s);
+    const float M = sqrtf((float)d) * delta + (float)(d + 6) * 1.1920929e-7f * fmaxf(dist, Rf);
+    if (dist - M > Rf) return 0;
+    if (dist + M < Rf) return 1;
+    return -1;
+}
+
 // state in grid order (gpos): coordinates xg, original index idg, v2, stat
 __global__ void ord_init_k(const double* __restrict__ x, int d, const int32_t* __restrict__ gsorted, int64_t N,
                            double* __restrict__ xg, int32_t* __restrict__ idg, double* __restrict__ v2,
@@ -57,10 +80,12 @@ __global__ void ord_init_k(const double* __restrict__ x, int d, const int32_t* _
     int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= N) return;
     int64_t id = gsorted[q];
+    const int df = row_floats(d);
     for (int t = 0; t < d; ++t) {
         xg[q * d + t] = x[id * d + t];
-        if (xgf) xgf[q * d + t] = (float)(x[id * d + t] - org.lo[t]);
+        xgf[q * df + t] = (float)(x[id * d + t] - org.lo[t]);
     }
+    for (int t = d; t < df; ++t) xgf[q * df + t] = 0.f;
     idg[q] = (int32_t)id;
     if (id == 0) {
         v2[q] = INFINITY;
@@ -84,13 +109,15 @@ __device__ __forceinline__ bool key_above(double va, int ia, double vb, int ib) 
 #define KC_DOM_BUDGET 32
 #endif
 constexpr int DOM_THREAD_BUDGET = KC_DOM_BUDGET;
+// Candidates of the first look of points in more than three dimensions (below).
+constexpr int LIST_BUDGET = 16;
 
 // What the band rounds read and write.  v2 and stat change between the phases of
 // one launch: they go without __restrict__, so that they are never read through
 // the non-coherent path.
 struct BandArgs {
     int64_t N;
-    int d, gs;
+    int d, gs, df;                      // df: floats of a row of xgf
     Grid g0;                            // fine grid of all points
     const int64_t* __restrict__ cstart;  // its cells
     const double* __restrict__ xg;      // coordinates in grid order
@@ -116,7 +143,7 @@ struct BandArgs {
 struct BandCtl {
     unsigned long long vmax[2];
     unsigned open[2], nb[2], occ[2];
-    unsigned nsel[3], nact[3], nhard[3];
+    unsigned nsel[3], nact[3], nhard[3], nlong[3];
     unsigned bar;
     int status, rounds;
 };
@@ -180,10 +207,11 @@ __device__ __forceinline__ int span_of_v(const Grid& g, double v, float inv_c, i
 
 // Does the undecided band point p dominate q (larger key, closer than sqrt(vq))?
 // Its squared distance if it does, else infinity.
+template <bool HIGH>
 __device__ __forceinline__ double dominates(const BandArgs& A, int p, int q, double vq, float rq, int idq) {
     if (p == q || A.stat[p] != 0) return INFINITY;
     if (!key_above(A.v2[p], A.idg[p], vq, idq)) return INFINITY;
-    if (screen_f32(A.xgf + (int64_t)p * A.d, A.xgf + (int64_t)q * A.d, A.d, rq, A.delta) == 0) return INFINITY;
+    if (screen_rows<HIGH>(A.xgf + (int64_t)p * A.df, A.xgf + (int64_t)q * A.df, A.d, rq, A.delta) == 0) return INFINITY;
     const double dd = dist2_exact(A.xg + (int64_t)p * A.d, A.xg + (int64_t)q * A.d, A.d);
     return dd < vq ? dd : INFINITY;
 }
@@ -194,7 +222,9 @@ __device__ __forceinline__ double dominates(const BandArgs& A, int p, int q, dou
 // (ring r holds no point closer than (r-1) cells).  It gives up (-2) when the
 // scan would go past DOM_THREAD_BUDGET candidates: an undominated point has to look at every band point within sqrt(v), which is a
 // warp's work.
-__device__ __forceinline__ int dominator_thread(const BandArgs& A, const Grid& gb, int q, double vq, double& wd) {
+template <bool HIGH>
+__device__ __forceinline__ int dominator_thread(const BandArgs& A, const Grid& gb, int q, double vq, int budget,
+                                                double& wd) {
     const long long bq = vbits(vq);
     const float rq = sqrtf((float)vq);
     const int idq = A.idg[q];
@@ -206,7 +236,6 @@ __device__ __forceinline__ int dominator_thread(const BandArgs& A, const Grid& g
         c[t] = cell_coord(gb, A.gxg[(int64_t)q * A.gs + t], t);
         maxr = max(maxr, span_for(gb, R, t));
     }
-    int budget = DOM_THREAD_BUDGET;
     for (int r = 0; r <= maxr; ++r) {
         if (r >= 2 && (double)(r - 1) * gb.c > R) break;
         const int z0 = dg > 2 ? max(0, c[2] - r) : 0, z1 = dg > 2 ? min(gb.n[2] - 1, c[2] + r) : 0;
@@ -225,7 +254,7 @@ __device__ __forceinline__ int dominator_thread(const BandArgs& A, const Grid& g
                     budget -= f1 - f0;
                     for (int f = f0; f < f1; ++f) {
                         const int p = A.bsorted[f];
-                        const double dd = dominates(A, p, q, vq, rq, idq);
+                        const double dd = dominates<HIGH>(A, p, q, vq, rq, idq);
                         if (dd < vq) {
                             wd = dd;
                             return p;
@@ -249,7 +278,7 @@ __device__ __forceinline__ int which_row(int inc, int m) {
 
 // The same by a warp, a lane per cell of the box around q.  (With the warp on
 // one cell at a time the cells of a box were a chain of dependent loads.)
-template <bool DENSE>
+template <bool HIGH, bool DENSE>
 __device__ __forceinline__ int dominator_warp(const BandArgs& A, const Grid& gb, int q, double vq, double& wd) {
     constexpr int SCAN = 4;
     const unsigned FULL = 0xffffffffu;
@@ -265,6 +294,9 @@ __device__ __forceinline__ int dominator_warp(const BandArgs& A, const Grid& gb,
         n[t] = min(gb.n[t] - 1, c + sp) - lo[t] + 1;
     }
     const int cells = n[0] * n[1] * n[2];
+    int own = 0;
+    if constexpr (HIGH)
+        for (int t = gb.dg - 1; t >= 0; --t) own = own * n[t] + cell_coord(gb, A.gxg[(int64_t)q * A.gs + t], t) - lo[t];
     auto cell_at = [&](int t) {
         const int row = t / n[0];
         return ((int64_t)(lo[2] + row / n[1]) * gb.n[1] + lo[1] + row % n[1]) * gb.n[0] + lo[0] + t % n[0];
@@ -277,7 +309,7 @@ __device__ __forceinline__ int dominator_warp(const BandArgs& A, const Grid& gb,
                 const int64_t cell = cell_at(t0 + lane);
                 if (A.cmax[cell] >= bq) {
                     p = A.champ[cell];  // there is one: its value is at least vq, so at least T
-                    dd = dominates(A, p, q, vq, rq, idq);
+                    dd = dominates<HIGH>(A, p, q, vq, rq, idq);
                 }
             }
             const unsigned hits = __ballot_sync(FULL, dd < vq);
@@ -292,7 +324,8 @@ __device__ __forceinline__ int dominator_warp(const BandArgs& A, const Grid& gb,
     for (int t0 = 0; t0 < cells; t0 += 32) {
         int f0 = 0, len = 0;
         if (t0 + lane < cells) {
-            const int64_t cell = cell_at(t0 + lane);
+            const int t = t0 + lane + own;
+            const int64_t cell = cell_at(t < cells ? t : t - cells);
             if (A.cmax[cell] >= bq) {
                 f0 = A.bstart[cell];
                 len = A.bstart[cell + 1] - f0;
@@ -318,15 +351,15 @@ __device__ __forceinline__ int dominator_warp(const BandArgs& A, const Grid& gb,
             int st[SCAN];
 #pragma unroll
             for (int u = 0; u < SCAN; ++u) {
-                v[u] = p[u] >= 0 ? A.v2[p[u]] : 0.0;
                 st[u] = p[u] >= 0 ? A.stat[p[u]] : 1;
+                v[u] = p[u] >= 0 ? A.v2[p[u]] : 0.0;
             }
             double dd = INFINITY;
             int hit = -1;
 #pragma unroll
             for (int u = 0; u < SCAN; ++u)
                 if (hit < 0 && st[u] == 0 && vbits(v[u]) >= bq) {
-                    dd = dominates(A, p[u], q, vq, rq, idq);
+                    dd = dominates<HIGH>(A, p[u], q, vq, rq, idq);
                     if (dd < vq) hit = p[u];
                 }
             const unsigned hits = __ballot_sync(FULL, hit >= 0);
@@ -358,6 +391,13 @@ constexpr int GREEDY_THREADS = 1024;
 #define KC_GREEDY_STEPS 128
 #endif
 constexpr int64_t GREEDY_STEPS = KC_GREEDY_STEPS;  // coarsest points selected one at a time
+// Where a twentieth of the variance lies outside the grid's three axes (a cube of
+// four dimensions has a quarter there, a noisy sheet next to nothing), the grid
+// prunes little and the first rounds look at nearly all pairs: more steps then.
+// 128, 512, 1024 and 2048 of them: 160, 149, 141 and 124 ms for 100,003 points of
+// the cube in R^8, 11.8, 10.8, 12.2 and 16.5 for 5000 in R^20, 18.5, 14.6, 14.7 and
+// 17.5 for 100,003 in R^4; 15.7, 17.6, 19.9 and 26.3 for 250,007 of a swiss roll.
+constexpr int64_t GREEDY_STEPS_SPREAD = 512;
 // A band holds the undecided points with v >= KC_ORDER_BAND * (largest v).
 #ifndef KC_ORDER_BAND
 #define KC_ORDER_BAND 0.16
@@ -470,6 +510,7 @@ __device__ __forceinline__ float float_below(unsigned long long v) {
 // A step took 14.6 us at 2^20 points and 7.4 at 2000 with a grid barrier and 608
 // blocks, 10.9 and 3.1 with the slots but every point looked at and FP64
 // compares, and 4.8 and 2.1 now.
+template <bool HIGH>
 __global__ void __launch_bounds__(GREEDY_THREADS, 1)
     ord_greedy_loop_k(const double* __restrict__ xg, int d, const int32_t* __restrict__ idg, double* v2, int* stat,
                       int64_t N, int64_t steps, ulonglong2* slots, const float* __restrict__ xgf, float delta,
@@ -483,7 +524,7 @@ __global__ void __launch_bounds__(GREEDY_THREADS, 1)
     const int64_t per = 32 * ((N + 1024 * nw - 1) / (1024 * nw)), ns = (N + per - 1) / per;
     const int64_t gw = (int64_t)wrp * nblk + blockIdx.x;
     const int mine = ns > gw ? (int)((ns - gw + nw - 1) / nw) : 0;  // the warp's stretches, at most 32
-    const int da = min(d, 3);
+    const int da = min(d, 3), df = row_floats(d);
     float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};  // box, first three axes
     for (int j = 0; j < mine; ++j) {
         const int64_t q0 = (gw + j * nw) * per, q1 = min(N, q0 + per);
@@ -492,7 +533,7 @@ __global__ void __launch_bounds__(GREEDY_THREADS, 1)
             if (t < da) {
                 float a = INFINITY, b = -INFINITY;
                 for (int64_t q = q0 + lane; q < q1; q += 32) {
-                    const float u = xgf[q * d + t];
+                    const float u = xgf[q * df + t];
                     a = fminf(a, u);
                     b = fmaxf(b, u);
                 }
@@ -518,7 +559,7 @@ __global__ void __launch_bounds__(GREEDY_THREADS, 1)
 #pragma unroll
             for (int t = 0; t < 3; ++t)
                 if (t < da) {
-                    const float u = xgf[w * d + t];
+                    const float u = xgf[w * df + t];
                     const float g = fmaxf(lo[t] - u, u - hi[t]) * (1.f - 1e-6f) - delta;
                     if (g > 0.f) s = fmaf(g, g, s);
                 }
@@ -533,7 +574,7 @@ __global__ void __launch_bounds__(GREEDY_THREADS, 1)
                 const int at = idg[q];
                 if (q == w) stat[q] = 1;  // v2[w] keeps its final value l^2
                 if (q == w || stat[q] != 0) continue;
-                if (w >= 0 && screen_f32(xgf + q * d, xgf + w * d, d, sqrtf(float_below(vq)), delta) != 0) {
+                if (w >= 0 && screen_rows<HIGH>(xgf + q * df, xgf + w * df, d, sqrtf(float_below(vq)), delta) != 0) {
                     const double dd = dist2_exact(xg + q * d, xg + w * d, d);
                     const unsigned long long u = (unsigned long long)__double_as_longlong(dd);
                     if (u < vq) {
@@ -600,6 +641,10 @@ __global__ void __launch_bounds__(GREEDY_THREADS, 1)
 // All bands and their rounds in one cooperative launch, a grid barrier between
 // the phases: the host waits once, where it used to wait three times per band
 // and twice per round, around a dozen launches each.
+//
+// HIGH: more than three dimensions.  (Registers for three blocks an SM without most of
+// the spills: 329.8 against 305.0 ms for 60,000 points of the cube in R^20.)
+template <bool HIGH>
 __global__ void __launch_bounds__(256, 4) ord_bands_k(BandArgs A) {
     __shared__ int wsum[8];
     __shared__ int carry;
@@ -756,7 +801,7 @@ __global__ void __launch_bounds__(256, 4) ord_bands_k(BandArgs A) {
                             if (p == best.g || A.stat[p] != 0) continue;
                             const double vp = A.v2[p];
                             if (!(vp >= T)) continue;
-                            const int sc = screen_f32(A.xgf + (int64_t)p * A.d, A.xgf + (int64_t)best.g * A.d, A.d,
+                            const int sc = screen_rows<HIGH>(A.xgf + (int64_t)p * A.df, A.xgf + (int64_t)best.g * A.df, A.d,
                                                       sqrtf((float)vp), A.delta);
                             if (sc > 0) continue;
                             if (sc == 0 || !(dist2_exact(A.xg + (int64_t)p * A.d, A.xg + (int64_t)best.g * A.d, A.d) < vp))
@@ -791,7 +836,7 @@ __global__ void __launch_bounds__(256, 4) ord_bands_k(BandArgs A) {
                 const int w0 = A.wit[q];
                 if (w0 >= 0 && A.stat[w0] == 0 && A.wd[q] < vq && key_above(A.v2[w0], A.idg[w0], vq, A.idg[q])) continue;
                 double wd = 0.0;
-                const int k = dominator_thread(A, gb, q, vq, wd);
+                const int k = dominator_thread<HIGH>(A, gb, q, vq, DOM_THREAD_BUDGET, wd);
                 if (k == -1) A.sel[list_slot(&C->nsel[rp])] = q;
                 else if (k == -2) A.hard[list_slot(&C->nhard[rp])] = q;
                 else {
@@ -804,11 +849,36 @@ __global__ void __launch_bounds__(256, 4) ord_bands_k(BandArgs A) {
                 if (!barrier()) return;
             }
             if (*(volatile unsigned*)&C->nact[rp] == 0u) break;  // band exhausted
-            const int64_t nh = *(volatile unsigned*)&C->nhard[rp];
+            int64_t nh = *(volatile unsigned*)&C->nhard[rp];
+            const int32_t* left = A.hard;
+            if (HIGH && dense && nh > nw) {
+                // More points left than warps: a thread each looks at the nearest few
+                // candidates first.  Where points spread over many dimensions, their cells
+                // hold points that are far apart, so few are dominated by their cell's
+                // largest one, but most by one of the next few; a warp a point spent
+                // 843 of the 990 ms of 60,000 points in the cube of R^20 on them.
+                for (int64_t e = tid; e < nh; e += nt) {
+                    const int q = A.hard[e];
+                    const double vq = A.v2[q];
+                    const int w0 = A.wit[q];
+                    if (w0 >= 0 && A.stat[w0] == 0 && A.wd[q] < vq && key_above(A.v2[w0], A.idg[w0], vq, A.idg[q])) continue;
+                    double wd = 0.0;
+                    const int k = dominator_thread<HIGH>(A, gb, q, vq, LIST_BUDGET, wd);
+                    if (k == -1) A.sel[list_slot(&C->nsel[rp])] = q;
+                    else if (k == -2) A.blist[list_slot(&C->nlong[rp])] = q;
+                    else {
+                        A.wit[q] = k;
+                        A.wd[q] = wd;
+                    }
+                }
+                if (!barrier()) return;
+                nh = *(volatile unsigned*)&C->nlong[rp];
+                left = A.blist;
+            }
             auto scan = [&](int q) {
                 double wd = 0.0;
                 const double vq = A.v2[q];
-                const int k = dense ? dominator_warp<true>(A, gb, q, vq, wd) : dominator_warp<false>(A, gb, q, vq, wd);
+                const int k = dense ? dominator_warp<HIGH, true>(A, gb, q, vq, wd) : dominator_warp<HIGH, false>(A, gb, q, vq, wd);
                 if (lane == 0) {
                     if (k == -1) {
                         A.sel[atomicAdd(&C->nsel[rp], 1u)] = q;
@@ -825,7 +895,7 @@ __global__ void __launch_bounds__(256, 4) ord_bands_k(BandArgs A) {
                     for (unsigned m = __ballot_sync(0xffffffffu, mine >= 0); m; m &= m - 1)
                         scan(__shfl_sync(0xffffffffu, mine, __ffs(m) - 1));
                 }
-            for (int64_t e = warp; e < nh; e += nw) scan(A.hard[e]);
+            for (int64_t e = warp; e < nh; e += nw) scan(left[e]);
             if (!barrier()) return;
             // lower v2 of the undecided points of smaller key around every selected point: W
             // warps a point.  A point selected in this
@@ -838,9 +908,10 @@ __global__ void __launch_bounds__(256, 4) ord_bands_k(BandArgs A) {
             }
             if (first) {
                 const int nx = (round + 1) % 3;
-                C->nsel[nx] = C->nact[nx] = C->nhard[nx] = 0u;
+                C->nsel[nx] = C->nact[nx] = C->nhard[nx] = C->nlong[nx] = 0u;
                 C->rounds = round + 1;
             }
+            constexpr int UPD = 2;
             const int64_t W = max((int64_t)1, min((int64_t)64, nw / ns));
             for (int64_t u = warp; u < ns * W; u += nw) {
                 const int p = A.sel[u / W];
@@ -883,21 +954,53 @@ __global__ void __launch_bounds__(256, 4) ord_bands_k(BandArgs A) {
                         if (lane >= o) inc += up;
                     }
                     const int total = __shfl_sync(0xffffffffu, inc, 31);
-                    for (int m0 = 0; m0 < total; m0 += 32) {
-                        const int m = m0 + lane;
-                        const int row = which_row(inc, m);
-                        const int64_t ra = __shfl_sync(0xffffffffu, a, row);
-                        const int rs = __shfl_sync(0xffffffffu, inc - len, row);
-                        if (m >= total) continue;
-                        const int64_t q = ra + (m - rs);
-                        if (A.stat[q] != 0) continue;
-                        const double vq = A.v2[q];
-                        if (!(vq < vp || (vq == vp && A.idg[q] > idp))) continue;
-                        if (screen_f32(A.xgf + q * A.d, A.xgf + (int64_t)p * A.d, A.d, sqrtf((float)vq), A.delta) == 0)
-                            continue;
-                        const double dd = dist2_exact(A.xg + q * A.d, xp, A.d);
-                        if (dd < vq)
-                            atomicMin((unsigned long long*)A.v2 + q, (unsigned long long)__double_as_longlong(dd));
+                    // UPD points a lane, places at[] (-1: none), so that their loads overlap (one at a
+                    // time: 1238 against 1152 ms for 100,000 points with heavy tails, whose grid has
+                    // most points in a few cells)
+                    auto lower = [&](const int64_t (&at)[UPD]) {
+                        int st[UPD];
+                        double v[UPD];
+#pragma unroll
+                        for (int u = 0; u < UPD; ++u) {
+                            st[u] = at[u] >= 0 ? A.stat[at[u]] : 1;
+                            v[u] = at[u] >= 0 ? A.v2[at[u]] : 0.0;
+                        }
+#pragma unroll
+                        for (int u = 0; u < UPD; ++u) {
+                            const int64_t q = at[u];
+                            const double vq = v[u];
+                            if (st[u] != 0 || !(vq < vp || (vq == vp && A.idg[q] > idp))) continue;
+                            if (screen_rows<HIGH>(A.xgf + q * A.df, A.xgf + (int64_t)p * A.df, A.d, sqrtf((float)vq), A.delta) == 0)
+                                continue;
+                            const double dd = dist2_exact(A.xg + q * A.d, xp, A.d);
+                            if (dd < vq)
+                                atomicMin((unsigned long long*)A.v2 + q, (unsigned long long)__double_as_longlong(dd));
+                        }
+                    };
+                    if (HIGH && total >= 32 * min(rb, rows - r0)) {  // long rows one by one, without the search
+                        for (int k = 0; k < min(rb, rows - r0); ++k) {
+                            const int64_t ra = __shfl_sync(0xffffffffu, a, k);
+                            const int ln = __shfl_sync(0xffffffffu, len, k);
+                            for (int m = lane; m < ln; m += 32 * UPD) {
+                                int64_t at[UPD];
+#pragma unroll
+                                for (int u = 0; u < UPD; ++u) at[u] = m + 32 * u < ln ? ra + m + 32 * u : -1;
+                                lower(at);
+                            }
+                        }
+                        continue;
+                    }
+                    for (int m0 = 0; m0 < total; m0 += 32 * UPD) {
+                        int64_t at[UPD];
+#pragma unroll
+                        for (int u = 0; u < UPD; ++u) {
+                            const int m = m0 + 32 * u + lane;
+                            const int row = which_row(inc, m);
+                            const int64_t ra = __shfl_sync(0xffffffffu, a, row);
+                            const int rs = __shfl_sync(0xffffffffu, inc - len, row);
+                            at[u] = m < total ? ra + (m - rs) : -1;
+                        }
+                        lower(at);
                     }
                 }
             }
@@ -906,7 +1009,7 @@ __global__ void __launch_bounds__(256, 4) ord_bands_k(BandArgs A) {
         ++round;  // its counters are used: selected none, so they stay as they are
         if (first) {
             const int nx = round % 3;
-            C->nsel[nx] = C->nact[nx] = C->nhard[nx] = 0u;
+            C->nsel[nx] = C->nact[nx] = C->nhard[nx] = C->nlong[nx] = 0u;
         }
     }
 }
@@ -948,7 +1051,8 @@ kc_status order_impl(const double* x, int64_t N, int d, int32_t* perm, double* l
     // grid coordinates: the points (d <= 3) or their principal-axes projections
     const double* gx;
     int gs;
-    KC_TRY(grid_coords(x, N, d, A, s, &gx, &gs));
+    double beyond = 0.0;  // share of the points' variance outside the grid's axes
+    KC_TRY(grid_coords(x, N, d, A, s, &gx, &gs, &beyond));
     double lo[3] = {org.lo[0], org.lo[1], org.lo[2]}, hi[3] = {top.lo[0], top.lo[1], top.lo[2]};
     if (gx != x) KC_TRY(bbox(gx, N, gs, lo, hi, A, s));
     // fine grid of all points, about two points per cell
@@ -971,7 +1075,7 @@ kc_status order_impl(const double* x, int64_t N, int d, int32_t* perm, double* l
     float* xgf = nullptr;
     // 2^-23 E; infinite, so that only exact tests decide, where floats could over- or underflow
     const float delta = E > 1e-12 && E < 1e18 ? (float)(E * 1.1920928955078125e-07) : INFINITY;
-    KC_TRY(A.get(&xgf, N * d));
+    KC_TRY(A.get(&xgf, N * row_floats(d)));
     ::kc::note_launch(), ord_init_k<<<blocks_for(N, 256), 256, 0, s>>>(x, d, gsorted, N, xg, idg, v2, stat, org, xgf);
     // grid coordinates in grid order
     const double* gxg = xg;
@@ -1001,7 +1105,8 @@ kc_status order_impl(const double* x, int64_t N, int d, int32_t* perm, double* l
         ulonglong2* slots;
         KC_TRY(A.get(&slots, 2 * nblk * nblk));
         KC_CUDA(cudaMemsetAsync(slots, 0, sizeof(ulonglong2) * 2 * nblk * nblk, s));
-        int64_t steps = N - 1 < GREEDY_STEPS ? N - 1 : GREEDY_STEPS;
+        const int64_t most = beyond > 0.05 ? GREEDY_STEPS_SPREAD : GREEDY_STEPS;
+        int64_t steps = N - 1 < most ? N - 1 : most;
         const double* a_xg = xg;
         const int32_t* a_idg = idg;
         const float* a_xgf = xgf;
@@ -1010,13 +1115,15 @@ kc_status order_impl(const double* x, int64_t N, int d, int32_t* perm, double* l
         float dl = delta;
         void* args[] = {(void*)&a_xg, (void*)&d, (void*)&a_idg, (void*)&v2, (void*)&stat, (void*)&N, (void*)&steps,
                         (void*)&slots, (void*)&a_xgf, (void*)&dl, (void*)&gst, (void*)&lim};
+        auto gfn = d > 3 ? ord_greedy_loop_k<true> : ord_greedy_loop_k<false>;
         ::kc::note_launch();
-        KC_CUDA(cudaLaunchCooperativeKernel((const void*)ord_greedy_loop_k, dim3(nblk), dim3(GREEDY_THREADS), args, 0, s));
+        KC_CUDA(cudaLaunchCooperativeKernel((const void*)gfn, dim3(nblk), dim3(GREEDY_THREADS), args, 0, s));
     }
     {
         BandArgs a;
         a.N = N;
         a.d = d;
+        a.df = row_floats(d);
         a.gs = gs;
         a.g0 = g0;
         a.cstart = cstart;
@@ -1046,16 +1153,20 @@ kc_status order_impl(const double* x, int64_t N, int d, int32_t* perm, double* l
         KC_TRY(A.get(&a.wit, N));
         KC_TRY(A.get(&a.wd, N));
         KC_CUDA(cudaMemsetAsync(a.wit, 0xff, sizeof(int32_t) * N, s));  // -1
+        auto kfn = d > 3 ? ord_bands_k<true> : ord_bands_k<false>;
         int per_sm = 0;
-        KC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ord_bands_k, 256, 0));
-        // a block per 256 points (few blocks keep the barriers short), at most what is resident at once
-        const int nblk = (int)std::min<int64_t>((int64_t)sms * std::max(1, per_sm), (N + 255) / 256);
+        KC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kfn, 256, 0));
+        // A block per 256 points (few blocks keep the barriers short), at most what is resident
+        // at once.  Past three dimensions a block per 16: a round's scans take longer than its
+        // barriers there (5000 points in R^20: 32.3 ms with a block per 256, 20.7 with one per
+        // 64 or 16; 10,000 of a swiss roll 5.5, 4.8 and 3.1).
+        const int nblk = (int)std::min<int64_t>((int64_t)sms * std::max(1, per_sm), d > 3 ? (N + 15) / 16 : (N + 255) / 256);
         KC_TRY(A.get(&a.part, nblk));
         KC_TRY(A.get(&a.flags, nblk * BAR_STRIDE));
         KC_CUDA(cudaMemsetAsync(a.flags, 0, sizeof(unsigned) * nblk * BAR_STRIDE, s));
         void* args[] = {(void*)&a};
         ::kc::note_launch();
-        KC_CUDA(cudaLaunchCooperativeKernel((const void*)ord_bands_k, dim3(nblk), dim3(256), args, 0, s));
+        KC_CUDA(cudaLaunchCooperativeKernel((const void*)kfn, dim3(nblk), dim3(256), args, 0, s));
         BandCtl h;
         KC_CUDA(cudaMemcpyAsync(&h, ctl, sizeof(h), cudaMemcpyDeviceToHost, s));
         KC_CUDA(cudaStreamSynchronize(s));
