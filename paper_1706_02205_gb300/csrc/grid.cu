@@ -15,7 +15,7 @@ Grid make_grid(int d, const double* lo, const double* hi, int64_t npts, double w
     int nz = 0;
     for (int t = 0; t < g.dg; ++t) {
         g.lo[t] = lo[t];
-        ext[t] = hi[t] - lo[t];
+        ext[t] = hi[t] > lo[t] ? hi[t] - lo[t] : 0.0;
         if (ext[t] > 0) {
             vol *= ext[t];
             nz++;
@@ -28,11 +28,18 @@ Grid make_grid(int d, const double* lo, const double* hi, int64_t npts, double w
         g.inv_c = 1.0;
         return g;
     }
+    // extents whose cells have no finite inverse, or differences of coordinates none: one cell
+    if (!(emax > 1e-290 && emax < 1e300)) {
+        one_cell(g);
+        return g;
+    }
     if (max_cells < 1) max_cells = 1;
     // smallest cell size allowed by the cell budget
     double cmin = nz > 0 ? pow(vol / (double)max_cells, 1.0 / nz) : emax;
     double c = want > 0 ? want : cmin;
     if (c < cmin) c = cmin;
+    // the volume of a very small or flat box underflows: an axis takes at most 1e6 cells
+    if (!(c > 0.0)) c = emax * 1e-6;
     for (;;) {
         int64_t tot = 1;
         bool ok = true;

@@ -17,10 +17,20 @@ struct Grid {
     int64_t ncells = 1;
 };
 
+// A single cell, whatever the coordinates; its size is not known.
+__host__ __device__ inline void one_cell(Grid& g) {
+    for (int t = 0; t < 3; ++t) {
+        g.lo[t] = 0.0;
+        g.n[t] = 1;
+    }
+    g.c = INFINITY;
+    g.inv_c = 0.0;
+    g.ncells = 1;
+}
+
 __device__ __forceinline__ int cell_coord(const Grid& g, double v, int t) {
-    double f = (v - g.lo[t]) * g.inv_c;
-    int q = (f <= 0.0) ? 0 : (f >= (double)(g.n[t] - 1) ? g.n[t] - 1 : (int)f);
-    return q;
+    const double f = (v - g.lo[t]) * g.inv_c;
+    return f >= (double)(g.n[t] - 1) ? g.n[t] - 1 : f > 0.0 ? (int)f : 0;  // (not a number: cell 0)
 }
 __device__ __forceinline__ int64_t cell_of(const Grid& g, const double* x) {
     int64_t key = 0;

@@ -159,7 +159,7 @@ __device__ __noinline__ void band_grid(const BandArgs& A, double vmax, int64_t n
     int nz = 0;
     for (int t = 0; t < g.dg; ++t) {
         g.lo[t] = A.lo[t];
-        ext[t] = A.hi[t] - A.lo[t];
+        ext[t] = A.hi[t] > A.lo[t] ? A.hi[t] - A.lo[t] : 0.0;
         if (ext[t] > 0.0) {
             vol *= ext[t];
             ++nz;
@@ -167,6 +167,10 @@ __device__ __noinline__ void band_grid(const BandArgs& A, double vmax, int64_t n
         emax = fmax(emax, ext[t]);
     }
     if (!(emax > 0.0)) return;
+    if (!(emax > 1e-290 && emax < 1e300)) {
+        one_cell(g);
+        return;
+    }
     const int64_t most = 2 * nb + 1;
     const double q = vol / (double)most;
     double c = nz == 1 ? q : nz == 2 ? sqrt(q) : cbrt(q);
@@ -191,10 +195,7 @@ __device__ __noinline__ void band_grid(const BandArgs& A, double vmax, int64_t n
         }
         c = c > 0.0 ? c * 1.25 : emax * 1e-6;
     }
-    g.n[0] = g.n[1] = g.n[2] = 1;  // a degenerate box: one cell
-    g.ncells = 1;
-    g.c = 2.0 * emax;
-    g.inv_c = 1.0 / g.c;
+    one_cell(g);
 }
 
 // Cells to either side of a point's own that cover sqrt(v) on the grid g, by FP32

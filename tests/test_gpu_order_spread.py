@@ -35,6 +35,13 @@ CASES = [(f"cube{N}_{d}", lambda N=N, d=d: inputs.uniform(N, d, seed=N + d))
 CASES += [(f"slab{b}", lambda b=b: slab(4000, 9, b, 31)) for b in (0.049, 0.051, 0.5)]
 CASES += [("repeated", lambda: np.repeat(inputs.uniform(600, 6, seed=32), 6, axis=0)),
           ("lattice", lambda: inputs.rng(33).integers(0, 4, (3000, 6)).astype(np.float64)),
+          ("tiny3", lambda: inputs.uniform(2500, 3, seed=37) * 1e-160),  # the volume of the box is no double
+          ("tiny7", lambda: inputs.uniform(2500, 7, seed=34) * 1e-160),
+          ("flat", lambda: inputs.uniform(2500, 3, seed=38) * np.array([1e100, 1e-250, 1e-250])),
+          ("smallest", lambda: inputs.rng(39).integers(0, 2, (300, 3)) * 5e-324),  # no cell size has an inverse
+          ("small1", lambda: inputs.uniform(300, 1, seed=40) * 1e-310),
+          ("largest3", lambda: (2 * inputs.uniform(600, 3, seed=41) - 1) * 1.7e308),  # no difference is a double
+          ("largest5", lambda: (2 * inputs.uniform(600, 5, seed=42) - 1) * 1.7e308),
           ("heavy", lambda: np.exp(4 * inputs.rng(35).standard_normal((6000, 2))))]
 
 
