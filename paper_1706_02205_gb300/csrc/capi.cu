@@ -15,7 +15,9 @@ struct NvtxRange {
 #define KC_RANGE(name) NvtxRange kc_nvtx_range_(name)
 
 namespace kc {
-kc_status order_impl(const double* x, int64_t N, int d, int32_t* perm, double* l, double* x_ord, cudaStream_t s);
+constexpr long long ORDER_WAIT_CYCLES = 4000000000LL;  // about 2 s
+kc_status order_impl(const double* x, int64_t N, int d, int32_t* perm, double* l, double* x_ord, long long limit,
+                     cudaStream_t s);
 kc_status pattern_count_impl(const double* x_ord, const double* l, int64_t N, int d, double rho, int rule,
                              int64_t* rowptr, int64_t* nnz_out, cudaStream_t s);
 kc_status pattern_fill_impl(const double* x_ord, const double* l, int64_t N, int d, double rho, int rule,
@@ -120,7 +122,15 @@ kc_status kc_order_points(const double* x, int64_t N, int32_t d, int32_t* perm, 
     KC_RANGE("kc_order_points");
     KC_TRY(check_points(x, N, d));
     if (!perm || !l || !x_ord) return fail(KC_EINVAL, "output arrays must be non-NULL");
-    return order_impl(x, N, d, perm, l, x_ord, (cudaStream_t)stream);
+    return order_impl(x, N, d, perm, l, x_ord, ORDER_WAIT_CYCLES, (cudaStream_t)stream);
+}
+
+// Test hook, not part of the interface: kc_order_points with another limit of its waits.
+kc_status kc_test_order_points(const double* x, int64_t N, int32_t d, int32_t* perm, double* l, double* x_ord,
+                               int64_t wait_cycles, void* stream) {
+    KC_TRY(check_points(x, N, d));
+    if (!perm || !l || !x_ord) return fail(KC_EINVAL, "output arrays must be non-NULL");
+    return order_impl(x, N, d, perm, l, x_ord, wait_cycles, (cudaStream_t)stream);
 }
 
 kc_status kc_pattern_count(const double* x_ord, const double* l, int64_t N, int32_t d, double rho, int32_t rule,

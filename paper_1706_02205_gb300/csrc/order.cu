@@ -32,7 +32,7 @@
 // swiss roll in R^20 22.4 -> 15.6 (34 in a process that has used many streams,
 // where every launch costs more), 131,071 points of the cube 13.3 -> 7.6, 100,003
 // in the square 9.2 -> 3.7, 2000 4.6 -> 1.2; 60,000 points of the cube in R^20 320 ->
-// 256, 100,003 in R^8 154 -> 147, 5000 in R^20 16.1 -> 10.7; 100,000 points with heavy
+// 260, 100,003 in R^8 154 -> 153, 5000 in R^20 16.1 -> 10.6; 100,000 points with heavy
 // tails (most of them in a few cells) 1170 -> 1155.
 #include <algorithm>
 #include <cmath>
@@ -138,15 +138,27 @@ struct BandArgs {
     unsigned* flags;  // of the grid barrier
     double lo[3], hi[3];
     long long limit;
+    int beat_shift;
 };
 // Counters: of a band by its parity, of a round modulo 3 (reset two phases before their next use).
 struct BandCtl {
     unsigned long long vmax[2];
     unsigned open[2], nb[2], occ[2];
     unsigned nsel[3], nact[3], nhard[3], nlong[3];
-    unsigned bar;
+    unsigned bar, beat;
     int status, rounds;
 };
+// A warp's sign of work, where an item or a long part of one begins: at most once per
+// 2^beat_shift cycles, a 16th of the limit or less.
+__device__ __forceinline__ void beat(const BandArgs& A) {
+    __shared__ unsigned last[8];
+    const unsigned t = (unsigned)(clock64() >> A.beat_shift);
+    volatile unsigned* mine = &last[threadIdx.x >> 5];
+    if (*mine != t) {
+        *mine = t;
+        atomicAdd(&A.ctl->beat, 1u);
+    }
+}
 
 // Band grid: cells a quarter of the largest search radius, at most about 2 nb of
 // them (any grid gives the same order).
@@ -340,6 +352,7 @@ __device__ __forceinline__ int dominator_warp(const BandArgs& A, const Grid& gb,
         }
         const int total = __shfl_sync(FULL, inc, 31);
         for (int m0 = 0; m0 < total; m0 += 32 * SCAN) {
+            if (lane == 0 && (m0 & 2047) == 2048 - 32 * SCAN) beat(A);
             int p[SCAN];
 #pragma unroll
             for (int u = 0; u < SCAN; ++u) {
@@ -427,11 +440,14 @@ struct Cand {
 // arrive at one counter, which only grows; the last of a phase tells every block
 // at a word in a sector of its own (a single word that all poll was slower:
 // 10.6 against 9.35 ms for the ordering of 2^20 points, 25.4 against 24.6 for
-// the 250,007 of a swiss roll).  A wait is at most `limit` cycles; after that, or when
-// another block has failed, the status word is set and false returned.
+// the 250,007 of a swiss roll).  A wait ends, with the status word set and false
+// returned, when no warp has given a sign of work (`beat`) for `limit` cycles, or
+// another block has failed: how long a phase's scans take depends on the points, so
+// a limit on the wait itself would refuse large sets that the grid prunes little.
 // `phase`: the barriers passed so far, kept by the caller (all threads).
 constexpr int BAR_STRIDE = 8;  // words between the blocks' flags
-__device__ bool grid_barrier(unsigned* count, unsigned* flags, unsigned& phase, int* status, long long limit) {
+__device__ bool grid_barrier(unsigned* count, unsigned* flags, unsigned& phase, int* status, const unsigned* beat,
+                             long long limit) {
     __shared__ int ok, last;
     __syncthreads();
     ++phase;
@@ -447,9 +463,17 @@ __device__ bool grid_barrier(unsigned* count, unsigned* flags, unsigned& phase, 
             asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(flags + b * BAR_STRIDE), "r"(phase) : "memory");
     } else if (threadIdx.x == 0) {
         const unsigned* mine = flags + blockIdx.x * BAR_STRIDE;
-        const long long t0 = clock64();
+        long long t0 = clock64();
+        unsigned seen = 0;
         for (int poll = 1; ld_acquire_u32(mine) != phase; ++poll) {
-            if (clock64() - t0 > limit || ((poll & 63) == 0 && ld_volatile_s32(status) != 0)) {
+            bool stop = (poll & 63) == 0 && ld_volatile_s32(status) != 0;
+            if (clock64() - t0 > limit) {
+                const unsigned now = *(const volatile unsigned*)beat;
+                stop |= now == seen;
+                seen = now;
+                t0 = clock64();
+            }
+            if (stop) {
                 atomicCAS(status, 0, DEV_TIMEOUT);
                 ok = 0;
                 break;
@@ -658,7 +682,7 @@ __global__ void __launch_bounds__(256, 4) ord_bands_k(BandArgs A) {
     const int64_t warp = tid >> 5, nw = nt >> 5;
     const bool first = tid == 0;
     unsigned phase = 0;
-    auto barrier = [&]() { return grid_barrier(&C->bar, A.flags, phase, &C->status, A.limit); };
+    auto barrier = [&]() { return grid_barrier(&C->bar, A.flags, phase, &C->status, &C->beat, A.limit); };
     int round = 0;
     for (int band = 0;; ++band) {
         const int bp = band & 1;
@@ -788,6 +812,7 @@ __global__ void __launch_bounds__(256, 4) ord_bands_k(BandArgs A) {
                         if (A.stat[p] == 0) best.take(A.v2[p], A.idg[p], p);
                     }
                     __syncwarp();
+                    if (wide && lane == 0) beat(A);
                     if (wide) best.warp_best();
                     else best.best_of<4>();
                     const bool act = best.g >= 0 && best.v >= T;
@@ -833,6 +858,7 @@ __global__ void __launch_bounds__(256, 4) ord_bands_k(BandArgs A) {
                 const double vq = A.v2[q];
                 if (!(vq >= T)) continue;
                 active = 1;
+                beat(A);
                 // the point that dominated it before may still do
                 const int w0 = A.wit[q];
                 if (w0 >= 0 && A.stat[w0] == 0 && A.wd[q] < vq && key_above(A.v2[w0], A.idg[w0], vq, A.idg[q])) continue;
@@ -860,6 +886,7 @@ __global__ void __launch_bounds__(256, 4) ord_bands_k(BandArgs A) {
                 // 843 of the 990 ms of 60,000 points in the cube of R^20 on them.
                 for (int64_t e = tid; e < nh; e += nt) {
                     const int q = A.hard[e];
+                    beat(A);
                     const double vq = A.v2[q];
                     const int w0 = A.wit[q];
                     if (w0 >= 0 && A.stat[w0] == 0 && A.wd[q] < vq && key_above(A.v2[w0], A.idg[w0], vq, A.idg[q])) continue;
@@ -877,6 +904,7 @@ __global__ void __launch_bounds__(256, 4) ord_bands_k(BandArgs A) {
                 left = A.blist;
             }
             auto scan = [&](int q) {
+                if (lane == 0) beat(A);
                 double wd = 0.0;
                 const double vq = A.v2[q];
                 const int k = dense ? dominator_warp<HIGH, true>(A, gb, q, vq, wd) : dominator_warp<HIGH, false>(A, gb, q, vq, wd);
@@ -940,6 +968,7 @@ __global__ void __launch_bounds__(256, 4) ord_bands_k(BandArgs A) {
                 const int ny = y1 - y0 + 1, rows = ny * (z1 - z0 + 1);
                 const int rb = max(1, min(32, (rows + (int)W - 1) / (int)W));
                 for (int r0 = part * rb; r0 < rows; r0 += (int)W * rb) {
+                    if (lane == 0) beat(A);
                     const int r = r0 + lane;
                     int64_t a = 0;
                     int len = 0;
@@ -983,6 +1012,7 @@ __global__ void __launch_bounds__(256, 4) ord_bands_k(BandArgs A) {
                             const int64_t ra = __shfl_sync(0xffffffffu, a, k);
                             const int ln = __shfl_sync(0xffffffffu, len, k);
                             for (int m = lane; m < ln; m += 32 * UPD) {
+                                if (lane == 0 && (m & 2047) == 2048 - 32 * UPD) beat(A);
                                 int64_t at[UPD];
 #pragma unroll
                                 for (int u = 0; u < UPD; ++u) at[u] = m + 32 * u < ln ? ra + m + 32 * u : -1;
@@ -992,6 +1022,7 @@ __global__ void __launch_bounds__(256, 4) ord_bands_k(BandArgs A) {
                         continue;
                     }
                     for (int m0 = 0; m0 < total; m0 += 32 * UPD) {
+                        if (lane == 0 && (m0 & 2047) == 2048 - 32 * UPD) beat(A);
                         int64_t at[UPD];
 #pragma unroll
                         for (int u = 0; u < UPD; ++u) {
@@ -1044,7 +1075,9 @@ __global__ void ord_out_k(const uint64_t* __restrict__ skey, const int64_t* __re
     for (int t = 0; t < d; ++t) x_ord[k * d + t] = x[id * d + t];
 }
 
-kc_status order_impl(const double* x, int64_t N, int d, int32_t* perm, double* l, double* x_ord, cudaStream_t s) {
+// limit: cycles without a sign of work after which a wait of the kernels gives up.
+kc_status order_impl(const double* x, int64_t N, int d, int32_t* perm, double* l, double* x_ord, long long limit,
+                     cudaStream_t s) {
     Arena A(s);
     Origin org, top;
     double E = 0.0;
@@ -1091,7 +1124,6 @@ kc_status order_impl(const double* x, int64_t N, int d, int32_t* perm, double* l
     ::kc::note_launch(), ord_cells_k<<<blocks_for(N, 256), 256, 0, s>>>(g0, gxg, gs, N, pcell);
     KC_CUDA(cudaGetLastError());
     const int sms = sm_count();
-    const long long limit = 4000000000LL;
 
     // Greedy phase: the coarsest points are selected one at a time (every
     // step updates every point), because while few points are selected the
@@ -1138,6 +1170,8 @@ kc_status order_impl(const double* x, int64_t N, int d, int32_t* perm, double* l
         a.stat = stat;
         a.ctl = ctl;
         a.limit = limit;
+        a.beat_shift = 0;
+        while ((32LL << a.beat_shift) <= limit) ++a.beat_shift;
         for (int t = 0; t < 3; ++t) {
             a.lo[t] = t < g0.dg ? lo[t] : 0.0;
             a.hi[t] = t < g0.dg ? hi[t] : 0.0;

@@ -3,6 +3,7 @@ against the oracle's brute force: rows of the float copy with and without fillin
 rounds with more and with fewer points left than warps, a spread just above and just
 below the line that decides the greedy steps; and that such points take no more of
 the time of as many points in the square than they need."""
+import ctypes as C
 import time
 
 import numpy as np
@@ -53,6 +54,22 @@ def test_order_is_the_greedy_one(name, make):
     assert np.array_equal(p.cpu().numpy(), perm)
     assert np.array_equal(ll.cpu().numpy(), l)
     assert np.array_equal(xo.cpu().numpy(), x[perm])
+
+
+@pytest.mark.parametrize("limit", [1_000_000, 2_000_000])
+def test_phases_longer_than_a_wait(limit):
+    """60,000 points of the cube in R^20: a round takes 5 ms and its blocks finish further apart than the limit of 0.5
+    or 1 ms; they are waited for as long as any of them is at work."""
+    N, d = 60000, 20
+    x = torch.from_numpy(inputs.uniform(N, d, seed=36)).to(DEV)
+    perm, l, xo = kc.order_points(x)
+    p, ll, xx = torch.empty_like(perm), torch.empty_like(l), torch.empty_like(xo)
+    fn = kc.lib().kc_test_order_points
+    fn.argtypes = [C.c_void_p, C.c_int64, C.c_int32, C.c_void_p, C.c_void_p, C.c_void_p, C.c_int64, C.c_void_p]
+    st = fn(x.data_ptr(), N, d, p.data_ptr(), ll.data_ptr(), xx.data_ptr(), limit,
+            torch.cuda.current_stream().cuda_stream)
+    assert st == kc.KC_OK
+    assert torch.equal(p, perm) and torch.equal(ll, l) and torch.equal(xx, xo)
 
 
 def test_time_beside_the_square():
