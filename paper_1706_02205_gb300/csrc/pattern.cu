@@ -14,6 +14,7 @@
 // gives the row lengths, a fill pass scatters the column indices with atomics,
 // and a sort of each row (bitonic, in registers) restores ascending order.
 #include <cmath>
+#include <type_traits>
 
 #include "grid.cuh"
 
@@ -194,12 +195,17 @@ __global__ void pat_chunks_k(PatArgs P, int64_t* __restrict__ nch) {
     nch[it] = (b - a + 31) / 32;
 }
 
-// Lanes per work item in the builder's two passes.  The finest columns, half of
+// Lanes per work item in the builder's two passes, PL.  The finest columns, half of
 // all, look at 10 to 16 candidates per row of cells: with a warp per item more
 // than half of the lanes idle, and the item's chain of dependent loads (its
 // column, box, cells) is walked once per item (pattern and schedule of 2^20 points,
-// rho = 3: 19.2 ms with 32 lanes, 18.9 with 16, 19.1 with 8).
-constexpr int PL = 16;
+// rho = 3: 19.2 ms with 32 lanes, 18.9 with 16, 19.1 with 8).  Where the grid leaves
+// many points in a cell, the walk over an item's candidates takes the time instead:
+// a warp an item from WIDE_ITEMS words (of 32 candidates) an item on average.  The
+// pattern alone with 16 and with 32 lanes: 8.25 and 9.41 ms on the 2^20 grid (1.9
+// words an item), 1.28 and 1.45 for 20,000 points in R^5 (2.9), 2.83 and 2.14 for
+// 100,000 in 20 clusters (54), 159 and 81 for as many with heavy tails (1540).
+constexpr int64_t WIDE_ITEMS = 8;
 
 // Search pass of the builder: PL lanes per item; every 32 candidates'
 // memberships as one mask word, and the members' counts by cell-sorted
@@ -208,7 +214,7 @@ constexpr int PL = 16;
 // search from 3.46 to 3.17 ms and the fill from 4.41 to 3.45, the thresholds of
 // Screen and D at compile time the search to 2.79).  Bound by instruction issue
 // (the tests of about three candidates an entry) and the counters' atomics.
-template <int D, bool MIN>
+template <int D, bool MIN, int PL>
 __global__ void __launch_bounds__(256) pat_mask_k(PatArgs P, const int64_t* __restrict__ moff, int* __restrict__ cntq,
                                                   uint32_t* __restrict__ masks) {
     const int64_t it = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / PL;
@@ -254,6 +260,7 @@ __global__ void pat_next_k(const int32_t* __restrict__ ps, const int64_t* __rest
 // Fill pass of the builder: the members from the masks, no distance tests.  Bound
 // by the scattered 4-byte stores, 188.7 M in 3.45 ms (places counted in 32 bits
 // beside a row base took as long).
+template <int PL>
 __global__ void __launch_bounds__(256) pat_mask_fill_k(PatArgs P, const int64_t* __restrict__ moff,
                                                        const uint32_t* __restrict__ masks,
                                                        unsigned long long* __restrict__ next,
@@ -559,6 +566,7 @@ struct PatternBuilder {
     int64_t N = 0;
     int64_t* moff = nullptr;
     uint32_t* masks = nullptr;
+    bool wide = false;  // a warp per work item
     int64_t* rowptr = nullptr;
     int64_t nnz = 0;
 };
@@ -594,11 +602,17 @@ kc_status pattern_begin_impl(const double* xo, const double* l, int64_t N, int d
         return fail_out(fail(KC_ECUDA, "pattern: chunk count"));
     if ((st = B->A->get(&B->masks, nchunks)) != KC_OK) return fail_out(st);
     if (cudaMemsetAsync(cntq, 0, sizeof(int) * N, s) != cudaSuccess) return fail_out(fail(KC_ECUDA, "memset"));
-    auto mask = rule == KC_RULE_MIN ? pat_mask_k<0, true>
-                : d == 2            ? pat_mask_k<2, false>
-                : d == 3            ? pat_mask_k<3, false>
-                                    : pat_mask_k<0, false>;
-    if (ni > 0) ::kc::note_launch(), mask<<<blocks_for(ni * PL, 256), 256, 0, s>>>(B->P, B->moff, cntq, B->masks);
+    B->wide = nchunks >= WIDE_ITEMS * ni;
+    auto pick = [&](auto lanes) {
+        constexpr int PL = decltype(lanes)::value;
+        return rule == KC_RULE_MIN ? pat_mask_k<0, true, PL>
+               : d == 2            ? pat_mask_k<2, false, PL>
+               : d == 3            ? pat_mask_k<3, false, PL>
+                                   : pat_mask_k<0, false, PL>;
+    };
+    auto mask = B->wide ? pick(std::integral_constant<int, 32>()) : pick(std::integral_constant<int, 16>());
+    if (ni > 0)
+        ::kc::note_launch(), mask<<<blocks_for(ni * (B->wide ? 32 : 16), 256), 256, 0, s>>>(B->P, B->moff, cntq, B->masks);
     ::kc::note_launch(), pat_len_k<<<blocks_for(N, 256), 256, 0, s>>>(B->S.gs, cntq, N, len);
     if (cudaGetLastError() != cudaSuccess) return fail_out(fail(KC_ECUDA, "pattern: search launch"));
     if ((st = exclusive_scan_i32_to_i64(len, rowptr, N, *B->A, s)) != KC_OK) return fail_out(st);
@@ -632,9 +646,11 @@ static kc_status pattern_fill_from(PatternBuilder* B, int32_t* col) {
     unsigned long long* next;
     KC_TRY(A.get(&next, N));
     ::kc::note_launch(), pat_next_k<<<blocks_for(N, 256), 256, 0, s>>>(B->S.gs, B->rowptr, N, next);
-    if (B->S.nitems > 0)
-        ::kc::note_launch(), pat_mask_fill_k<<<blocks_for(B->S.nitems * PL, 256), 256, 0, s>>>(B->P, B->moff, B->masks,
-                                                                                            next, col);
+    if (B->S.nitems > 0) {
+        auto fill = B->wide ? pat_mask_fill_k<32> : pat_mask_fill_k<16>;
+        ::kc::note_launch(), fill<<<blocks_for(B->S.nitems * (B->wide ? 32 : 16), 256), 256, 0, s>>>(B->P, B->moff, B->masks,
+                                                                                                next, col);
+    }
     KC_CUDA(cudaGetLastError());
     int32_t* long_rows;
     unsigned long long* nlong;
