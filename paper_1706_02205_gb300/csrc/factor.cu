@@ -1263,11 +1263,20 @@ static void pick_hash(FactorCore& F) {
 
 // Warps that share one table: so many that a warp's part of it is at most
 // 6 KB (FP64: 6 KB of its 12 bytes per slot), which keeps 24 warps per SM
-// beside their rings, as a power of two that divides the CTA.
+// beside their rings, as a divisor of the CTA's warps (CTAs of 3, 5 or 7 warps are
+// teams as a whole: 131,071 points of the cube, rho = 4, FP64, 3 warps: 397 ms with a
+// table a warp).  With the rows of a task asked for, no more than there are rounds of
+// rows in it, for the others would only help to stage (40,000 points of the cube,
+// rho = 4, FP32 form, 4 rows a task: 45 ms with a warp a task, 75 with teams of two).
 static void pick_team(FactorCore& F) {
-    int w = 1;
-    while (w < 8 && F.warps % (2 * w) == 0 && ((size_t)8 << F.hbits) > (size_t)w * 6144) w <<= 1;
-    F.team = F.stage_bytes > 0 ? 1 : w;
+    const int round = F.prec == KC_FP64 ? RingLayout<double>::RR : RingLayout<float>::RR;
+    const int most = F.rpt > 0 ? std::min(F.warps, std::max(1, F.rpt / round)) : F.warps;
+    F.team = 1;
+    for (int w = 1; w <= most && F.stage_bytes == 0; ++w)
+        if (F.warps % w == 0) {
+            F.team = w;
+            if (((size_t)8 << F.hbits) <= (size_t)w * 6144) break;
+        }
 }
 
 // Rows per task, unless set.  With R rows per level in the mean, a warp gets
