@@ -319,8 +319,14 @@ kc_status kc_solve_noalloc(const kc_pattern* pat, int32_t prec, const void* val,
 
 /* ---- a8: refinement: CG on the dense Theta preconditioned by L L^T ------ *
  * (task (2); CG with the factor as preconditioner, Section 4.3).  The
- * matrix-vector product with Theta is evaluated from the coordinates in
- * FP64, O(N^2) per iteration.  Starts from x = 0; stops when every rhs has
+ * matrix-vector product with Theta is evaluated from the coordinates,
+ * O(N^2) per iteration, every row to the accuracy of FP64 sums: for the
+ * closed-form Matern functions entries and vectors are split into digits
+ * (entries to 2^-57 of sigma2, values to 2^-57 of the largest of their 128
+ * neighbours in the order) where all rows carry enough beside the largest
+ * values, judged by L L^T |v|; other products (vectors with parts of very
+ * different scales, as one-hot vectors or far clusters) and other covariance
+ * functions are in FP64 throughout, about seven times as slow.  Starts from x = 0; stops when every rhs has
  * ||b - Theta x||_2 <= rtol ||b||_2 or after maxit iterations.
  * iters_out (host int32[1]), relres_out (host double[nrhs]): recursive
  * relative residuals.  Returns KC_ENOTCONV or KC_EINDEF on failure. */

@@ -28,7 +28,8 @@
 // arithmetic the products of 777 to 1500 points are 1.1e-16 to 2.0e-16 off in
 // the 2-norm, 1.0e-15 to 1.8e-15 before.  Bound by the integer multiplications
 // and, from 16 right-hand sides on, by the 86 small products of 16 columns; two
-// CTAs an SM instead of three (168 registers): 5.7 ms.
+// CTAs an SM instead of three (168 registers): 5.7 ms.  The check below, that no row
+// loses by it, takes 0.17 ms of a product of 16 vectors.
 #include <algorithm>
 #include <cmath>
 
@@ -63,6 +64,7 @@ struct DenseArgs {
     int64_t blocks_per_split;
     int ns;
     double* out;  // [split][N][ns]
+    const int* exact;  // nonzero: leave this product to FP64
 };
 
 __device__ __forceinline__ uint32_t half2_sub(uint32_t a, uint32_t b) {
@@ -175,6 +177,7 @@ template <int D, int NT, bool INT>
 __global__ void __launch_bounds__(32 * DT_WARPS, 3) dense_theta_mma_k(DenseArgs A) {
     __shared__ double tab[256];
     __shared__ unsigned long long itab[INT ? 256 : 1];
+    if (*A.exact) return;
     for (int q = threadIdx.x; q < 256; q += 32 * DT_WARPS) {
         tab[q] = A.tab[q];
         if constexpr (INT) itab[q] = A.itab[q];
@@ -278,7 +281,10 @@ __global__ void __launch_bounds__(32 * DT_WARPS, 3) dense_theta_mma_k(DenseArgs 
 // value that is not finite gets a NaN for a scale.
 template <int NT>
 __global__ void __launch_bounds__(128) dense_split_k(const double* __restrict__ v, int64_t N, int ns, double sigma2,
-                                                     uint32_t* __restrict__ vf, double* __restrict__ coef) {
+                                                     uint32_t* __restrict__ vf, double* __restrict__ coef,
+                                                     double* __restrict__ bmax, double* __restrict__ w,
+                                                     int* __restrict__ exact) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *exact = 0;
     const int lane = threadIdx.x & 31;
     const int64_t b = blockIdx.x;
     for (int r = threadIdx.x >> 5; r < 8 * NT; r += 4) {
@@ -289,6 +295,7 @@ __global__ void __launch_bounds__(128) dense_split_k(const double* __restrict__ 
         for (int i = 0; i < 4; ++i) {
             const int64_t k = b * DT_BLOCK + 4 * lane + i;
             x[i] = r < ns && k < N ? v[k * ns + r] : 0.0;
+            if (r < ns && k < N) w[k * ns + r] = fabs(x[i]);
             fine &= isfinite(x[i]) != 0;
             mx = fmax(mx, fabs(x[i]));
         }
@@ -308,6 +315,7 @@ __global__ void __launch_bounds__(128) dense_split_k(const double* __restrict__ 
         if (lane == 0) {
             const double c = zero ? 0.0 : scalbn(sigma2, e - 42);
             coef[b * 16 + r] = fine ? c : nan("");
+            bmax[b * 16 + r] = fine ? mx : nan("");
         }
 #pragma unroll
         for (int p = 0; p < 2; ++p) {
@@ -326,12 +334,54 @@ __global__ void __launch_bounds__(128) dense_split_k(const double* __restrict__ 
 
 // y = sum over the splits in order + nugget v
 __global__ void dense_sum_k(const double* __restrict__ part, int splits, int64_t n, double nugget,
-                            const double* __restrict__ v, double* __restrict__ y) {
+                            const double* __restrict__ v, double* __restrict__ y, const int* __restrict__ exact) {
     const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= n) return;
+    if (q >= n || *exact) return;
     double s = part[q];
     for (int p = 1; p < splits; ++p) s += part[(int64_t)p * n + q];
     y[q] = fma(nugget, v[q], s);
+}
+
+// ---- Is every row as accurate as FP64 sums would make it?
+// The split rounds entries to 2^-57 and a block's values to 2^-57 of its largest, so
+// row j is off by some 2^-57 S, S the mean over the vector of its blocks' largest
+// values, whatever the row's own weight T_j = sum_k Theta_jk |v_k| / sigma2 is.  FP64
+// entries and sums are off by 5 to 20 units of 2^-53 T_j in a set's worst row.  Measured against
+// 80-bit sums over 1000 points in two and three dimensions, three kernels, ranges of
+// 0.05 to 0.3, random vectors and their solutions: the split's worst row and its rows
+// of least weight are more accurate wherever T_j >= S / 17, and not all at S / 40;
+// points far from all that is large (one-hot vectors, far clusters of other scales)
+// lie far below.  T_j is estimated by L L^T |v| with the preconditioner's factor (2 x nnz
+// products beside the N^2); a product with a row below S / 16 is left to FP64, as are
+// values or points that are not finite.
+constexpr double LEAST_WEIGHT = 1.0 / 16.0;
+
+// Every block adds up S for itself (16 x nblocks values beside the block's 256 rows).
+__global__ void __launch_bounds__(256) dense_check_k(const double* __restrict__ bmax, const double* __restrict__ tw,
+                                                     double sigma2, const double* __restrict__ x, int64_t N,
+                                                     int64_t nblocks, int d, int ns, int* __restrict__ exact) {
+    __shared__ double sum[16][17], least[16];
+    const int r = threadIdx.x & 15, g = threadIdx.x >> 4;
+    double s = 0.0;
+    if (r < ns)
+        for (int64_t b = g; b < nblocks; b += 16) s += bmax[b * 16 + r] * (double)min((int64_t)DT_BLOCK, N - b * DT_BLOCK);
+    sum[g][r] = s;
+    __syncthreads();
+    if (threadIdx.x < 16) {
+        double t = 0.0;
+        for (int q = 0; q < 16; ++q) t += sum[q][threadIdx.x];
+        least[threadIdx.x] = LEAST_WEIGHT * sigma2 * (t / (double)N);
+    }
+    __syncthreads();
+    const int64_t n = N * ns, q0 = (int64_t)blockIdx.x * 256 * ns;
+    bool bad = false;
+    for (int64_t q = q0 + threadIdx.x; q < min(n, q0 + 256 * ns); q += 256) {
+        const int c = (int)(q & (ns - 1));
+        bad |= !(tw[q] >= least[c]) || !(tw[q] < INFINITY);
+        if (c == 0)
+            for (int t = 0; t < d; ++t) bad |= !isfinite(x[q / ns * d + t]);
+    }
+    if (bad) *exact = 1;
 }
 
 template <int NT>
@@ -339,7 +389,12 @@ kc_status launch(const DenseSplit& S, DenseArgs a, const double* v, double sigma
                  cudaStream_t s) {
     const int64_t nblocks = (a.N + DT_BLOCK - 1) / DT_BLOCK;
     ::kc::note_launch(), dense_split_k<NT><<<(unsigned)nblocks, 128, 0, s>>>(v, a.N, a.ns, sigma2, (uint32_t*)S.vf,
-                                                                          S.coef);
+                                                                          S.coef, S.bmax, S.w, S.exact);
+    KC_CUDA(cudaGetLastError());
+    KC_TRY(S.LL.apply(S.w, S.tw, s));
+    ::kc::note_launch(), dense_check_k<<<blocks_for(a.N, 256), 256, 0, s>>>(S.bmax, S.tw, sigma2, a.x, a.N, nblocks, a.d,
+                                                                         a.ns, S.exact);
+    const int64_t n = a.N * a.ns;
     const dim3 grid(blocks_for(a.N, DT_ROWS), (unsigned)S.splits);
     void (*kfn)(DenseArgs);
     if (a.nu_code < 2)
@@ -353,15 +408,16 @@ kc_status launch(const DenseSplit& S, DenseArgs a, const double* v, double sigma
               : a.d == 3 ? dense_theta_mma_k<3, NT, false>
                          : dense_theta_mma_k<0, NT, false>;
     ::kc::note_launch(), kfn<<<grid, 32 * DT_WARPS, 0, s>>>(a);
-    ::kc::note_launch(), dense_sum_k<<<blocks_for(a.N * a.ns, 256), 256, 0, s>>>(S.part, S.splits, a.N * a.ns, nugget, v,
-                                                                                y);
+    ::kc::note_launch(), dense_sum_k<<<blocks_for(n, 256), 256, 0, s>>>(S.part, S.splits, n, nugget, v, y, S.exact);
     KC_CUDA(cudaGetLastError());
     return KC_OK;
 }
 
 }  // namespace
 
-kc_status dense_split_init(DenseSplit& S, int64_t N, int ns, Arena& A, cudaStream_t s) {
+kc_status dense_split_init(DenseSplit& S, const kc_pattern* P, int prec, const void* val, const double* diag, int ns,
+                           Arena& A, cudaStream_t s) {
+    const int64_t N = P->N;
     const int64_t nblocks = (N + DT_BLOCK - 1) / DT_BLOCK, rows = (N + DT_ROWS - 1) / DT_ROWS;
     // column ranges so that there are about 16 CTAs per SM (two are resident: the last wave is then
     // a small part), at most 32, each of whole blocks
@@ -373,6 +429,11 @@ kc_status dense_split_init(DenseSplit& S, int64_t N, int ns, Arena& A, cudaStrea
     KC_TRY(A.get(&S.coef, nblocks * 16));
     KC_TRY(A.get(&S.part, (int64_t)S.splits * N * ns));
     KC_TRY(A.get(&S.tab, 512));
+    KC_TRY(A.get(&S.bmax, nblocks * 16));
+    KC_TRY(A.get(&S.w, N * ns));
+    KC_TRY(A.get(&S.tw, N * ns));
+    KC_TRY(A.get(&S.exact, 1));
+    KC_TRY(S.LL.init(P, prec, val, diag, ns, A, s));
     // 2^(-j/256) as doubles and as whole multiples of 2^-63: the 64-bit mantissas by seven
     // square roots of 1/2 multiplied up in integers (the host's long double is a double on some machines)
     double h[512];
@@ -418,6 +479,7 @@ kc_status dense_theta_split(const DenseSplit& S, const double* x, int64_t N, int
     a.blocks_per_split = S.per;
     a.ns = ns;
     a.out = S.part;
+    a.exact = S.exact;
     return S.nt == 2 ? launch<2>(S, a, v, kp.sigma2, kp.nugget, y, s) : launch<1>(S, a, v, kp.sigma2, kp.nugget, y, s);
 }
 

@@ -1,7 +1,7 @@
 // Workspace of the dense product by split entries (dense.cu), sized once for
 // all products of a refined solve.
 #pragma once
-#include "common.cuh"
+#include "solver.cuh"
 
 namespace kc {
 
@@ -12,9 +12,17 @@ struct DenseSplit {
     double* tab = nullptr;   // 2^(-j/256)
     int64_t per = 0;         // blocks per column range
     int splits = 0, nt = 0;
+    // whether a product keeps FP64's accuracy row by row
+    double* bmax = nullptr;           // largest value of every block, 16 per block
+    double *w = nullptr, *tw = nullptr;  // |v| and L L^T |v|
+    FactorProduct LL;
+    int* exact = nullptr;             // device: nonzero, this product is left to FP64
 };
-kc_status dense_split_init(DenseSplit& S, int64_t N, int ns, Arena& A, cudaStream_t s);
-// y = Theta v (point-major with stride ns <= 16, a power of two), closed-form Matern kernels (nu_code <= 2)
+// P, val, diag: a factor L with L L^T like Theta (the preconditioner).
+kc_status dense_split_init(DenseSplit& S, const kc_pattern* P, int prec, const void* val, const double* diag, int ns,
+                           Arena& A, cudaStream_t s);
+// y = Theta v (point-major with stride ns <= 16, a power of two), closed-form Matern kernels (nu_code <= 2).
+// Where *S.exact is nonzero afterwards y is not written: the caller forms it in FP64.
 kc_status dense_theta_split(const DenseSplit& S, const double* x, int64_t N, int d, const KernelParams& kp,
                             const double* v, double* y, int ns, cudaStream_t s);
 

@@ -4,8 +4,8 @@
 // factor as preconditioner, M = L L^T (Section 4.3 suggests CG preconditioned
 // with the factor).  Theta is never stored: Theta v is evaluated from the
 // coordinates to FP64 accuracy, O(N^2) per product: for the closed-form Matern
-// kernels by split entries on the tensor cores (dense.cu), for the other
-// covariance functions in FP64 below.  The masked matrix Theta restricted to S
+// kernels by split entries on the tensor cores (dense.cu) where that is as accurate
+// row by row, and else, and for the other covariance functions, in FP64 below.  The masked matrix Theta restricted to S
 // is not positive definite in general, so it is not used as the CG operator.
 //
 // a9's error check uses the same dense product with FP32 entries and
@@ -23,7 +23,8 @@ constexpr int DM_MAXD = 32;
 template <int NRHS>
 __global__ void __launch_bounds__(DM_THREADS) dense_theta_f64_k(const double* __restrict__ x, int64_t N, int d,
                                                               KernelParams kp, const double* __restrict__ v,
-                                                              double* __restrict__ y) {
+                                                              double* __restrict__ y, const int* __restrict__ wanted) {
+    if (wanted && !*wanted) return;
     extern __shared__ __align__(16) double sh[];
     double* sx = sh;                       // DM_THREADS * d
     double* sv = sh + DM_THREADS * d;      // DM_THREADS * NRHS
@@ -64,23 +65,24 @@ __global__ void __launch_bounds__(DM_THREADS) dense_theta_f64_k(const double* __
 
 template <int NRHS>
 static kc_status dense_f64_launch(const double* x, int64_t N, int d, const KernelParams& kp, const double* v,
-                                  double* y, cudaStream_t s) {
+                                  double* y, const int* wanted, cudaStream_t s) {
     size_t sm = sizeof(double) * DM_THREADS * (d + NRHS);
     KC_TRY(allow_dynamic_smem(dense_theta_f64_k<NRHS>));
-    ::kc::note_launch(), dense_theta_f64_k<NRHS><<<blocks_for(N, DM_THREADS), DM_THREADS, sm, s>>>(x, N, d, kp, v, y);
+    ::kc::note_launch(), dense_theta_f64_k<NRHS><<<blocks_for(N, DM_THREADS), DM_THREADS, sm, s>>>(x, N, d, kp, v, y, wanted);
     KC_CUDA(cudaGetLastError());
     return KC_OK;
 }
 
+// wanted (device, may be NULL): zero, nothing is done
 kc_status dense_theta_f64(const double* x, int64_t N, int d, const KernelParams& kp, const double* v, double* y,
-                          int nrhs, cudaStream_t s) {
+                          int nrhs, const int* wanted, cudaStream_t s) {
     if (d > DM_MAXD) return fail(KC_EINVAL, "dense product supports d <= 32");
     switch (nrhs) {
-        case 1: return dense_f64_launch<1>(x, N, d, kp, v, y, s);
-        case 2: return dense_f64_launch<2>(x, N, d, kp, v, y, s);
-        case 4: return dense_f64_launch<4>(x, N, d, kp, v, y, s);
-        case 8: return dense_f64_launch<8>(x, N, d, kp, v, y, s);
-        case 16: return dense_f64_launch<16>(x, N, d, kp, v, y, s);
+        case 1: return dense_f64_launch<1>(x, N, d, kp, v, y, wanted, s);
+        case 2: return dense_f64_launch<2>(x, N, d, kp, v, y, wanted, s);
+        case 4: return dense_f64_launch<4>(x, N, d, kp, v, y, wanted, s);
+        case 8: return dense_f64_launch<8>(x, N, d, kp, v, y, wanted, s);
+        case 16: return dense_f64_launch<16>(x, N, d, kp, v, y, wanted, s);
         default: return fail(KC_EINVAL, "internal: nrhs slot must be 1,2,4,8,16");
     }
 }
@@ -225,8 +227,8 @@ struct CgOperator {
     SparseOp M{};
     kc_status apply(int64_t N, const double* v, double* y, int ns, cudaStream_t s) const {
         if (M.arp) return sparse_pos_mv(M, N, v, y, ns, s);
-        if (split.vf) return dense_theta_split(split, x_ord, N, d, kp, v, y, ns, s);
-        return dense_theta_f64(x_ord, N, d, kp, v, y, ns, s);
+        if (split.vf) KC_TRY(dense_theta_split(split, x_ord, N, d, kp, v, y, ns, s));
+        return dense_theta_f64(x_ord, N, d, kp, v, y, ns, split.exact, s);
     }
 };
 
@@ -275,7 +277,7 @@ static kc_status refine_core(const kc_pattern* P, CgOperator& op, double fb, int
     while (ns < nrhs) ns <<= 1;  // padded slot count (extra columns stay zero)
     Solver S;
     KC_TRY(solver_init(S, P, ns, o, A, s));
-    if (!op.M.arp && op.kp.nu_code <= 2) KC_TRY(dense_split_init(op.split, N, ns, A, s));
+    if (!op.M.arp && op.kp.nu_code <= 2) KC_TRY(dense_split_init(op.split, P, prec, val, diag, ns, A, s));
     const int64_t n = N * ns;
     double *bp, *xs, *r, *z, *p, *q, *partial, *sc;
     int* active;

@@ -21,6 +21,22 @@ struct Solver {
     long long spin = 4000000000LL;
 };
 
+// out = L L^T in for point-major vectors of stride ns (a power of two <= 16) in
+// positions order, with the workspace of one such product (tasks.cu).
+struct FactorProduct {
+    const kc_pattern* P = nullptr;
+    int prec = 0;
+    const void* val = nullptr;
+    const double* diag = nullptr;
+    int ns = 1;
+    int64_t* off = nullptr;
+    int32_t* owner = nullptr;
+    int64_t cap = 0;
+    double *part = nullptr, *mid = nullptr;
+    kc_status init(const kc_pattern* pat, int p, const void* v, const double* dg, int stride, Arena& A, cudaStream_t s);
+    kc_status apply(const double* in, double* out, cudaStream_t s) const;
+};
+
 int64_t tasks_bound(const kc_pattern* P, int rpt);
 kc_status build_tasks(const kc_pattern* P, int rpt, Arena& A, cudaStream_t s, int2** tasks_out,
                       const int64_t** count_out, int64_t* ntasks_out, bool adaptive = false);

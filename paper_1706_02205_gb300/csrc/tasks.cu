@@ -247,6 +247,32 @@ static kc_status mv_dispatch(const kc_pattern* P, bool transpose, const T* val, 
     }
 }
 
+kc_status FactorProduct::init(const kc_pattern* pat, int p, const void* v, const double* dg, int stride, Arena& A,
+                              cudaStream_t s) {
+    P = pat;
+    prec = p;
+    val = v;
+    diag = dg;
+    ns = stride;
+    LtChunks C;
+    KC_TRY(lt_chunks_build(P, A, s, C));
+    off = C.off;
+    owner = C.owner;
+    cap = C.cap;
+    KC_TRY(A.get(&part, C.cap * ns));
+    KC_TRY(A.get(&mid, P->N * ns));
+    return KC_OK;
+}
+kc_status FactorProduct::apply(const double* in, double* out, cudaStream_t s) const {
+    const LtChunks C{off, owner, cap};
+    auto step = [&](bool tr, const double* x, double* y) {
+        return prec == KC_FP64 ? mv_dispatch<double>(P, tr, (const double*)val, diag, x, y, ns, C, part, s)
+                               : mv_dispatch<float>(P, tr, (const float*)val, diag, x, y, ns, C, part, s);
+    };
+    KC_TRY(step(true, in, mid));
+    return step(false, mid, out);
+}
+
 // which: 0 = L, 1 = L^T, 2 = L L^T
 kc_status factor_matvec_impl(const kc_pattern* P, int prec, const void* val, const double* diag, const int32_t* perm,
                              const double* in, int nrhs, double* out, int which, cudaStream_t s) {
