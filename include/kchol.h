@@ -259,7 +259,8 @@ kc_status kc_factor_blocked(const kc_pattern* pat, const double* x_ord, int32_t 
  * is used.  kc_factor_plan_finish synchronises and reports a timeout or the
  * dropped pivots of the last launch.  kc_factor_plan_tune times every
  * combination of lanes per row {2,4,8,16} and staging depth {8,16} once on the
- * plan's own problem and keeps the fastest (it overwrites val and diag). */
+ * plan's own problem (the default number of lanes, which has no depth, once)
+ * and keeps the fastest (it overwrites val and diag). */
 typedef struct kc_factor_plan kc_factor_plan;
 kc_status kc_factor_plan_create(const kc_pattern* pat, const double* x_ord, int32_t d, const kc_kernel* kerns,
                                 int32_t nsets, const int32_t* col_set, int32_t prec, const kc_opts* opts,

@@ -1083,6 +1083,13 @@ struct FactorCore {
     int hold = -1;
 };
 
+// The ring form: the default number of lanes per row, arrays on 16-byte boundaries.
+static bool takes_ring(const FactorCore& F, const void* val) {
+    const int lanes = F.prec == KC_FP64 ? RingLayout<double>::G : RingLayout<float>::G;
+    const bool bulk = F.stage_bytes > 0 && !F.aval && !F.general;  // the other entry sources: ring or register form
+    return !bulk && (F.lanes == 0 || F.lanes == lanes) && ((uintptr_t)F.P.col & 15) == 0 && ((uintptr_t)val & 15) == 0;
+}
+
 template <typename T, int U, int ENT>
 static kc_status launch_core(const FactorCore& F, T* val, double* diag, cudaStream_t s) {
     FactorArgs<T> a;
@@ -1113,9 +1120,8 @@ static kc_status launch_core(const FactorCore& F, T* val, double* diag, cudaStre
     a.lanes = F.lanes;
     a.adaptive = F.adaptive;
     a.stage_bytes = F.stage_bytes;
-    const bool bulk = ENT == 0 && F.stage_bytes > 0;  // the other entry sources: ring or register form
-    const bool ring = !bulk && (F.lanes == 0 || F.lanes == RingLayout<T>::G) && ((uintptr_t)F.P.col & 15) == 0 &&
-                      ((uintptr_t)val & 15) == 0;
+    const bool bulk = ENT == 0 && F.stage_bytes > 0;
+    const bool ring = takes_ring(F, val);
     const int team = bulk ? 1 : F.team;
     int dev = 0, optin = 0;
     KC_CUDA(cudaGetDevice(&dev));
@@ -1448,7 +1454,8 @@ kc_status plan_finish_impl(kc_factor_plan* pl, int64_t* zero_out, cudaStream_t s
 }
 
 // Pick lanes per row (the warp share of one row) and the staging depth by
-// timing every combination once on the plan's own problem.
+// timing every combination once on the plan's own problem.  The ring form has
+// no depth: its lanes are timed once, with the plan's depth.
 kc_status plan_tune_impl(kc_factor_plan* pl, void* val, double* diag, int32_t* lanes_out, int32_t* unroll_out,
                          double* best_ms_out, cudaStream_t s) {
     FactorCore& F = pl->F;
@@ -1459,12 +1466,17 @@ kc_status plan_tune_impl(kc_factor_plan* pl, void* val, double* diag, int32_t* l
     KC_CUDA(cudaEventCreate(&e1));
     double best = 1e300;
     int bl = F.lanes, bu = F.unroll;
+    const int depth = F.unroll;
     KC_TRY(launch_any(F, val, diag, s));  // warm-up
     KC_TRY(read_status(F, nullptr, s));
     for (int L : lanes_c)
         for (int U : unroll_c) {
             F.lanes = L;
             F.unroll = U;
+            if (takes_ring(F, val)) {
+                if (U != unroll_c[0]) continue;
+                F.unroll = depth;
+            }
             KC_CUDA(cudaEventRecord(e0, s));
             KC_TRY(launch_any(F, val, diag, s));
             KC_CUDA(cudaEventRecord(e1, s));
@@ -1474,7 +1486,7 @@ kc_status plan_tune_impl(kc_factor_plan* pl, void* val, double* diag, int32_t* l
             if (ms < best) {
                 best = ms;
                 bl = L;
-                bu = U;
+                bu = F.unroll;
             }
         }
     cudaEventDestroy(e0);
