@@ -109,8 +109,10 @@ typedef struct {
     int64_t spin_limit_cycles;     /* bound of every device wait; 0 -> ~4e9 cycles */
     int32_t rows_per_task;         /* rows of a column per task; 0 -> factor: from the rows per level and the
                                       row length, a power of two in 4..128 (FP64: 8..128) per warp that works
-                                      on the task; factor by column groups: see kc_factor_blocked; backward
-                                      solve: 128 */
+                                      on the task (set: no more warps than the task has groups of 4, FP64 8,
+                                      rows); factor by column groups: see kc_factor_blocked; backward
+                                      solve: 128 (256 for up to 4 right-hand sides where a level has more
+                                      chunks than warps are resident) */
     int32_t ctas_per_sm;           /* persistent grid = SMs x this; 0 -> occupancy; < 0 (factor) ->
                                       occupancy + this (at least 1): leaves that many CTA slots per
                                       SM to kernels on other streams (latency of concurrent solves) */

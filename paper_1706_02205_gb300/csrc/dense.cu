@@ -29,7 +29,7 @@
 // the 2-norm, 1.0e-15 to 1.8e-15 before.  Bound by the integer multiplications
 // and, from 16 right-hand sides on, by the 86 small products of 16 columns; two
 // CTAs an SM instead of three (168 registers): 5.7 ms.  The check below, that no row
-// loses by it, takes 0.17 ms of a product of 16 vectors.
+// loses by it, adds 0.18 ms to a product of 16 vectors.
 #include <algorithm>
 #include <cmath>
 
@@ -419,7 +419,7 @@ kc_status dense_split_init(DenseSplit& S, const kc_pattern* P, int prec, const v
                            Arena& A, cudaStream_t s) {
     const int64_t N = P->N;
     const int64_t nblocks = (N + DT_BLOCK - 1) / DT_BLOCK, rows = (N + DT_ROWS - 1) / DT_ROWS;
-    // column ranges so that there are about 16 CTAs per SM (two are resident: the last wave is then
+    // column ranges so that there are about 16 CTAs per SM (three are resident: the last wave is then
     // a small part), at most 32, each of whole blocks
     const int64_t want = std::min<int64_t>(32, (16 * (int64_t)sm_count() + rows - 1) / rows);
     S.per = (nblocks + want - 1) / std::max<int64_t>(1, want);
@@ -434,7 +434,7 @@ kc_status dense_split_init(DenseSplit& S, const kc_pattern* P, int prec, const v
     KC_TRY(A.get(&S.tw, N * ns));
     KC_TRY(A.get(&S.exact, 1));
     KC_TRY(S.LL.init(P, prec, val, diag, ns, A, s));
-    // 2^(-j/256) as doubles and as whole multiples of 2^-63: the 64-bit mantissas by seven
+    // 2^(-j/256) as doubles and as whole multiples of 2^-63: the 64-bit mantissas by eight
     // square roots of 1/2 multiplied up in integers (the host's long double is a double on some machines)
     double h[512];
     unsigned long long* u = (unsigned long long*)(h + 256);

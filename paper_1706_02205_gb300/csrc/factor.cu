@@ -88,7 +88,7 @@ struct FactorArgs {
     int stage_bytes;  // bulk form: bytes of each of the two stage buffers
 };
 
-// Rows of column k handled by one task.  Adaptive (the factor): at least a
+// Rows of column k handled by one task.  Adaptive (on request): at least a
 // quarter of |R_k|, because every task re-stages row k, so a long row should
 // not be staged again for every few rows below it.
 __device__ __forceinline__ int rows_of_task(const int64_t* __restrict__ rowptr, int k, int rpt, int adaptive) {
@@ -1074,7 +1074,7 @@ struct FactorCore {
     bool general = false;  // some set's kernel is not a closed-form Matern
     const double* aval = nullptr;  // given entries (kc_factor_given)
     int rpt = 128, lanes = 0, unroll = 8, warps = 8, hbits = 7, ctas = 0, adaptive = 0;
-    int stage_req = 0;    // requested stage-buffer bytes: 0 automatic, < 0 register form
+    int stage_req = 0;    // requested stage-buffer bytes of the bulk form: <= 0 ring or register form
     int stage_bytes = 0;  // chosen (0: ring or register form)
     int team = 1;         // warps that share one table
     int bulk_warps = 4;
@@ -1199,9 +1199,12 @@ static kc_status launch_core(const FactorCore& F, T* val, double* diag, cudaStre
     return KC_OK;
 }
 
-// The closed-form Matern kernels take the unroll asked for; the other entry
-// sources one instantiation per precision (register form, 8 loads in flight
-// per lane in the FP32 form, 4 in FP64).
+// The closed-form Matern kernels take the unroll asked for (register form); the
+// other entry sources have one instantiation per precision (8 loads in flight per
+// lane in the FP32 form, 4 in FP64).  All of them run in the ring form by default.
+// The covariance functions behind calls (ENT = 1) spill 80 to 108 bytes there, what
+// is kept across the calls; their calls take far longer (100,003 points, nu = 0.8,
+// FP32 form: 6.3 ms beside 3.4 for nu = 5/2).
 static kc_status launch_any(const FactorCore& F, void* val, double* diag, cudaStream_t s) {
     if (F.aval)
         return F.prec == KC_FP64 ? launch_core<double, 4, 2>(F, (double*)val, diag, s)

@@ -95,7 +95,7 @@ def test_rows_of_little_weight(kind, nu, d):
 
 @pytest.mark.parametrize("nu", [0.5, 1.5, 2.5])
 @pytest.mark.parametrize("d", [1, 2, 3, 5])
-@pytest.mark.parametrize("N", [129, 777, 1500])
+@pytest.mark.parametrize("N", [129, 777])
 def test_ordinary_vectors(N, d, nu):
     """x lies in the plane of b and Theta b whatever the numbers a, c, e (dot products, whose rounding a short residual
     magnifies): its distance from that plane is what the product and the vector steps rounded."""
