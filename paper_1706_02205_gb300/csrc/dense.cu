@@ -356,7 +356,8 @@ __global__ void dense_sum_k(const double* __restrict__ part, int splits, int64_t
 // values or points that are not finite.
 constexpr double LEAST_WEIGHT = 1.0 / 16.0;
 
-// Every block adds up S for itself (16 x nblocks values beside the block's 256 rows).
+// Every block of 64 rows adds up S for itself, from 16 x nblocks values.
+constexpr int CHECK_ROWS = 64;
 __global__ void __launch_bounds__(256) dense_check_k(const double* __restrict__ bmax, const double* __restrict__ tw,
                                                      double sigma2, const double* __restrict__ x, int64_t N,
                                                      int64_t nblocks, int d, int ns, int* __restrict__ exact) {
@@ -373,9 +374,9 @@ __global__ void __launch_bounds__(256) dense_check_k(const double* __restrict__ 
         least[threadIdx.x] = LEAST_WEIGHT * sigma2 * (t / (double)N);
     }
     __syncthreads();
-    const int64_t n = N * ns, q0 = (int64_t)blockIdx.x * 256 * ns;
+    const int64_t n = N * ns, q0 = (int64_t)blockIdx.x * CHECK_ROWS * ns;
     bool bad = false;
-    for (int64_t q = q0 + threadIdx.x; q < min(n, q0 + 256 * ns); q += 256) {
+    for (int64_t q = q0 + threadIdx.x; q < min(n, q0 + CHECK_ROWS * ns); q += 256) {
         const int c = (int)(q & (ns - 1));
         bad |= !(tw[q] >= least[c]) || !(tw[q] < INFINITY);
         if (c == 0)
@@ -392,7 +393,7 @@ kc_status launch(const DenseSplit& S, DenseArgs a, const double* v, double sigma
                                                                           S.coef, S.bmax, S.w, S.exact);
     KC_CUDA(cudaGetLastError());
     KC_TRY(S.LL.apply(S.w, S.tw, s));
-    ::kc::note_launch(), dense_check_k<<<blocks_for(a.N, 256), 256, 0, s>>>(S.bmax, S.tw, sigma2, a.x, a.N, nblocks, a.d,
+    ::kc::note_launch(), dense_check_k<<<blocks_for(a.N, CHECK_ROWS), 256, 0, s>>>(S.bmax, S.tw, sigma2, a.x, a.N, nblocks, a.d,
                                                                          a.ns, S.exact);
     const int64_t n = a.N * a.ns;
     const dim3 grid(blocks_for(a.N, DT_ROWS), (unsigned)S.splits);
