@@ -29,7 +29,7 @@
 // Bound by latency: about 50 rounds of dependent scans, each between grid
 // barriers.  Measured (before: a dozen launches and two waits of the host per
 // round): 2^20 points of a jittered grid 16.0 -> 8.4 ms, 250,007 points of a
-// swiss roll in R^20 22.4 -> 15.6 (34 in a process that has used many streams,
+// swiss roll in R^20 22.4 -> 15.3 (34 in a process that has used many streams,
 // where every launch costs more), 131,071 points of the cube 13.3 -> 7.6, 100,003
 // in the square 9.2 -> 3.7, 2000 4.6 -> 1.2; 60,000 points of the cube in R^20 320 ->
 // 260, 100,003 in R^8 154 -> 153, 5000 in R^20 16.1 -> 10.6; 100,000 points with heavy
@@ -844,6 +844,7 @@ __global__ void __launch_bounds__(256, 4) ord_bands_k(BandArgs A) {
                 for (int64_t c = tid; c < gb.ncells; c += nt) {
                     long long m = -1;
                     for (int f = A.bstart[c]; f < A.bstart[c + 1]; ++f) {
+                        if ((f & 4095) == 4095) beat(A);
                         const int p = A.bsorted[f];
                         if (A.stat[p] == 0) m = max(m, vbits(A.v2[p]));
                     }

@@ -5,8 +5,9 @@
 // with the factor).  Theta is never stored: Theta v is evaluated from the
 // coordinates to FP64 accuracy, O(N^2) per product: for the closed-form Matern
 // kernels by split entries on the tensor cores (dense.cu) where that is as accurate
-// row by row, and else, and for the other covariance functions, in FP64 below.  The masked matrix Theta restricted to S
-// is not positive definite in general, so it is not used as the CG operator.
+// row by row, and else, and for the other covariance functions, in FP64 below.
+// The masked matrix Theta restricted to S is not positive definite in general, so
+// it is not used as the CG operator.
 //
 // a9's error check uses the same dense product with FP32 entries and
 // compensated (Dot2) tile sums combined in FP64.
