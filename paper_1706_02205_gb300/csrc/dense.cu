@@ -29,7 +29,7 @@
 // the 2-norm, 1.0e-15 to 1.8e-15 before.  Bound by the integer multiplications
 // and, from 16 right-hand sides on, by the 86 small products of 16 columns; two
 // CTAs an SM instead of three (168 registers): 5.7 ms.  The check below, that no row
-// loses by it, adds 0.18 ms to a product of 16 vectors.
+// loses by it, adds 0.06 ms to a product of 16 vectors.
 #include <algorithm>
 #include <cmath>
 
@@ -282,8 +282,8 @@ __global__ void __launch_bounds__(32 * DT_WARPS, 3) dense_theta_mma_k(DenseArgs 
 template <int NT>
 __global__ void __launch_bounds__(128) dense_split_k(const double* __restrict__ v, int64_t N, int ns, double sigma2,
                                                      uint32_t* __restrict__ vf, double* __restrict__ coef,
-                                                     double* __restrict__ bmax, double* __restrict__ w,
-                                                     int* __restrict__ exact) {
+                                                     double* __restrict__ bmax, const double* __restrict__ scale,
+                                                     float* __restrict__ w, int* __restrict__ exact) {
     if (blockIdx.x == 0 && threadIdx.x == 0) *exact = 0;
     const int lane = threadIdx.x & 31;
     const int64_t b = blockIdx.x;
@@ -295,7 +295,7 @@ __global__ void __launch_bounds__(128) dense_split_k(const double* __restrict__ 
         for (int i = 0; i < 4; ++i) {
             const int64_t k = b * DT_BLOCK + 4 * lane + i;
             x[i] = r < ns && k < N ? v[k * ns + r] : 0.0;
-            if (r < ns && k < N) w[k * ns + r] = fabs(x[i]);
+            if (r < ns && k < N) w[k * ns + r] = (float)(fabs(x[i]) * scale[r]);
             fine &= isfinite(x[i]) != 0;
             mx = fmax(mx, fabs(x[i]));
         }
@@ -351,17 +351,29 @@ __global__ void dense_sum_k(const double* __restrict__ part, int splits, int64_t
 // 0.05 to 0.3, random vectors and their solutions: the split's worst row and its rows
 // of least weight are more accurate wherever T_j >= S / 17, and not all at S / 40;
 // points far from all that is large (one-hot vectors, far clusters of other scales)
-// lie far below.  T_j is estimated by L L^T |v| with the preconditioner's factor (2 x nnz
-// products beside the N^2); a product with a row below S / 16 is left to FP64, as are
+// lie far below.  T_j is estimated by L L^T |v| with the preconditioner's factor in floats
+// (2 x nnz products beside the N^2; in doubles they took three times as long, 0.17 ms
+// for 1.7 M entries and 16 vectors); a product with a row below S / 16 is left to FP64, as are
 // values or points that are not finite.
 constexpr double LEAST_WEIGHT = 1.0 / 16.0;
 
+// scale = the power of two by which a vector like the right-hand side, over sigma2, is of size 1
+__global__ void dense_scale_k(const double* __restrict__ norm2, int64_t N, double sigma2, int ns,
+                              double* __restrict__ scale) {
+    const int r = threadIdx.x;
+    if (r >= 16) return;
+    const double m = r < ns ? sqrt(norm2[r] / (double)N) : 0.0;
+    scale[r] = m > 0.0 && m < INFINITY ? scalbn(1.0, max(-1000, min(1000, -ilogb(m) - ilogb(sigma2)))) : 1.0;
+}
+
 // Every block of 64 rows adds up S for itself, from 16 x nblocks values.
 constexpr int CHECK_ROWS = 64;
-__global__ void __launch_bounds__(256) dense_check_k(const double* __restrict__ bmax, const double* __restrict__ tw,
-                                                     double sigma2, const double* __restrict__ x, int64_t N,
-                                                     int64_t nblocks, int d, int ns, int* __restrict__ exact) {
-    __shared__ double sum[16][17], least[16];
+__global__ void __launch_bounds__(256) dense_check_k(const double* __restrict__ bmax, const double* __restrict__ scale,
+                                                     const float* __restrict__ tw, double sigma2,
+                                                     const double* __restrict__ x, int64_t N, int64_t nblocks, int d,
+                                                     int ns, int* __restrict__ exact) {
+    __shared__ double sum[16][17];
+    __shared__ float least[16];
     const int r = threadIdx.x & 15, g = threadIdx.x >> 4;
     double s = 0.0;
     if (r < ns)
@@ -371,7 +383,7 @@ __global__ void __launch_bounds__(256) dense_check_k(const double* __restrict__ 
     if (threadIdx.x < 16) {
         double t = 0.0;
         for (int q = 0; q < 16; ++q) t += sum[q][threadIdx.x];
-        least[threadIdx.x] = LEAST_WEIGHT * sigma2 * (t / (double)N);
+        least[threadIdx.x] = (float)(LEAST_WEIGHT * sigma2 * (t / (double)N) * scale[threadIdx.x]);
     }
     __syncthreads();
     const int64_t n = N * ns, q0 = (int64_t)blockIdx.x * CHECK_ROWS * ns;
@@ -390,11 +402,11 @@ kc_status launch(const DenseSplit& S, DenseArgs a, const double* v, double sigma
                  cudaStream_t s) {
     const int64_t nblocks = (a.N + DT_BLOCK - 1) / DT_BLOCK;
     ::kc::note_launch(), dense_split_k<NT><<<(unsigned)nblocks, 128, 0, s>>>(v, a.N, a.ns, sigma2, (uint32_t*)S.vf,
-                                                                          S.coef, S.bmax, S.w, S.exact);
+                                                                          S.coef, S.bmax, S.scale, S.w, S.exact);
     KC_CUDA(cudaGetLastError());
     KC_TRY(S.LL.apply(S.w, S.tw, s));
-    ::kc::note_launch(), dense_check_k<<<blocks_for(a.N, CHECK_ROWS), 256, 0, s>>>(S.bmax, S.tw, sigma2, a.x, a.N, nblocks, a.d,
-                                                                         a.ns, S.exact);
+    ::kc::note_launch(), dense_check_k<<<blocks_for(a.N, CHECK_ROWS), 256, 0, s>>>(S.bmax, S.scale, S.tw, sigma2, a.x, a.N,
+                                                                                  nblocks, a.d, a.ns, S.exact);
     const int64_t n = a.N * a.ns;
     const dim3 grid(blocks_for(a.N, DT_ROWS), (unsigned)S.splits);
     void (*kfn)(DenseArgs);
@@ -416,8 +428,8 @@ kc_status launch(const DenseSplit& S, DenseArgs a, const double* v, double sigma
 
 }  // namespace
 
-kc_status dense_split_init(DenseSplit& S, const kc_pattern* P, int prec, const void* val, const double* diag, int ns,
-                           Arena& A, cudaStream_t s) {
+kc_status dense_split_init(DenseSplit& S, const kc_pattern* P, int prec, const void* val, const double* diag,
+                           double sigma2, const double* norm2, int ns, Arena& A, cudaStream_t s) {
     const int64_t N = P->N;
     const int64_t nblocks = (N + DT_BLOCK - 1) / DT_BLOCK, rows = (N + DT_ROWS - 1) / DT_ROWS;
     // column ranges so that there are about 16 CTAs per SM (three are resident: the last wave is then
@@ -434,6 +446,8 @@ kc_status dense_split_init(DenseSplit& S, const kc_pattern* P, int prec, const v
     KC_TRY(A.get(&S.w, N * ns));
     KC_TRY(A.get(&S.tw, N * ns));
     KC_TRY(A.get(&S.exact, 1));
+    KC_TRY(A.get(&S.scale, 16));
+    ::kc::note_launch(), dense_scale_k<<<1, 32, 0, s>>>(norm2, N, sigma2, ns, S.scale);
     KC_TRY(S.LL.init(P, prec, val, diag, ns, A, s));
     // 2^(-j/256) as doubles and as whole multiples of 2^-63: the 64-bit mantissas by eight
     // square roots of 1/2 multiplied up in integers (the host's long double is a double on some machines)

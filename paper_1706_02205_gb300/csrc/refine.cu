@@ -278,7 +278,6 @@ static kc_status refine_core(const kc_pattern* P, CgOperator& op, double fb, int
     while (ns < nrhs) ns <<= 1;  // padded slot count (extra columns stay zero)
     Solver S;
     KC_TRY(solver_init(S, P, ns, o, A, s));
-    if (!op.M.arp && op.kp.nu_code <= 2) KC_TRY(dense_split_init(op.split, P, prec, val, diag, ns, A, s));
     const int64_t n = N * ns;
     double *bp, *xs, *r, *z, *p, *q, *partial, *sc;
     int* active;
@@ -313,6 +312,8 @@ static kc_status refine_core(const kc_pattern* P, CgOperator& op, double fb, int
     const unsigned gb = blocks_for(n, 256);
     ::kc::note_launch(), copy_k<<<gb, 256, 0, s>>>(r, bp, n);
     KC_TRY(dots(bp, bp, N, ns, partial, bb, s));
+    if (!op.M.arp && op.kp.nu_code <= 2)
+        KC_TRY(dense_split_init(op.split, P, prec, val, diag, op.kp.sigma2, bb, ns, A, s));
     KC_TRY(precond(r, z));
     ::kc::note_launch(), copy_k<<<gb, 256, 0, s>>>(p, z, n);
     KC_TRY(dots(r, z, N, ns, partial, rz, s));

@@ -22,8 +22,8 @@ struct Solver {
 };
 
 // out = L L^T in for point-major vectors of stride ns (a power of two <= 16) in
-// positions order, with the workspace of one such product (tasks.cu).
-struct FactorProduct {
+// positions order, in floats, with the workspace of one such product (tasks.cu).
+struct FactorEstimate {
     const kc_pattern* P = nullptr;
     int prec = 0;
     const void* val = nullptr;
@@ -32,9 +32,9 @@ struct FactorProduct {
     int64_t* off = nullptr;
     int32_t* owner = nullptr;
     int64_t cap = 0;
-    double *part = nullptr, *mid = nullptr;
+    float *part = nullptr, *mid = nullptr;
     kc_status init(const kc_pattern* pat, int p, const void* v, const double* dg, int stride, Arena& A, cudaStream_t s);
-    kc_status apply(const double* in, double* out, cudaStream_t s) const;
+    kc_status apply(const float* in, float* out, cudaStream_t s) const;
 };
 
 int64_t tasks_bound(const kc_pattern* P, int rpt);

@@ -33,25 +33,37 @@ struct MvLayout {
     static constexpr int EL = 32 / P;  // entries at a time
 };
 
+// Vectors are doubles, or floats where an estimate will do (FactorEstimate).
+template <typename V>
+struct Two;
+template <>
+struct Two<double> {
+    using type = double2;
+};
+template <>
+struct Two<float> {
+    using type = float2;
+};
+
 // acc[r] += w v[k * NS + part + r] over 32 entries of the row (column), entry
 // t held by lane t (w = 0 past its end, k then anything valid)
-template <int NS>
-__device__ __forceinline__ void block_fma(double (&acc)[MvLayout<NS>::NSL], int k, double w, int cnt,
-                                          const double* __restrict__ v, int lane) {
+template <int NS, typename V>
+__device__ __forceinline__ void block_fma(V (&acc)[MvLayout<NS>::NSL], int k, V w, int cnt, const V* __restrict__ v,
+                                          int lane) {
     using ML = MvLayout<NS>;
     const int el = lane / ML::P, part = (lane % ML::P) * ML::NSL;
 #pragma unroll
     for (int t0 = 0; t0 < 32; t0 += ML::EL) {
         const int kk = ML::P == 1 ? k : __shfl_sync(0xffffffffu, k, t0 + el);
-        const double ww = ML::P == 1 ? w : __shfl_sync(0xffffffffu, w, t0 + el);
+        const V ww = ML::P == 1 ? w : __shfl_sync(0xffffffffu, w, t0 + el);
         if (t0 + el < cnt) {
-            const double* p = v + (int64_t)kk * NS + part;
+            const V* p = v + (int64_t)kk * NS + part;
             if constexpr (ML::NSL == 1) {
                 acc[0] = fma(ww, __ldg(p), acc[0]);
             } else {
 #pragma unroll
                 for (int r = 0; r < ML::NSL; r += 2) {
-                    const double2 x = __ldg((const double2*)(p + r));
+                    const typename Two<V>::type x = __ldg((const typename Two<V>::type*)(p + r));
                     acc[r] = fma(ww, x.x, acc[r]);
                     acc[r + 1] = fma(ww, x.y, acc[r + 1]);
                 }
@@ -63,8 +75,8 @@ __device__ __forceinline__ void block_fma(double (&acc)[MvLayout<NS>::NSL], int 
 // The warp's total of one vector: a reduce-scatter over the lanes of one part
 // (the sums a lane keeps halve, then plain sums).  The lane ends with the total
 // of vector `r`; `writer` is true in one lane per vector.
-template <int NS>
-__device__ __forceinline__ double warp_total(double (&acc)[MvLayout<NS>::NSL], int lane, int& r, bool& writer) {
+template <int NS, typename V>
+__device__ __forceinline__ V warp_total(V (&acc)[MvLayout<NS>::NSL], int lane, int& r, bool& writer) {
     using ML = MvLayout<NS>;
     r = (lane % ML::P) * ML::NSL;
     int o = 16;
@@ -73,7 +85,7 @@ __device__ __forceinline__ double warp_total(double (&acc)[MvLayout<NS>::NSL], i
         const bool up = (lane & o) != 0;
 #pragma unroll
         for (int q = 0; q < h; ++q) {
-            const double send = up ? acc[q] : acc[q + h], keep = up ? acc[q + h] : acc[q];
+            const V send = up ? acc[q] : acc[q + h], keep = up ? acc[q + h] : acc[q];
             acc[q] = keep + __shfl_xor_sync(0xffffffffu, send, o);
         }
         if (up) r += h;
@@ -86,35 +98,35 @@ __device__ __forceinline__ double warp_total(double (&acc)[MvLayout<NS>::NSL], i
 
 // y = L z: row j of L is col/val[rowptr[j] .. rowptr[j+1]-1), the diagonal last
 // (taken from diag, the FP64 L_jj).
-template <typename T, int NS>
+template <typename T, int NS, typename V>
 __global__ void __launch_bounds__(TK_THREADS) l_rows_k(const int64_t* __restrict__ rowptr,
                                                        const int32_t* __restrict__ col, const T* __restrict__ val,
                                                        const double* __restrict__ diag, int64_t N,
-                                                       const double* __restrict__ z, double* __restrict__ y) {
+                                                       const V* __restrict__ z, V* __restrict__ y) {
     const int64_t j = (int64_t)blockIdx.x * TK_WARPS + (threadIdx.x >> 5);
     if (j >= N) return;
     const int lane = lane_id();
-    double acc[MvLayout<NS>::NSL] = {};
+    V acc[MvLayout<NS>::NSL] = {};
     const int64_t e0 = rowptr[j];
-    const double dj = diag[j];
+    const V dj = (V)diag[j];
     if constexpr (NS == 1) {  // (the blocks below cost one vector 5 %: 110 against 116 us, 40,000 points)
         const int64_t e1 = rowptr[j + 1] - 1;
 #pragma unroll 4
         for (int64_t e = e0 + lane; e < e1; e += 32)
-            acc[0] = fma((double)__ldg(&val[e]), __ldg(&z[__ldg(&col[e])]), acc[0]);
+            acc[0] = fma((V)__ldg(&val[e]), __ldg(&z[__ldg(&col[e])]), acc[0]);
     } else {
         const int n = (int)(rowptr[j + 1] - 1 - e0);
 #pragma unroll (NS <= 2 ? 4 : 2)
         for (int t = 0; t < n; t += 32) {
             const bool in = t + lane < n;
             const int k = in ? __ldg(&col[e0 + t + lane]) : 0;
-            const double w = in ? (double)__ldg(&val[e0 + t + lane]) : 0.0;
+            const V w = in ? (V)__ldg(&val[e0 + t + lane]) : (V)0;
             block_fma<NS>(acc, k, w, n - t, z, lane);
         }
     }
     int r;
     bool writer;
-    const double s = warp_total<NS>(acc, lane, r, writer);
+    const V s = warp_total<NS>(acc, lane, r, writer);
     if (writer) y[j * NS + r] = fma(dj, z[j * NS + r], s);
 }
 
@@ -139,15 +151,15 @@ __global__ void lt_owner_k(const int64_t* __restrict__ off, int64_t N, int32_t* 
     for (int64_t c = off[i]; c < off[i + 1]; ++c) owner[c] = (int32_t)i;
 }
 
-template <typename T, int NS>
+template <typename T, int NS, typename V>
 __global__ void __launch_bounds__(TK_THREADS) lt_chunks_k(const int64_t* __restrict__ colptr,
                                                           const int32_t* __restrict__ rowidx,
                                                           const int64_t* __restrict__ slot, const T* __restrict__ val,
                                                           const double* __restrict__ diag,
                                                           const int64_t* __restrict__ off,
                                                           const int32_t* __restrict__ owner, int64_t N,
-                                                          const double* __restrict__ v, double* __restrict__ y,
-                                                          double* __restrict__ part) {
+                                                          const V* __restrict__ v, V* __restrict__ y,
+                                                          V* __restrict__ part) {
     const int64_t c = (int64_t)blockIdx.x * TK_WARPS + (threadIdx.x >> 5);
     if (c >= off[N]) return;
     const int i = owner[c];
@@ -155,25 +167,25 @@ __global__ void __launch_bounds__(TK_THREADS) lt_chunks_k(const int64_t* __restr
     const int64_t q0 = colptr[i] + 1 + k * LT_CHUNK;
     const int64_t q1 = min(colptr[i + 1], q0 + LT_CHUNK);
     const int lane = lane_id();
-    double acc[MvLayout<NS>::NSL] = {};
-    const double di = diag[i];
+    V acc[MvLayout<NS>::NSL] = {};
+    const V di = (V)diag[i];
     if constexpr (NS == 1) {
 #pragma unroll 4
         for (int64_t q = q0 + lane; q < q1; q += 32)
-            acc[0] = fma((double)__ldg(&val[__ldg(&slot[q])]), __ldg(&v[__ldg(&rowidx[q])]), acc[0]);
+            acc[0] = fma((V)__ldg(&val[__ldg(&slot[q])]), __ldg(&v[__ldg(&rowidx[q])]), acc[0]);
     } else {
         const int n = (int)(q1 - q0);
 #pragma unroll (NS <= 2 ? 4 : 2)
         for (int t = 0; t < n; t += 32) {
             const bool in = t + lane < n;
             const int j = in ? __ldg(&rowidx[q0 + t + lane]) : 0;
-            const double w = in ? (double)__ldg(&val[__ldg(&slot[q0 + t + lane])]) : 0.0;
+            const V w = in ? (V)__ldg(&val[__ldg(&slot[q0 + t + lane])]) : (V)0;
             block_fma<NS>(acc, j, w, n - t, v, lane);
         }
     }
     int r;
     bool writer;
-    const double s = warp_total<NS>(acc, lane, r, writer);
+    const V s = warp_total<NS>(acc, lane, r, writer);
     if (writer) {
         if (off[i + 1] - off[i] == 1) y[(int64_t)i * NS + r] = fma(di, v[(int64_t)i * NS + r], s);
         else part[c * NS + r] = s;
@@ -181,18 +193,18 @@ __global__ void __launch_bounds__(TK_THREADS) lt_chunks_k(const int64_t* __restr
 }
 
 // y[i][r] of the columns cut into several chunks: the chunk sums in order
-template <int NS>
+template <int NS, typename V>
 __global__ void lt_finish_k(const int64_t* __restrict__ off, int64_t N, const double* __restrict__ diag,
-                            const double* __restrict__ v, const double* __restrict__ part, double* __restrict__ y) {
+                            const V* __restrict__ v, const V* __restrict__ part, V* __restrict__ y) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= N * NS) return;
     const int64_t i = t / NS;
     const int r = (int)(t % NS);
     const int64_t c0 = off[i], c1 = off[i + 1];
     if (c1 - c0 == 1) return;
-    double s = 0.0;
+    V s = (V)0;
     for (int64_t c = c0; c < c1; ++c) s += part[c * NS + r];
-    y[i * NS + r] = fma(diag[i], v[i * NS + r], s);
+    y[i * NS + r] = fma((V)diag[i], v[i * NS + r], s);
 }
 
 // Chunk layout of the columns (independent of the vectors): off[i] = first
@@ -218,36 +230,36 @@ static kc_status lt_chunks_build(const kc_pattern* P, Arena& A, cudaStream_t s, 
     return KC_OK;
 }
 
-template <typename T, int NS>
-static kc_status mv_launch(const kc_pattern* P, bool transpose, const T* val, const double* diag, const double* in,
-                           double* out, const LtChunks& C, double* part, cudaStream_t s) {
+template <typename T, int NS, typename V>
+static kc_status mv_launch(const kc_pattern* P, bool transpose, const T* val, const double* diag, const V* in,
+                           V* out, const LtChunks& C, V* part, cudaStream_t s) {
     if (transpose) {
         // the grid covers the most chunks there can be; surplus warps return
-        note_launch(), lt_chunks_k<T, NS><<<blocks_for(C.cap, TK_WARPS), TK_THREADS, 0, s>>>(
+        note_launch(), lt_chunks_k<T, NS, V><<<blocks_for(C.cap, TK_WARPS), TK_THREADS, 0, s>>>(
             P->colptr, P->rowidx, P->slot, val, diag, C.off, C.owner, P->N, in, out, part);
         KC_CUDA(cudaGetLastError());
-        note_launch(), lt_finish_k<NS><<<blocks_for(P->N * NS, 256), 256, 0, s>>>(C.off, P->N, diag, in, part, out);
+        note_launch(), lt_finish_k<NS, V><<<blocks_for(P->N * NS, 256), 256, 0, s>>>(C.off, P->N, diag, in, part, out);
     } else {
-        note_launch(), l_rows_k<T, NS><<<blocks_for(P->N, TK_WARPS), TK_THREADS, 0, s>>>(P->rowptr, P->col, val, diag,
+        note_launch(), l_rows_k<T, NS, V><<<blocks_for(P->N, TK_WARPS), TK_THREADS, 0, s>>>(P->rowptr, P->col, val, diag,
                                                                                          P->N, in, out);
     }
     KC_CUDA(cudaGetLastError());
     return KC_OK;
 }
 
-template <typename T>
-static kc_status mv_dispatch(const kc_pattern* P, bool transpose, const T* val, const double* diag, const double* in,
-                             double* out, int ns, const LtChunks& C, double* part, cudaStream_t s) {
+template <typename T, typename V>
+static kc_status mv_dispatch(const kc_pattern* P, bool transpose, const T* val, const double* diag, const V* in,
+                             V* out, int ns, const LtChunks& C, V* part, cudaStream_t s) {
     switch (ns) {
-        case 1: return mv_launch<T, 1>(P, transpose, val, diag, in, out, C, part, s);
-        case 2: return mv_launch<T, 2>(P, transpose, val, diag, in, out, C, part, s);
-        case 4: return mv_launch<T, 4>(P, transpose, val, diag, in, out, C, part, s);
-        case 8: return mv_launch<T, 8>(P, transpose, val, diag, in, out, C, part, s);
-        default: return mv_launch<T, 16>(P, transpose, val, diag, in, out, C, part, s);
+        case 1: return mv_launch<T, 1, V>(P, transpose, val, diag, in, out, C, part, s);
+        case 2: return mv_launch<T, 2, V>(P, transpose, val, diag, in, out, C, part, s);
+        case 4: return mv_launch<T, 4, V>(P, transpose, val, diag, in, out, C, part, s);
+        case 8: return mv_launch<T, 8, V>(P, transpose, val, diag, in, out, C, part, s);
+        default: return mv_launch<T, 16, V>(P, transpose, val, diag, in, out, C, part, s);
     }
 }
 
-kc_status FactorProduct::init(const kc_pattern* pat, int p, const void* v, const double* dg, int stride, Arena& A,
+kc_status FactorEstimate::init(const kc_pattern* pat, int p, const void* v, const double* dg, int stride, Arena& A,
                               cudaStream_t s) {
     P = pat;
     prec = p;
@@ -263,11 +275,11 @@ kc_status FactorProduct::init(const kc_pattern* pat, int p, const void* v, const
     KC_TRY(A.get(&mid, P->N * ns));
     return KC_OK;
 }
-kc_status FactorProduct::apply(const double* in, double* out, cudaStream_t s) const {
+kc_status FactorEstimate::apply(const float* in, float* out, cudaStream_t s) const {
     const LtChunks C{off, owner, cap};
-    auto step = [&](bool tr, const double* x, double* y) {
-        return prec == KC_FP64 ? mv_dispatch<double>(P, tr, (const double*)val, diag, x, y, ns, C, part, s)
-                               : mv_dispatch<float>(P, tr, (const float*)val, diag, x, y, ns, C, part, s);
+    auto step = [&](bool tr, const float* x, float* y) {
+        return prec == KC_FP64 ? mv_dispatch<double, float>(P, tr, (const double*)val, diag, x, y, ns, C, part, s)
+                               : mv_dispatch<float, float>(P, tr, (const float*)val, diag, x, y, ns, C, part, s);
     };
     KC_TRY(step(true, in, mid));
     return step(false, mid, out);
@@ -292,8 +304,8 @@ kc_status factor_matvec_impl(const kc_pattern* P, int prec, const void* val, con
     }
     KC_TRY(to_point_major(in, perm, P->N, nrhs, a, s, ns));
     auto step = [&](bool tr, const double* x, double* y) {
-        return prec == KC_FP64 ? mv_dispatch<double>(P, tr, (const double*)val, diag, x, y, ns, C, part, s)
-                               : mv_dispatch<float>(P, tr, (const float*)val, diag, x, y, ns, C, part, s);
+        return prec == KC_FP64 ? mv_dispatch<double, double>(P, tr, (const double*)val, diag, x, y, ns, C, part, s)
+                               : mv_dispatch<float, double>(P, tr, (const float*)val, diag, x, y, ns, C, part, s);
     };
     const double* res = b;
     if (which == 0) KC_TRY(step(false, a, b));
